@@ -1,4 +1,5 @@
-"""ctypes binding of libbtc_b200.so: argument marshalling only.
+"""Binding of libbtc_b200.so: argument marshalling only.  The entry points of a serving loop go through the extension
+module _native (csrc/native.cpp); the rest, and the raw C ABI as `lib`, through ctypes.
 
 Every step of the layer runs in the library's CUDA kernels; torch supplies device memory
 and the current stream.  There is no CPU or eager-PyTorch fallback: if the shared library
@@ -99,6 +100,7 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
+from . import _native  # noqa: E402  (linked against the library that _load has just built or found)
 
 
 def _stream() -> int:
@@ -153,61 +155,22 @@ def linear_workspace_bytes(M: int, N: int, K: int, v: int, Kc: int) -> int:
     return int(lib.btc_linear_workspace_bytes(M, N, K, v, Kc))
 
 
-def _linear(fn, name, x, idx, C_packed, alpha, v, Kc, mu, out, out_dtype, workspace, transform):
-    for t, n in ((x, "x"), (idx, "idx"), (C_packed, "C_packed"), (alpha, "alpha")):
-        _dev(t, n)
-    if x.dim() != 2 or idx.dim() != 2:
-        raise ValueError("x must be [M, K] and idx [N, K/v]")
-    if x.dtype not in (torch.float16, torch.bfloat16):
-        raise ValueError("x must be fp16 or bf16")
-    if idx.element_size() != 2 or alpha.dtype != torch.float16 or C_packed.element_size() != 4:
-        raise ValueError("idx must be 16-bit integers, alpha fp16, C_packed 32-bit words")
-    M, K = x.shape
-    N, Kb = idx.shape
-    if C_packed.numel() != packed_words(Kc, v):
-        raise ValueError("C_packed is not the buffer codebook_pack wrote for this (Kc, v)")
-    if Kb * v != K or alpha.numel() != N:
-        raise ValueError("shape mismatch between x, idx, v and alpha")
-    if mu is not None:
-        _dev(mu, "mu")
-        if mu.dtype != torch.float16 or mu.numel() != N:
-            raise ValueError("mu must be fp16 [N]")
-    if out is None:
-        out = torch.empty((M, N), dtype=out_dtype, device=x.device)
-    else:
-        _dev(out, "out")
-        if tuple(out.shape) != (M, N):
-            raise ValueError("out must be [M, N]")
-    tr = None
-    if transform is not None:
-        sig, P1, P2 = transform
-        tr = BtcTransform(sig.data_ptr(), P1.data_ptr(), P2.data_ptr(), P1.shape[0], P2.shape[0])
-    need = int(lib.btc_linear_workspace_bytes_ex(M, N, K, v, Kc, int(transform is not None)))
-    ws_ptr, ws_bytes = None, 0
-    if need:
-        if workspace is None:
-            workspace = torch.empty(need, dtype=torch.uint8, device=x.device)
-        ws_ptr, ws_bytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
-    st = fn(x.data_ptr(), _DT[x.dtype], idx.data_ptr(), C_packed.data_ptr(), alpha.data_ptr(), _ptr(mu),
-            ctypes.byref(tr) if tr is not None else None, out.data_ptr(), _DT[out.dtype],
-            M, N, K, v, Kc, ws_ptr, ws_bytes, _stream())
-    if st:
-        raise BtcError(st, name)
-    return out
-
-
 def linear_gemv(x, idx, C_packed, alpha, v, Kc, mu=None, out=None, out_dtype=torch.float32, workspace=None,
                 transform=None):
     """Decode path (M <= 8): y[M, N] = x * W^T with W^ = alpha * C[idx] (+ mu)."""
-    return _linear(lib.btc_linear_gemv, "btc_linear_gemv", x, idx, C_packed, alpha, v, Kc, mu, out, out_dtype,
-                   workspace, transform)
+    y = _native.linear(0, x, idx, C_packed, alpha, v, Kc, mu, out, out_dtype, workspace, transform)
+    if y.__class__ is int:
+        raise BtcError(y, "btc_linear_gemv")
+    return y
 
 
 def linear_gemm(x, idx, C_packed, alpha, v, Kc, mu=None, out=None, out_dtype=torch.float32, workspace=None,
                 transform=None):
     """Tensor-core path (any M, built for large M)."""
-    return _linear(lib.btc_linear_gemm, "btc_linear_gemm", x, idx, C_packed, alpha, v, Kc, mu, out, out_dtype,
-                   workspace, transform)
+    y = _native.linear(1, x, idx, C_packed, alpha, v, Kc, mu, out, out_dtype, workspace, transform)
+    if y.__class__ is int:
+        raise BtcError(y, "btc_linear_gemm")
+    return y
 
 
 class GemvBatch:
@@ -244,11 +207,11 @@ class GemvBatch:
             arr[i] = BtcLinearProblem(x.data_ptr(), idx.data_ptr(), Cp.data_ptr(), alpha.data_ptr(), _ptr(mu),
                                       out.data_ptr(), _DT[x.dtype], _DT[out.dtype], M, N, K, v, Kc, bits, 0, 0)
             self.layers.append((x, idx, Cp, alpha, mu, out))          # keeps the tensors alive
-        self._arr = arr
+        self._arr, self._addr = arr, ctypes.addressof(arr)
         self.outs = [t[5] for t in self.layers]
 
     def run(self):
-        st = lib.btc_linear_gemv_batch(self._arr, len(self.layers), _stream())
+        st = _native.gemv_batch(self._addr, len(self.layers))
         if st:
             raise BtcError(st, "btc_linear_gemv_batch")
         return self.outs
@@ -257,18 +220,10 @@ class GemvBatch:
 def activation_transform(x, transform, out_dtype=torch.float32, out=None):
     """x' = x * diag(sigma) * (P1 kron P2) for the rows of x (fp16 / bf16 [M, K]); transform = (sigma_bits int32
     [ceil(K/32)], P1 fp32 [k1, k1], P2 fp32 [k2, k2]).  out_dtype: torch.float32 or the dtype of x."""
-    _dev(x, "x")
-    sig, P1, P2 = transform
-    for t, n in ((sig, "sigma_bits"), (P1, "P1"), (P2, "P2")):
-        _dev(t, n)
-    M, K = x.shape
-    if out is None:
-        out = torch.empty((M, K), dtype=out_dtype, device=x.device)
-    T = BtcTransform(sig.data_ptr(), P1.data_ptr(), P2.data_ptr(), P1.shape[0], P2.shape[0])
-    st = lib.btc_activation_transform(x.data_ptr(), _DT[x.dtype], ctypes.byref(T), out.data_ptr(), _DT[out.dtype], M, K, _stream())
-    if st:
-        raise BtcError(st, "btc_activation_transform")
-    return out
+    y = _native.activation_transform(x, transform, out_dtype, out)
+    if y.__class__ is int:
+        raise BtcError(y, "btc_activation_transform")
+    return y
 
 
 def linear_gemv_batch(layers):
@@ -393,9 +348,12 @@ def linear_gemv_packed(x, idx_packed, C_packed, alpha, v, Kc, mu=None, out=None,
     return out
 
 
-def linear(x, idx, C_packed, alpha, v, Kc, **kw):
+def linear(x, idx, C_packed, alpha, v, Kc, mu=None, out=None, out_dtype=torch.float32, workspace=None, transform=None):
     """Routes by M the way a caller would: decode path up to 8 rows, tensor-core path above."""
-    return (linear_gemv if x.shape[0] <= 8 else linear_gemm)(x, idx, C_packed, alpha, v, Kc, **kw)
+    y = _native.linear(2, x, idx, C_packed, alpha, v, Kc, mu, out, out_dtype, workspace, transform)
+    if y.__class__ is int:
+        raise BtcError(y, "btc_linear")
+    return y
 
 
 def codebook_kmeans(vecs: torch.Tensor, v: int, Kc: int, max_iter: int = 20, workspace: Optional[torch.Tensor] = None):

@@ -1,4 +1,5 @@
-"""Builds libbtc_b200.so (sm_100a only) from csrc/ with nvcc, in-tree next to this file."""
+"""Builds libbtc_b200.so (sm_100a only) from csrc/*.cu with nvcc and the Python call path _native (csrc/native.cpp) on top
+of it with g++, in-tree next to this file."""
 from __future__ import annotations
 
 import glob
@@ -6,12 +7,15 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "libbtc_b200.so")
+NATIVE = os.path.join(HERE, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
+NATIVE_SRC = os.path.join(CSRC, "native.cpp")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -30,12 +34,31 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _older(target, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(p) > os.path.getmtime(target) for p in deps)
+
+
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
-    return any(os.path.getmtime(p) > t for p in deps)
+    headers = glob.glob(os.path.join(INCLUDE, "*.h"))
+    return (_older(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + headers)
+            or _older(NATIVE, [NATIVE_SRC] + headers))
+
+
+def build_native() -> None:
+    """The extension module: torch's C++ headers, linked against the library (found beside it at run time)."""
+    import torch
+    from torch.utils import cpp_extension
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", INCLUDE, "-I", sysconfig.get_paths()["include"]]
+    for d in cpp_extension.include_paths() + ["/usr/local/cuda/include"]:
+        cmd += ["-isystem", d]
+    for d in cpp_extension.library_paths() + [HERE]:
+        cmd += ["-L", d]
+    cmd += [NATIVE_SRC, "-o", tmp, "-l:" + os.path.basename(LIB), "-ltorch_python", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda",
+            "-Wl,-rpath,$ORIGIN"]
+    subprocess.check_call(cmd)
+    os.replace(tmp, NATIVE)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
@@ -64,6 +87,7 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.check_call([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp, *objs])
     os.replace(tmp, LIB)
+    build_native()
     return LIB
 
 

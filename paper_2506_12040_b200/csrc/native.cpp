@@ -1,0 +1,210 @@
+// Call path of the hot entry points: Python objects in, C ABI calls out.
+//
+// A decode-path layer runs for about 4 us on the GPU, so a program that calls layers one by one is paced by the host.
+// Marshalling a call through ctypes (attribute look-ups on the tensors, boxed pointers, torch.empty, the stream object)
+// took about 13 of the 16.4 us of a 4096 x 4096 call at M = 1; the same checks on the C++ tensors take about one.
+// Every function takes its arguments positionally (the Python functions around them carry names and defaults) and
+// returns its result, or the btc_status as an int when the library refused the call; bad arguments raise ValueError.
+#include <Python.h>
+
+#include <ATen/core/Tensor.h>
+#include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDAGuard.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Dtype.h>
+#include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "btc.h"
+
+namespace {
+
+struct Refused {};                       // a Python error has been set
+
+[[noreturn]] void refuse(const char *msg)
+{
+    PyErr_SetString(PyExc_ValueError, msg);
+    throw Refused();
+}
+
+const at::Tensor &tensor(PyObject *o, const char *name)
+{
+    if (!THPVariable_Check(o)) {
+        PyErr_Format(PyExc_TypeError, "%s must be a tensor", name);
+        throw Refused();
+    }
+    return THPVariable_Unpack(o);
+}
+
+const at::Tensor &device_tensor(PyObject *o, const char *name)
+{
+    const at::Tensor &t = tensor(o, name);
+    if (!t.is_cuda() || !t.is_contiguous()) {
+        PyErr_Format(PyExc_ValueError, t.is_cuda() ? "%s must be contiguous" : "%s must be a CUDA tensor", name);
+        throw Refused();
+    }
+    return t;
+}
+
+int dtype_code(at::ScalarType t)
+{
+    if (t == at::kHalf) return BTC_F16;
+    if (t == at::kBFloat16) return BTC_BF16;
+    if (t == at::kFloat) return BTC_F32;
+    PyErr_SetString(PyExc_KeyError, c10::toString(t));
+    throw Refused();
+}
+
+int integer(PyObject *o)
+{
+    const long v = PyLong_AsLong(o);
+    if (v == -1 && PyErr_Occurred()) throw Refused();
+    if (v != (int)v) refuse("integer argument out of range");
+    return (int)v;
+}
+
+at::ScalarType scalar_type(PyObject *o)
+{
+    if (!THPDtype_Check(o)) refuse("out_dtype must be a torch.dtype");
+    return reinterpret_cast<THPDtype *>(o)->scalar_type;
+}
+
+at::Tensor empty(at::IntArrayRef shape, at::ScalarType t, const at::Tensor &like)
+{
+    return at::detail::empty_cuda(shape, t, like.device(), std::nullopt);
+}
+
+void *stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
+
+// (sigma_bits, P1, P2) or None
+bool transform(PyObject *o, btc_transform *T)
+{
+    if (o == Py_None) return false;
+    PyObject *seq = PySequence_Fast(o, "transform must be (sigma_bits, P1, P2)");
+    if (!seq) throw Refused();
+    const bool three = PySequence_Fast_GET_SIZE(seq) == 3;
+    PyObject **it = PySequence_Fast_ITEMS(seq);
+    bool tensors = three;
+    for (int i = 0; tensors && i < 3; ++i) tensors = THPVariable_Check(it[i]);
+    if (tensors) {
+        const at::Tensor &s = THPVariable_Unpack(it[0]), &p1 = THPVariable_Unpack(it[1]), &p2 = THPVariable_Unpack(it[2]);
+        for (const at::Tensor *t : {&s, &p1, &p2}) tensors = tensors && t->is_cuda() && t->is_contiguous();
+        tensors = tensors && p1.dim() == 2 && p2.dim() == 2;
+        if (tensors) {
+            T->sigma_bits = static_cast<const uint32_t *>(s.data_ptr());
+            T->P1 = static_cast<const float *>(p1.data_ptr());
+            T->P2 = static_cast<const float *>(p2.data_ptr());
+            T->k1 = (int)p1.size(0);
+            T->k2 = (int)p2.size(0);
+        }
+    }
+    Py_DECREF(seq);                      // (the caller's argument keeps the tensors alive)
+    if (!tensors) refuse("transform must be three contiguous CUDA tensors (sigma_bits, P1 [k1, k1], P2 [k2, k2])");
+    return true;
+}
+
+// linear(path, x, idx, C_packed, alpha, v, Kc, mu, out, out_dtype, workspace, transform)
+// path: 0 btc_linear_gemv, 1 btc_linear_gemm, 2 the former up to 8 rows of x and the latter above
+PyObject *linear_impl(PyObject *const *a)
+{
+    int path = integer(a[0]);
+    const at::Tensor &x = device_tensor(a[1], "x"), &idx = device_tensor(a[2], "idx");
+    const at::Tensor &Cp = device_tensor(a[3], "C_packed"), &alpha = device_tensor(a[4], "alpha");
+    const int v = integer(a[5]), Kc = integer(a[6]);
+    if (x.dim() != 2 || idx.dim() != 2) refuse("x must be [M, K] and idx [N, K/v]");
+    const at::ScalarType xt = x.scalar_type();
+    if (xt != at::kHalf && xt != at::kBFloat16) refuse("x must be fp16 or bf16");
+    if (idx.element_size() != 2 || alpha.scalar_type() != at::kHalf || Cp.element_size() != 4)
+        refuse("idx must be 16-bit integers, alpha fp16, C_packed 32-bit words");
+    const int64_t M = x.size(0), K = x.size(1), N = idx.size(0), Kb = idx.size(1);
+    if (M > INT32_MAX || K > INT32_MAX || N > INT32_MAX) refuse("a dimension is out of range");
+    const size_t packed = btc_codebook_packed_bytes(Kc, v);
+    if (packed == 0) refuse("invalid codebook shape");
+    if ((size_t)Cp.numel() * 4 != packed) refuse("C_packed is not the buffer codebook_pack wrote for this (Kc, v)");
+    if (Kb * v != K || alpha.numel() != N) refuse("shape mismatch between x, idx, v and alpha");
+    const void *mu = nullptr;
+    if (a[7] != Py_None) {
+        const at::Tensor &t = device_tensor(a[7], "mu");
+        if (t.scalar_type() != at::kHalf || t.numel() != N) refuse("mu must be fp16 [N]");
+        mu = t.data_ptr();
+    }
+    at::Tensor out;
+    if (a[8] == Py_None) {
+        out = empty({M, N}, scalar_type(a[9]), x);
+    } else {
+        out = device_tensor(a[8], "out");
+        if (out.dim() != 2 || out.size(0) != M || out.size(1) != N) refuse("out must be [M, N]");
+    }
+    btc_transform T;
+    const bool has_t = transform(a[11], &T);
+    const size_t need = btc_linear_workspace_bytes_ex((int)M, (int)N, (int)K, v, Kc, has_t);
+    at::Tensor ws;
+    void *ws_ptr = nullptr;
+    size_t ws_bytes = 0;
+    if (need) {
+        if (a[10] == Py_None) ws = empty({(int64_t)need}, at::kByte, x);
+        else ws = tensor(a[10], "workspace");
+        ws_ptr = ws.data_ptr();
+        ws_bytes = (size_t)ws.numel() * ws.element_size();
+    }
+    if (path == 2) path = M <= 8 ? 0 : 1;
+    const int st = (path == 0 ? btc_linear_gemv : btc_linear_gemm)(
+        x.data_ptr(), dtype_code(xt), static_cast<const uint16_t *>(idx.data_ptr()), static_cast<const uint32_t *>(Cp.data_ptr()),
+        alpha.data_ptr(), mu, has_t ? &T : nullptr, out.data_ptr(), dtype_code(out.scalar_type()), (int)M, (int)N, (int)K, v, Kc,
+        ws_ptr, ws_bytes, stream());
+    if (st) return PyLong_FromLong(st);
+    if (a[8] != Py_None) return Py_NewRef(a[8]);
+    return THPVariable_Wrap(std::move(out));
+}
+
+// gemv_batch(address of the btc_linear_problem array, count)
+PyObject *gemv_batch_impl(PyObject *const *a)
+{
+    const auto *p = static_cast<const btc_linear_problem *>(PyLong_AsVoidPtr(a[0]));
+    if (!p && PyErr_Occurred()) throw Refused();
+    return PyLong_FromLong(btc_linear_gemv_batch(p, integer(a[1]), stream()));
+}
+
+// activation_transform(x, transform, out_dtype, out)
+PyObject *activation_transform_impl(PyObject *const *a)
+{
+    const at::Tensor &x = device_tensor(a[0], "x");
+    btc_transform T;
+    if (x.dim() != 2 || !transform(a[1], &T)) refuse("x must be [M, K], transform (sigma_bits, P1, P2)");
+    at::Tensor out;
+    if (a[3] == Py_None) out = empty(x.sizes(), scalar_type(a[2]), x);
+    else out = tensor(a[3], "out");
+    const int st = btc_activation_transform(x.data_ptr(), dtype_code(x.scalar_type()), &T, out.data_ptr(), dtype_code(out.scalar_type()),
+                                            (int)x.size(0), (int)x.size(1), stream());
+    if (st) return PyLong_FromLong(st);
+    if (a[3] != Py_None) return Py_NewRef(a[3]);
+    return THPVariable_Wrap(std::move(out));
+}
+
+template <PyObject *(*F)(PyObject *const *), int NARGS>
+PyObject *entry(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    if (n != NARGS) {
+        PyErr_Format(PyExc_TypeError, "expected %d arguments, got %zd", NARGS, n);
+        return nullptr;
+    }
+    HANDLE_TH_ERRORS                     // (an allocation that failed, among others)
+    try {
+        return F(args);
+    } catch (const Refused &) {
+        return nullptr;
+    }
+    END_HANDLE_TH_ERRORS
+}
+
+PyMethodDef methods[] = {
+    {"linear", (PyCFunction)(void (*)(void))entry<linear_impl, 12>, METH_FASTCALL, nullptr},
+    {"gemv_batch", (PyCFunction)(void (*)(void))entry<gemv_batch_impl, 2>, METH_FASTCALL, nullptr},
+    {"activation_transform", (PyCFunction)(void (*)(void))entry<activation_transform_impl, 4>, METH_FASTCALL, nullptr},
+    {nullptr, nullptr, 0, nullptr},
+};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&module); }
