@@ -84,17 +84,8 @@ static int run_linear(Path path, const void *x, int x_dt, const uint16_t *idx, c
 
     rc = BTC_ERR_UNSUPPORTED;
     if (path == PATH_GEMV || M <= 8) {
-        // the decode kernel (integer form up to two rows of x, fp16 form above; the older fp16 kernel where the table
-        // does not fit shared memory); for M = 5..8 with few row tiles and a
-        // very long K the tensor-core launch with K split over the SMs, when the workspace has room for its partial
-        // sums; the older fp16 kernel and the any-shape kernel take what the first does not cover
-        if (M > 2 && a.x_dt != BTC_F32 && gemm_tcgen05_small_m_pays(M, N, K, v)) rc = launch_gemm_tcgen05(a, s, true);
-        // M = 3..8, one layer per call: the older fp16 kernel (a CTA per row tile over the whole K) is the faster one --
-        // 8.5 against 10.1 us for 4096 x 4096 at M = 3, 15.8 against 24.6 us for 4096 x 11008, 13.8 against 19.6 us for
-        // 5120 x 5120 with 65536 centroids at M = 4; the newer fp16 form earns its keep in the fused multi-layer launch
-        if (rc == BTC_ERR_UNSUPPORTED && M > 2 && a.x_dt != BTC_F32) rc = launch_gemv_decode(a, s);
-        if (rc == BTC_ERR_UNSUPPORTED && M <= 2) rc = launch_gemv_imma_wide(&a, 1, s);     // (plain launches at M <= 2: the faster geometry)
-        if (rc == BTC_ERR_UNSUPPORTED) rc = launch_gemv_imma(&a, 1, s);
+        // the decode kernel; the older fp16 kernel and the any-shape kernel take what it does not cover
+        rc = launch_gemv(&a, 1, s);
         if (rc == BTC_ERR_UNSUPPORTED) rc = launch_gemv_decode(a, s);
     }
     else rc = launch_gemm_tcgen05(a, s);
@@ -233,19 +224,11 @@ static int btc::run_batch(const btc_linear_problem *problems, int count, void *s
             a.x_dt = p.x_dtype; a.y_dt = p.y_dtype;
             a.M = p.M; a.N = p.N; a.K = p.K; a.v = p.v; a.Kc = p.Kc; a.Kb = p.K / p.v;
         }
-        // plain launches at M <= 2 take the one-CTA-per-SM geometry (it declines anything else); a sum of terms never does,
-        // so that all its terms share one arithmetic
-        int rc = accumulate_from > 0 ? BTC_ERR_UNSUPPORTED : launch_gemv_imma_wide(group, n, s);
-        // a run of one plain layer at M = 3..8: the older fp16 kernel, as in btc_linear_gemv
-        if (rc == BTC_ERR_UNSUPPORTED && n == 1 && accumulate_from == 0 && group[0].M > 2 && group[0].x_dt != BTC_F32 &&
-            !group[0].idx_bits && !group[0].x_stride && !group[0].idx_stride)
-            rc = launch_gemv_decode(group[0], s);
-        if (rc == BTC_ERR_UNSUPPORTED) rc = launch_gemv_imma(group, n, s);
+        int rc = launch_gemv(group, n, s);
         if (rc == BTC_ERR_UNSUPPORTED) {
             // some layer of the run is outside the fused kernel: one launch per layer instead
             for (int k = 0; k < n; ++k) {
-                rc = accumulate_from > 0 ? BTC_ERR_UNSUPPORTED : launch_gemv_imma_wide(&group[k], 1, s);
-                if (rc == BTC_ERR_UNSUPPORTED) rc = launch_gemv_imma(&group[k], 1, s);
+                rc = launch_gemv(&group[k], 1, s);
                 // only the decode kernel reads dense indices, fp32 activations, column ranges of wider matrices, or adds to y
                 if (rc == BTC_ERR_UNSUPPORTED && (group[k].idx_bits || group[k].x_stride || group[k].idx_stride || group[k].accumulate ||
                                                   group[k].x_dt == BTC_F32)) return rc;

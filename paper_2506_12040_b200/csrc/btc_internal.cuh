@@ -40,8 +40,8 @@ inline int cuda_check_launch() {
 // gemv_generic.cu: any v / Kc / M (M is tiled by 8 over grid.y), plain CUDA cores.
 int launch_linear_generic(const LinearArgs &a, cudaStream_t s);
 
-// gemv_decode.cu: the tuned decode path (M <= 8).  Returns BTC_ERR_UNSUPPORTED when the shape
-// is outside what it covers, in which case the caller falls back to the generic kernel.
+// gemv_decode.cu: decode path for rows of indices that are not a whole number of 16-byte pieces (M <= 8, v a multiple of 4).
+// Returns BTC_ERR_UNSUPPORTED when the shape is outside what it covers, in which case the caller falls back to the generic kernel.
 int launch_gemv_decode(const LinearArgs &a, cudaStream_t s);
 size_t gemv_decode_workspace_bytes(int M, int N, int K, int v, int Kc);
 
@@ -51,13 +51,13 @@ bool gemm_tcgen05_small_m_pays(int M, int N, int K, int v);
 size_t gemm_tcgen05_workspace_bytes(int M, int N, int K, int v, int Kc);   // with room for a K split where one pays
 size_t gemm_tcgen05_workspace_min(int M);                                 // what the kernels cannot do without
 
-// gemv_imma.cu: integer-MMA decode path; runs up to IM_MAXP independent layers (M <= 8 each) in one launch.
-// Returns BTC_ERR_UNSUPPORTED when a shape is outside what it covers (nothing is launched then).
+// gemv.cu: the decode path; runs up to IM_MAXP independent layers (M <= 8 each), one launch for those that share a kernel.
+// Returns BTC_ERR_UNSUPPORTED when some layer is outside what it covers (nothing is launched then).
 constexpr int IM_MAXP = 8;
-int launch_gemv_imma(const LinearArgs *problems, int count, cudaStream_t s);
-int imma_status_read(int *out);
-int imma_status_reset();
-int imma_selftest_wait(cudaStream_t s);
+int launch_gemv(const LinearArgs *problems, int count, cudaStream_t s);
+int gemv_status_read(int *out);
+int gemv_status_reset();
+int gemv_selftest_wait(cudaStream_t s);
 
 // pack.cu: debug check of the index range (BTC_DEBUG_CHECK_INDICES=1) and its status word.
 bool debug_check_indices_enabled();
@@ -68,11 +68,6 @@ int index_status_reset();
 // gemv_lut.cu: the paper's two-stage lookup scheme (alternative route, own entry point).
 int launch_gemv_lut(const LinearArgs &a, cudaStream_t s);
 size_t gemv_lut_workspace_bytes(int M, int N, int K, int v);
-
-// gemv_imma_wide.cu: the integer form for M <= 2 in its one-CTA-per-SM geometry (plain launches only; UNSUPPORTED otherwise).
-int launch_gemv_imma_wide(const LinearArgs *problems, int count, cudaStream_t s);
-int wide_status_read(int *out);
-int wide_status_reset();
 
 // transform.cu: x' = x * D * (P1 (x) P2) into xt (same shape as x, dtype out_dt).
 int launch_transform(const void *x, int x_dt, const btc_transform &T, void *xt, int out_dt, int M, int K,

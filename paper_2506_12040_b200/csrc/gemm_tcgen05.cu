@@ -808,14 +808,12 @@ extern "C" BTC_API int btc_device_status_reset(void)
     if (e != cudaSuccess) return btc::cuda_fail(e);
     int rc = btc::index_status_reset();
     if (rc != BTC_OK) return rc;
-    rc = btc::wide_status_reset();
-    if (rc != BTC_OK) return rc;
-    return btc::imma_status_reset();
+    return btc::gemv_status_reset();
 }
 
 extern "C" BTC_API int btc_selftest_bounded_wait(void *stream)
 {
-    return btc::imma_selftest_wait((cudaStream_t)stream);
+    return btc::gemv_selftest_wait((cudaStream_t)stream);
 }
 
 extern "C" BTC_API int btc_device_status(int *status_host)
@@ -825,15 +823,12 @@ extern "C" BTC_API int btc_device_status(int *status_host)
     cudaError_t e = cudaMemcpyFromSymbol(&v, btc::g_gemm_status, sizeof(int));
     if (e != cudaSuccess) return btc::cuda_fail(e);
     int v2 = 0;
-    const int rc = btc::imma_status_read(&v2);
+    const int rc = btc::gemv_status_read(&v2);
     if (rc != BTC_OK) return rc;
     int v3 = 0;
     const int rc3 = btc::index_status_read(&v3);
     if (rc3 != BTC_OK) return rc3;
-    int v4 = 0;
-    const int rc4 = btc::wide_status_read(&v4);
-    if (rc4 != BTC_OK) return rc4;
-    *status_host = v ? v : (v2 ? v2 : (v4 ? v4 : v3));
+    *status_host = v ? v : (v2 ? v2 : v3);
     return BTC_OK;
 }
 

@@ -1,0 +1,327 @@
+// Decode path, host side: grouping of layers into launches, shared-memory plan, split of the row tiles over the CTAs.
+#include <memory>
+#include <new>
+#include "gemv.cuh"
+
+namespace btc {
+namespace gv {
+
+__device__ int g_status = 0;
+
+static int *status_word()
+{
+    // (device address of the status word, per device)
+    static std::atomic<int *> addr[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    int *p = addr[dev].load(std::memory_order_acquire);
+    if (!p) {
+        void *q = nullptr;
+        if (cudaGetSymbolAddress(&q, g_status) != cudaSuccess) return nullptr;
+        p = static_cast<int *>(q);
+        addr[dev].store(p, std::memory_order_release);
+    }
+    return p;
+}
+
+static int sm_count()
+{
+    static int n = 0;
+    if (n == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
+    }
+    return n;
+}
+
+struct Shape { bool half; int ncls, slices_log2, parts; };
+
+// Eight slices per K-pass, four where those cover K (then a CTA's warps work on twice the rows): a function of the layer
+// alone.
+static Shape shape_of(const LinearArgs &a)
+{
+    Shape s;
+    s.ncls = (a.v + 3) / 4;
+    s.half = a.M > 2 || a.v % 4 != 0 || a.v == 4 || a.v > 20;
+    const int slice = 4 * lane_blocks(s.half, s.ncls);
+    s.slices_log2 = a.Kb <= 4 * slice ? 2 : 3;
+    s.parts = (a.Kb + (slice << s.slices_log2) - 1) / (slice << s.slices_log2);
+    return s;
+}
+
+// v even up to 24 (a block's bits fit the fp16 form), rows of idx a whole number of 16-byte pieces, x rows 16-byte aligned
+// where 8 activations are read at once; dense index widths 12 and 13 (the v = 16 codebooks of 4096 / 8192), v up to 16.
+static bool covered(const LinearArgs &a)
+{
+    if (a.M < 1 || a.M > 8 || a.v % 2 != 0 || a.v > 24 || a.Kb % 8 != 0 || a.K > (1 << 20)) return false;
+    if (a.accumulate && a.y_dt != BTC_F32) return false;
+    if (a.x_stride % 8 || a.idx_stride % 8 || (a.idx_bits && a.idx_stride)) return false;
+    if (a.idx_bits && ((a.idx_bits != 12 && a.idx_bits != 13) || a.v > 16)) return false;
+    return true;
+}
+
+static int round_up(int x, int m) { return (x + m - 1) / m * m; }
+
+static Layout layout(bool half, int ncls, int rows, int ib, int nw, int tab_bytes, int stages)
+{
+    Layout L;
+    L.stages = stages;
+    L.stage_bytes = nw * 16 * (4 * lane_blocks(half, ncls)) * (ib ? ib : 16) / 8;    // (slices x rows per stage is 16 nw, however many slices)
+    int o = round_up(stages * L.stage_bytes + (ib ? 16 : 0), 128);   // (a lane's last word of dense fields may lie just past its row)
+    L.tab = o; o += round_up(tab_bytes, 16);
+    L.park = o; o += half ? park_bytes<true>() : park_bytes<false>();
+    L.stage_x_pitch = stage_x_bytes(half, ncls, rows);
+    L.stage_x = o; o += (half ? MAX_SLICES : nw) * L.stage_x_pitch;
+    L.misc = round_up(o, 16);
+    L.total = L.misc + MISC_BYTES;
+    return L;
+}
+
+typedef CUresult (*encode_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
+                              const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+static encode_fn get_encode()
+{
+    static encode_fn fn = nullptr;
+    if (!fn) {
+        void *ptr = nullptr;
+        cudaDriverEntryPointQueryResult qr;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qr) == cudaSuccess && qr == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<encode_fn>(ptr);
+    }
+    return fn;
+}
+
+// Tensor map of an index matrix.  Encoding goes through the driver and costs about a microsecond, a quarter of a launch; a
+// decoder re-uses the same matrices token after token (a 32-block model has 224), so maps are kept per host thread in a
+// table of 1024 slots (two per hash), keyed by everything the encoding depends on.
+struct MapKey {
+    const void *idx;
+    int Kb, N, rows, ib;
+    long long pitch;
+    bool operator==(const MapKey &o) const { return idx == o.idx && Kb == o.Kb && N == o.N && rows == o.rows && ib == o.ib && pitch == o.pitch; }
+};
+
+static bool tensor_map(const MapKey &k, int box_words, CUtensorMap *out)
+{
+    struct Slot { MapKey key; CUtensorMap map; };
+    constexpr int SETS = 512;
+    thread_local std::unique_ptr<Slot[]> slots;
+    if (!slots) {
+        slots.reset(new (std::nothrow) Slot[2 * SETS]());
+        if (!slots) return false;
+    }
+    uint64_t h = reinterpret_cast<uintptr_t>(k.idx) / 256 * 0x9E3779B97F4A7C15ull;
+    h ^= (uint64_t)(k.rows + 64 * k.ib + 4096 * (box_words / 4)) * 0xBF58476D1CE4E5B9ull;
+    Slot *set = slots.get() + 2 * ((h >> 40) % SETS);
+    for (int i = 0; i < 2; ++i)
+        if (set[i].key == k) { *out = set[i].map; return true; }
+    encode_fn enc = get_encode();
+    if (!enc) return false;
+    const cuuint32_t estr[2] = {1, 1};
+    const cuuint64_t strides[1] = {(cuuint64_t)k.pitch};
+    CUtensorMap m;
+    CUresult r;
+    if (k.ib == 0) {
+        const cuuint64_t dims[2] = {(cuuint64_t)k.Kb, (cuuint64_t)k.N};
+        const cuuint32_t box[2] = {64u, (cuuint32_t)k.rows};
+        r = enc(&m, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, const_cast<void *>(k.idx), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    } else {
+        // dense fields: rows of `pitch` bytes seen as 32-bit words; one box = a pass of `rows` rows, no swizzle
+        const cuuint64_t dims[2] = {(cuuint64_t)(k.pitch / 4), (cuuint64_t)k.N};
+        const cuuint32_t box[2] = {(cuuint32_t)box_words, (cuuint32_t)k.rows};
+        r = enc(&m, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<void *>(k.idx), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    }
+    if (r != CUDA_SUCCESS) return false;
+    set[1] = set[0];                                     // (the older of the two goes)
+    set[0].key = k;
+    set[0].map = m;
+    *out = m;
+    return true;
+}
+
+// Gives every layer a whole number of CTAs so that the largest load of any CTA -- ceil(groups / CTAs) row groups times the
+// layer's cost, plus its set-up cost -- is as small as the budget allows (bisection), and returns the grid size.
+static int assign_ctas(Batch &b, int budget)
+{
+    auto per_cta = [&](int i, long long T) { return (T - b.p[i].fixed) / b.p[i].cost; };
+    auto needed = [&](long long T) {
+        long long sum = 0;
+        for (int i = 0; i < b.count; ++i) {
+            const long long per = per_cta(i, T);
+            if (per < 1) return (long long)1 << 40;
+            sum += (b.p[i].groups + per - 1) / per;
+        }
+        return sum;
+    };
+    long long lo = 1, hi = 0;
+    for (int i = 0; i < b.count; ++i) {
+        const long long all = (long long)b.p[i].groups * b.p[i].cost + b.p[i].fixed;
+        if (all > hi) hi = all;                          // one CTA per layer always fits (budget >= count)
+    }
+    while (lo < hi) {
+        const long long mid = (lo + hi) / 2;
+        if (needed(mid) <= budget) hi = mid; else lo = mid + 1;
+    }
+    int sum = 0;
+    for (int i = 0; i < b.count; ++i) {
+        const long long per = per_cta(i, lo);
+        b.p[i].cta_count = (int)((b.p[i].groups + per - 1) / per);
+        sum += b.p[i].cta_count;
+    }
+    while (sum < budget) {                               // spare CTAs go where the average load is highest
+        int best = -1;
+        double most = 0;
+        for (int i = 0; i < b.count; ++i) {
+            const double load = (double)b.p[i].groups * b.p[i].cost / b.p[i].cta_count + b.p[i].fixed;
+            if (b.p[i].cta_count < b.p[i].groups && (best < 0 || load > most)) { best = i; most = load; }
+        }
+        if (best < 0) break;
+        ++b.p[best].cta_count; ++sum;
+    }
+    int begin = 0;
+    for (int i = 0; i < b.count; ++i) {
+        b.p[i].cta_begin = begin;
+        begin += b.p[i].cta_count;
+        b.p[i].per = b.p[i].groups / b.p[i].cta_count;
+        b.p[i].rem = b.p[i].groups % b.p[i].cta_count;
+    }
+    return begin;
+}
+
+// One launch over layers of one form, class count and index format.
+static int launch_group(const LinearArgs *const *args, int count, cudaStream_t s)
+{
+    Batch b;
+    b.count = count;
+    b.status = status_word();
+    if (!b.status) return cuda_fail(cudaErrorUnknown);
+    const Shape s0 = shape_of(*args[0]);
+    const int ib = args[0]->idx_bits;
+    int words = 0, halves = 0, m_even = 2;
+    for (int i = 0; i < count; ++i) {
+        const LinearArgs &a = *args[i];
+        words = a.Kc > words ? a.Kc : words;
+        if (a.M > m_even) m_even = round_up(a.M, 2);
+    }
+    halves = round_up(words, 8) * 2;
+    words = round_up(words, 4) * 4;
+    // Table: 16-bit halves in the integer form up to v = 16 (half the shared memory and half the bytes that every CTA loads; 65536
+    // codewords take 128 KB), else 32-bit words; two CTAs per SM where that leaves room for them (integer form), else one; else as
+    // much of the words as fits (frequency-ordered codebooks: the head serves most lookups).
+    constexpr int half_sm = 113 * 1024, whole_sm = 227 * 1024;
+    auto fits = [&](int nw, int tab, int stages) { return layout(s0.half, s0.ncls, m_even, ib, nw, tab, stages).total <= (nw == 8 ? half_sm : whole_sm); };
+    int nw = s0.half ? 16 : 8, tab = !s0.half && s0.ncls <= 4 ? TAB_HALVES : TAB_WORDS, tab_bytes = tab == TAB_HALVES ? halves : words;
+    if (!fits(nw, tab_bytes, 3)) {
+        if (ib) return BTC_ERR_UNSUPPORTED;
+        nw = 16;
+        if (!fits(16, tab_bytes, 2)) {
+            tab = TAB_HEAD;
+            tab_bytes = (whole_sm - layout(s0.half, s0.ncls, m_even, ib, nw, 0, 3).total - 128) / 128 * 128;
+        }
+    }
+    b.tab_head = tab_bytes / 4;
+    int stages = 2;
+    while (stages < MAX_STAGES && fits(nw, tab_bytes, stages + 1)) ++stages;
+    b.L = layout(s0.half, s0.ncls, m_even, ib, nw, tab_bytes, stages);
+
+    long long work = 0, groups = 0;
+    for (int i = 0; i < count; ++i) {
+        const LinearArgs &a = *args[i];
+        const Shape sh = shape_of(a);
+        Problem &p = b.p[i];
+        const int Kc4 = round_up(a.Kc, 4);
+        p.x = a.x; p.alpha = a.alpha; p.mu = a.mu; p.y = a.y;
+        const int rows = 16 * (nw >> sh.slices_log2), pass = 4 * lane_blocks(sh.half, sh.ncls) << sh.slices_log2;
+        const MapKey key = {ib ? a.idx_packed : static_cast<const void *>(a.idx), a.Kb, a.N, rows, ib,
+                            ib ? (long long)a.idx_pitch : (long long)(a.idx_stride ? a.idx_stride : a.Kb) * 2};
+        if (!tensor_map(key, pass * ib / 32, &b.map[i])) return BTC_ERR_UNSUPPORTED;
+        p.tab = tab == TAB_HALVES ? static_cast<const void *>(a.Cp + 3 * (size_t)Kc4) : static_cast<const void *>(a.Cp + (sh.half ? 1 : 2) * (size_t)Kc4);
+        p.tab_bytes = tab == TAB_HALVES ? round_up(a.Kc, 8) * 2 : (Kc4 * 4 < tab_bytes ? Kc4 * 4 : tab_bytes);
+        p.M = a.M; p.N = a.N; p.v = a.v; p.Kb = a.Kb;
+        p.xs = a.x_stride ? a.x_stride : a.K;
+        p.acc = a.accumulate ? 1 : 0;
+        p.x_dt = a.x_dt; p.y_dt = a.y_dt;
+        p.slices_log2 = sh.slices_log2; p.parts = sh.parts;
+        p.groups = (a.N + rows - 1) / rows;
+        // in sixteenths of a (stage, pass); a pass's fragments cost about as much as one and a half of them
+        p.cost = p.parts * 16;
+        p.fixed = p.parts * 24 * (sh.half ? 1 : a.M);
+        groups += p.groups;
+        work += (long long)p.groups * p.parts;
+    }
+    const int sms = sm_count();
+    const int slots = nw == 8 && work > 3 * sms ? 2 * sms : sms;
+    const int grid = assign_ctas(b, groups < slots ? (int)groups : slots);
+    return (s0.half ? launch_half : launch_int)(b, s0.ncls, tab, ib, nw, args[0]->x_dt == BTC_F32, grid, s);
+}
+
+static bool same_kernel(const LinearArgs &a, const LinearArgs &b)
+{
+    const Shape s = shape_of(a), t = shape_of(b);
+    return s.half == t.half && s.ncls == t.ncls && a.idx_bits == b.idx_bits && (!s.half || (a.x_dt == BTC_F32) == (b.x_dt == BTC_F32));
+}
+
+// Self-test of the bounded wait: one warp waits (with a ~1 ms limit) on a barrier that nothing ever arrives on, which
+// must raise the status word and return -- the same code path a lost producer or consumer would take in the kernel.
+__global__ void selftest_wait_kernel(int *status)
+{
+    __shared__ uint64_t bar;
+    __shared__ int abort_flag;
+    if (threadIdx.x == 0) {
+        mbar_init(smem_addr(&bar), 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    (void)mbar_wait(smem_addr(&bar), 0, &abort_flag, status, 2000000LL);
+}
+
+}  // namespace gv
+
+int launch_gemv(const LinearArgs *problems, int count, cudaStream_t s)
+{
+    if (count < 1 || count > IM_MAXP) return BTC_ERR_UNSUPPORTED;
+    for (int i = 0; i < count; ++i)
+        if (!gv::covered(problems[i])) return BTC_ERR_UNSUPPORTED;
+    bool taken[IM_MAXP] = {};
+    for (int i = 0; i < count; ++i) {
+        if (taken[i]) continue;
+        const LinearArgs *group[IM_MAXP];
+        int n = 0;
+        for (int k = i; k < count; ++k)
+            if (!taken[k] && gv::same_kernel(problems[i], problems[k])) { taken[k] = true; group[n++] = &problems[k]; }
+        const int rc = gv::launch_group(group, n, s);
+        if (rc != BTC_OK) return rc;
+    }
+    return BTC_OK;
+}
+
+int gemv_selftest_wait(cudaStream_t s)
+{
+    int *status = gv::status_word();
+    if (!status) return cuda_fail(cudaErrorUnknown);
+    gv::selftest_wait_kernel<<<1, 32, 0, s>>>(status);
+    return cuda_check_launch();
+}
+
+int gemv_status_reset()
+{
+    const int zero = 0;
+    cudaError_t e = cudaMemcpyToSymbol(gv::g_status, &zero, sizeof(int));
+    return e == cudaSuccess ? BTC_OK : cuda_fail(e);
+}
+
+int gemv_status_read(int *out)
+{
+    int v = 0;
+    cudaError_t e = cudaMemcpyFromSymbol(&v, gv::g_status, sizeof(int));
+    if (e != cudaSuccess) return cuda_fail(e);
+    *out = v;
+    return BTC_OK;
+}
+
+}  // namespace btc

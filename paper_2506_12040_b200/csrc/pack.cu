@@ -5,12 +5,12 @@
 namespace btc {
 
 // Kernel-private word of one centroid for the decode path ("MMA layout"): the bit of weight t sits
-// at (t & 1) * 16 + P0 + (t >> 1) with P0 = 12 - v/2, so that `word & mask` with one bit kept per
-// 16-bit half is a pair of fp16 numbers {0, 2^(pos-24)}.  Defined for v % 4 == 0, v <= 24; 0 otherwise.
+// at (t & 1) * 16 + P0 + (t >> 1) with P0 = 12 - 2 * ceil(v/4), so that `word & mask` with one bit kept per
+// 16-bit half is a pair of fp16 numbers {0, 2^(pos-24)}.  Defined for v <= 24; 0 otherwise.
 __host__ __device__ inline uint32_t mma_layout_word(uint32_t pub, int v)
 {
-    if (v % 4 != 0 || v > 24) return 0u;
-    const int p0 = 12 - v / 2;
+    if (v > 24) return 0u;
+    const int p0 = 12 - 2 * ((v + 3) / 4);
     uint32_t w = 0;
     for (int t = 0; t < v; ++t)
         if ((pub >> t) & 1u) w |= 1u << ((t & 1) * 16 + p0 + (t >> 1));

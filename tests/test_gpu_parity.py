@@ -87,6 +87,37 @@ def test_gemv_parity_small(N, K, v, Kc, M, dist, mu):
     assert rel <= TOL_GEMV and fwd <= TOL_GEMV, (rel, fwd)
 
 
+# The decode kernel where it can go wrong: block lengths that are no multiple of 4 (the last class half empty), four or eight
+# slices per pass (K/v = 128 | 136 at v <= 16), several passes with an empty or partial last slice, one row and one row more
+# than a tile or a chunk of tiles, tables as words, halves and head, with one and two CTAs per SM.
+EDGES = [
+    # N, K, v, Kc, M, dtype, mu
+    (16, 8 * 10, 10, 256, 1, "f16", True),
+    (17, 136 * 14, 14, 2353, 8, "bf16", False),
+    (3000, 128 * 18, 18, 21619, 1, "bf16", True),
+    (129, 776 * 18, 18, 21619, 3, "f16", False),
+    (40, 64 * 22, 22, 900, 2, "f16", False),
+    (64, 264 * 24, 24, 5000, 5, "bf16", True),
+    (48, 16 * 2, 2, 4, 1, "f16", False),
+    (4800, 128 * 16, 16, 9000, 2, "f16", True),
+    (9500, 136 * 16, 16, 65536, 1, "bf16", False),
+    (9480, 520 * 8, 8, 85, 7, "f16", True),
+    (2400, 264 * 20, 20, 40000, 1, "f16", False),
+    (2385, 264 * 20, 20, 40000, 4, "bf16", True),
+    (1, 8 * 16, 16, 65536, 6, "f16", False),
+]
+
+
+@pytest.mark.parametrize("N,K,v,Kc,M,dt,mu", EDGES)
+def test_gemv_edges(N, K, v, Kc, M, dt, mu):
+    L = wl.make_layer(_spec(N, K, v, Kc, x_dtype=dt, with_mu=mu, outlier_frac=0.01), M, seed=N + K + M)
+    y, d = run_layer(L, "gemv")
+    rel, fwd = errors(y, oracle_y(L), L)
+    assert rel <= TOL_GEMV and fwd <= TOL_GEMV, (rel, fwd)
+    again = btc.linear_gemv(d["x"], d["idx"], d["Cp"], d["alpha"], v, Kc, mu=d["mu"])
+    assert torch.equal(y, again) and btc.device_status() == 0
+
+
 @pytest.mark.parametrize("config", [1, 2, 3])
 def test_gemv_parity_benchmark_configs(config):
     """Full-size layers of the benchmark configs, every output compared (the oracle needs seconds)."""
