@@ -1,304 +1,407 @@
 // Binary codebook construction (paper Section 4.1 "Flash and Accurate Binary Codebook"; loop of the appendix
 // Algorithm "Binary Codebook Optimization"): initial centroids = the most frequent distinct vectors, then
-//   E-step  z_i = argmin_k d_H(b_i, c_k) = POPCNT(b_i xor c_k)      (||b - c||^2 = 4 d_H; smallest k among equals)
+//   E-step  z_i = argmin_k d_H(b_i, c_k)      (||b - c||^2 = 4 d_H; smallest k among equals)
 //   M-step  c_k = element-wise majority of the vectors assigned to k  (ties -> +1; an empty cluster keeps its centroid)
 // until no assignment changes or max_iter E-steps have run.
 //
-// Everything is done in the space of the 2^v possible patterns (v <= 20: the paper's range; 65536 of them at v = 16),
-// not per vector:
-// identical vectors have identical nearest centroids, so one histogram pass over the n vectors (the only pass that
-// streams them, besides the final look-up of z) reduces every later step to at most 2^v weighted patterns:
-//   histogram       cnt[p]                                     n atomic adds
-//   initial order   rank(p) = #{q : (cnt[q], -q) > (cnt[p], -p)}  (frequency descending, packed word ascending);
-//                   pattern p becomes centroid rank(p) when rank(p) < c; counted among the patterns at least as
-//                   frequent as the c-th most frequent one (threshold by bisection, then a candidate list)
-//   E-step          one thread per occurring pattern, centroids broadcast from shared memory;
-//                   min over k of (POPCNT << 16 | k) is the nearest centroid with the smallest index among equals
-//   M-step          per occurring pattern: add cnt[p] to the vote counters of its cluster; then one thread per centroid
-// No step synchronises with the host: the iteration loop is unrolled into max_iter rounds of launches, and every
-// kernel of a round returns at once when an earlier round has already found the assignments unchanged.
+// Everything is done in the space of the 2^v possible patterns (v <= 20: the paper's range; 65536 of them at v = 16), not
+// per vector: identical vectors have identical nearest centroids, so one histogram pass over the n vectors (the only pass
+// that streams them, besides the final look-up of z) reduces every later step to at most 2^v weighted patterns.
+//
+// One cooperative launch, a CTA per SM, the steps separated by a barrier over the grid:
+//   histogram  each CTA counts its vectors in shared memory as 16-bit counters (v <= 16: 128 KB; a hot pattern is a few
+//              per cent of all vectors, and that many atomics on one address of L2 serialise), then adds the non-zero ones
+//   ranking    rank(p) = #{q : (cnt[q], -q) > (cnt[p], -p)}, centroid rank(p) = p when rank(p) < c: a counting sort by frequency
+//              (a histogram of the frequencies per CTA and in total; word order among equals from the CTAs before and the
+//              patterns before; frequencies past the last bin are ranked pairwise)
+//   E-step     the Hamming distance is a sum over the bits, so min over k of (distance, k) for ALL patterns at once is a
+//              separable min-plus convolution: start from key(c_k) = (0, k), and for every bit b
+//              key(p) = min(key(p), key(p ^ 2^b) + (1, 0)).  v 2^v steps instead of distinct patterns x centroids (1 M
+//              instead of 487 M for a 4096 x 4096 layer at v = 16 with 8192 centroids).  The low nine bits within 512
+//              neighbouring patterns, the others on columns of four, with a grid barrier between.
+//   M-step     every occurring pattern adds cnt[p] to its cluster's total and to the counts of its set bits, several counts
+//              to a 64-bit atomic; then one thread per centroid
+//   assign     z through the label table in shared memory (v <= 16)
+// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 66 us a call (706 us with an E-step over (pattern,
+// centroid) pairs, a kernel per step and max_iter rounds of launches, of which those after convergence returned at once).
+// Of these ten grid barriers at 1.1 to 1.5 us, clearing and histogram 8 us, ranking 10 us, an E-step 3 + 6 us (half of it
+// the votes' atomics), an M-step 4 us, assignment 4 us.
 // Integer arithmetic only; results are bit-exact against the definition.
+#include <atomic>
 #include "btc_internal.cuh"
 
 namespace btc {
 
 constexpr int KM_VMAX = 20;                  // longest vector: the steps keep tables of 2^v entries
-constexpr int KM_VMAX_SLOTS = 32;            // vote counters per centroid
+constexpr int KM_THREADS = 1024;
+constexpr int KM_BINS = 2048;                // frequencies 0 .. 2046, and all larger ones together
+constexpr int KM_MAX_CTAS = 256;
+constexpr int KM_LOW = 9;                    // bits of the first half of an E-step: 512 patterns
+constexpr uint32_t KM_NONE = (255u << 16) | 0xffffu;
+constexpr int KM_MAX_WORDS = 11;             // 64-bit words that hold 21 counts of 32 bits, two each
+constexpr size_t KM_SMEM = 128 * 1024;
 
-struct KmState {
-    int done;         // 1: assignments unchanged in an E-step (the loop has ended)
-    int iters;        // E-steps run
-    int kc_eff;       // min(c, number of distinct vectors)
-    int n_unique;
-    int changed;      // set by the E-step of the current round
-    unsigned thr;     // frequency of the c-th most frequent distinct vector (1 when there are fewer than c)
-    int n_cand;       // distinct vectors more frequent than that (fewer than c): ranked pairwise; the ones exactly that
-                      // frequent follow them in the order of their packed words
+__device__ int g_km_status = 0;
+
+struct KmState {                             // zeroed by the host
+    unsigned arrived;     // grid barrier
+    int changed[2];       // set by the E-step of round i in slot i & 1
+    int n_over;           // patterns whose frequency is past the last bin
 };
 
-struct KmWorkspace {
+struct KmArgs {
+    const uint32_t *vecs;
+    size_t n;
+    int v, Kc, max_iter;
+    uint32_t *C;
+    uint16_t *z;
+    int *info;
     KmState *st;
-    uint32_t *cnt;        // [P]
-    uint32_t *label;      // [2][P], E-step i writes half i & 1
-    uint32_t *tot;        // [Kc]
-    uint32_t *ones;       // [Kc][KM_VMAX_SLOTS]
-    uint32_t *cand_p;     // [P] candidate patterns (unordered) ...
-    uint32_t *cand_c;     // [P] ... and their frequencies
+    uint32_t *cnt;        // [P] frequencies
+    uint32_t *seed;       // [P] key (0, k) at the centroids
+    uint32_t *key;        // [P] after the low bits
+    uint16_t *label;      // [P] assignment of the last E-step
+    uint32_t *bins;       // [KM_BINS] patterns per frequency
+    uint16_t *cols;       // [KM_BINS][KM_MAX_CTAS] the same per CTA
+    uint2 *over;          // [P] (frequency, pattern) past the last bin
+    unsigned long long *votes;   // [Kc][words]
+    int words, fields;    // 64-bit words per centroid, counts per word
 };
 
 __host__ __device__ inline size_t km_align(size_t x) { return (x + 255) & ~(size_t)255; }
 
-static KmWorkspace km_carve(void *ws, int v, int Kc)
+// Carves the workspace (ws may be null: returns the bytes needed).
+static size_t km_carve(KmArgs &a, void *ws, int v, int Kc, size_t n)
 {
     const size_t P = (size_t)1 << v;
-    unsigned char *p = reinterpret_cast<unsigned char *>(ws);
-    KmWorkspace w;
-    w.st = reinterpret_cast<KmState *>(p); p += km_align(sizeof(KmState));
-    w.cnt = reinterpret_cast<uint32_t *>(p); p += km_align(P * 4);
-    w.label = reinterpret_cast<uint32_t *>(p); p += km_align(2 * P * 4);
-    w.tot = reinterpret_cast<uint32_t *>(p); p += km_align((size_t)Kc * 4);
-    w.ones = reinterpret_cast<uint32_t *>(p); p += km_align((size_t)Kc * KM_VMAX_SLOTS * 4);
-    w.cand_p = reinterpret_cast<uint32_t *>(p); p += km_align(P * 4);
-    w.cand_c = reinterpret_cast<uint32_t *>(p);
-    return w;
+    size_t o = 0;
+    auto take = [&](size_t bytes) { void *p = static_cast<char *>(ws) + o; o += km_align(bytes); return p; };
+    a.fields = n < (1u << 21) ? 3 : 2;       // counts of 21 or 32 bits
+    a.words = (v + 1 + a.fields - 1) / a.fields;
+    a.st = static_cast<KmState *>(take(sizeof(KmState)));
+    a.cnt = static_cast<uint32_t *>(take(P * 4));
+    a.seed = static_cast<uint32_t *>(take(P * 4));
+    a.key = static_cast<uint32_t *>(take(P * 4));
+    a.label = static_cast<uint16_t *>(take(P * 2));
+    a.bins = static_cast<uint32_t *>(take(KM_BINS * 4));
+    a.cols = static_cast<uint16_t *>(take((size_t)KM_BINS * KM_MAX_CTAS * 2));
+    a.over = static_cast<uint2 *>(take(P * 8));
+    a.votes = static_cast<unsigned long long *>(take((size_t)Kc * a.words * 8));
+    return o;
 }
 
 static size_t km_workspace_bytes(int v, int Kc)
 {
-    const size_t P = (size_t)1 << v;
-    return km_align(sizeof(KmState)) + km_align(P * 4) + km_align(2 * P * 4) + km_align((size_t)Kc * 4) + km_align((size_t)Kc * KM_VMAX_SLOTS * 4) +
-           2 * km_align(P * 4);
+    KmArgs a;
+    return km_carve(a, nullptr, v, Kc, (size_t)1 << 31);   // (the wider counts)
 }
 
-__global__ void km_hist_kernel(const uint32_t *__restrict__ vecs, size_t n, uint32_t mask, uint32_t *__restrict__ cnt)
+// Barrier over the grid (co-resident: cooperative launch).  Bounded: false once about 2 s have passed.
+__device__ __forceinline__ bool km_sync(KmState *st, unsigned &target, int *s_ok)
 {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (; i < n; i += stride) atomicAdd(cnt + (vecs[i] & mask), 1u);
-}
-
-// Initial centroids: occurring pattern p goes to slot rank(p) if that is below c, where rank counts the patterns that
-// are more frequent, or as frequent with a smaller packed word.  Only patterns at least as frequent as the c-th most
-// frequent one can get a slot.  Those strictly more frequent (fewer than c) are ranked against one another; those
-// exactly as frequent (possibly many: frequencies of rare patterns tie) come after them in word order, which is a
-// prefix count, not a comparison of pairs.
-constexpr int KM_TILE = 2048;
-
-// One CTA: number of distinct vectors, and the largest threshold t with #{p : cnt[p] >= t} >= c (bisection over t).
-__global__ void __launch_bounds__(1024)
-km_threshold_kernel(const uint32_t *__restrict__ cnt, int P, int Kc, KmState *st)
-{
-    __shared__ unsigned s_red[32];
-    __shared__ unsigned s_val;
-    auto block_sum = [&](unsigned v) -> unsigned {
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            unsigned w = s_red[threadIdx.x];
-            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            if (threadIdx.x == 0) s_val = w;
-        }
-        __syncthreads();
-        return s_val;
-    };
-    // up to 65536 patterns (v <= 16) the thread's 64 frequencies stay in registers over the bisection
-    constexpr int KEEP = 64;
-    const bool kept = P <= KEEP * 1024;
-    uint32_t mine[KEEP];
-#pragma unroll
-    for (int i = 0; i < KEEP; ++i) {
-        const int p = threadIdx.x + i * 1024;
-        mine[i] = (kept && p < P) ? cnt[p] : 0u;
-    }
-    auto count_ge = [&](unsigned t) -> unsigned {
-        unsigned c = 0;
-        if (kept) {
-#pragma unroll
-            for (int i = 0; i < KEEP; ++i) c += (mine[i] >= t) ? 1u : 0u;
-        } else {
-            for (int p = threadIdx.x; p < P; p += blockDim.x) c += (cnt[p] >= t) ? 1u : 0u;
-        }
-        return block_sum(c);
-    };
-    unsigned mx = 0;
-    for (int p = threadIdx.x; p < P; p += blockDim.x) mx = max(mx, cnt[p]);
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    target += gridDim.x;
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = 0;
-    for (int i = 0; i < 32; ++i) mx = max(mx, s_red[i]);
-    const unsigned n_unique = count_ge(1u);
-    unsigned lo = 1u, hi = max(mx, 1u);                     // invariant: count_ge(lo) >= min(c, n_unique)
-    if (n_unique > (unsigned)Kc) {
-        while (lo < hi) {
-            const unsigned mid = lo + (hi - lo + 1u) / 2u;
-            if (count_ge(mid) >= (unsigned)Kc) lo = mid; else hi = mid - 1u;
-        }
-    }
     if (threadIdx.x == 0) {
-        st->n_unique = (int)n_unique;
-        st->kc_eff = min(Kc, (int)n_unique);
-        st->thr = (n_unique > (unsigned)Kc) ? lo : 1u;
-    }
-}
-
-__global__ void km_candidates_kernel(const uint32_t *__restrict__ cnt, int P, uint32_t *__restrict__ cand_p, uint32_t *__restrict__ cand_c, KmState *st)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const uint32_t c = cnt[p];
-    if (c > st->thr) {                                      // strictly more frequent than the c-th: fewer than c of them
-        const int pos = atomicAdd(&st->n_cand, 1);
-        cand_p[pos] = (uint32_t)p;
-        cand_c[pos] = c;
-    }
-}
-
-// (frequency, word) of a candidate as one key: larger key = earlier slot.
-__device__ __forceinline__ unsigned long long km_key(uint32_t c, uint32_t p) { return ((unsigned long long)c << 32) | (0xffffffffu - p); }
-
-constexpr int KM_RANK_THREADS = 64;                         // small blocks: a few thousand candidates should still fill the SMs
-__global__ void __launch_bounds__(KM_RANK_THREADS)
-km_init_rank_kernel(const uint32_t *__restrict__ cand_p, const uint32_t *__restrict__ cand_c, int Kc, uint32_t *__restrict__ C, const KmState *st)
-{
-    __shared__ __align__(16) unsigned long long s_key[KM_TILE];
-    const int L = st->n_cand;
-    if ((int)(blockIdx.x * blockDim.x) >= L) return;        // (uniform over the block)
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = i < L;
-    const uint32_t p = live ? cand_p[i] : 0u;
-    const unsigned long long mine = live ? km_key(cand_c[i], p) : ~0ull;
-    int rank = 0;
-    for (int q0 = 0; q0 < L; q0 += KM_TILE) {
-        __syncthreads();
-        for (int j = threadIdx.x; j < KM_TILE; j += blockDim.x)
-            s_key[j] = (q0 + j < L) ? km_key(cand_c[q0 + j], cand_p[q0 + j]) : 0ull;     // (key 0 ranks before nothing)
-        __syncthreads();
-#pragma unroll 8
-        for (int j = 0; j < KM_TILE; ++j) rank += (s_key[j] > mine) ? 1 : 0;
-    }
-    if (live && rank < Kc) C[rank] = p;
-}
-
-// The patterns exactly as frequent as the c-th most frequent one follow the strictly more frequent ones in the order
-// of their packed words: rank = n_cand + (number of such patterns with a smaller word), a prefix count over p.
-__global__ void __launch_bounds__(1024)
-km_ties_kernel(const uint32_t *__restrict__ cnt, int P, int Kc, uint32_t *__restrict__ C, const KmState *st)
-{
-    // each warp takes a contiguous range of patterns and walks it 32 at a time (coalesced); the order inside a step comes
-    // from a ballot, the order of the warps from a prefix over their totals
-    __shared__ int s_tot[32];
-    const unsigned thr = st->thr;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int seg = (((P + 31) / 32) + 31) & ~31;           // patterns per warp, a multiple of 32
-    const int p_begin = warp * seg;
-    int total = 0;
-    for (int q = p_begin; q < p_begin + seg; q += 32) {
-        const int p = q + lane;
-        total += __popc(__ballot_sync(0xffffffffu, p < P && cnt[p] == thr));
-    }
-    if (lane == 0) s_tot[warp] = total;
-    __syncthreads();
-    int rank = st->n_cand;
-    for (int w = 0; w < warp; ++w) rank += s_tot[w];
-    for (int q = p_begin; q < p_begin + seg; q += 32) {
-        const int p = q + lane;
-        const bool tie = p < P && cnt[p] == thr;
-        const unsigned b = __ballot_sync(0xffffffffu, tie);
-        if (tie) {
-            const int r = rank + __popc(b & ((1u << lane) - 1u));
-            if (r < Kc) C[r] = (uint32_t)p;
-        }
-        rank += __popc(b);
-    }
-}
-
-__global__ void __launch_bounds__(256)
-km_estep_kernel(const uint32_t *__restrict__ cnt, int P, const uint32_t *__restrict__ C, uint32_t *__restrict__ label, KmState *st)
-{
-    __shared__ __align__(16) uint32_t s_C[KM_TILE];
-    if (st->done) return;                                   // (uniform over the grid: set only between launches)
-    const int it = st->iters, kc = st->kc_eff;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = (p < P) && cnt[p] != 0u;
-    uint32_t best = 0xffffffffu;
-    for (int k0 = 0; k0 < kc; k0 += KM_TILE) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < KM_TILE; i += blockDim.x) s_C[i] = (k0 + i < kc) ? C[k0 + i] : 0u;
-        __syncthreads();
-        if (live) {
-            const int lim = min(KM_TILE, kc - k0);
-            int i = 0;
-            for (; i + 4 <= lim; i += 4) {
-                const uint4 c = *reinterpret_cast<const uint4 *>(s_C + i);
-                best = min(best, ((uint32_t)__popc((uint32_t)p ^ c.x) << 16) | (uint32_t)(k0 + i));
-                best = min(best, ((uint32_t)__popc((uint32_t)p ^ c.y) << 16) | (uint32_t)(k0 + i + 1));
-                best = min(best, ((uint32_t)__popc((uint32_t)p ^ c.z) << 16) | (uint32_t)(k0 + i + 2));
-                best = min(best, ((uint32_t)__popc((uint32_t)p ^ c.w) << 16) | (uint32_t)(k0 + i + 3));
+        unsigned seen;
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(&st->arrived) : "memory");
+        const long long t0 = clock64();
+        int ok = 1;
+        for (;;) {
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&st->arrived) : "memory");
+            if ((int)(seen - target) >= 0) break;
+            if (clock64() - t0 > 4000000000LL) {
+                atomicExch(&g_km_status, (int)BTC_ERR_TIMEOUT);
+                ok = 0;
+                break;
             }
-            for (; i < lim; ++i) best = min(best, ((uint32_t)__popc((uint32_t)p ^ s_C[i]) << 16) | (uint32_t)(k0 + i));
+        }
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        *s_ok = ok;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+}
+
+// f(word) for every vector of [begin, end): 16-byte loads, four in flight.
+template <typename F>
+__device__ __forceinline__ void km_stream(const uint32_t *__restrict__ vecs, size_t begin, size_t end, F f)
+{
+    if ((reinterpret_cast<uintptr_t>(vecs) & 15u) == 0) {   // (begin is a multiple of 4)
+        const uint4 *src = reinterpret_cast<const uint4 *>(vecs);
+        const size_t q1 = end / 4;
+        for (size_t q0 = begin / 4; q0 < q1; q0 += 4 * KM_THREADS) {
+            uint4 w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const size_t q = q0 + threadIdx.x + u * KM_THREADS;
+                if (q < q1) w[u] = __ldg(src + q);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const size_t q = q0 + threadIdx.x + u * KM_THREADS;
+                if (q < q1) { f(4 * q, w[u].x); f(4 * q + 1, w[u].y); f(4 * q + 2, w[u].z); f(4 * q + 3, w[u].w); }
+            }
+        }
+        begin = end & ~(size_t)3;
+    }
+    for (size_t i = begin + threadIdx.x; i < end; i += KM_THREADS) f(i, __ldg(vecs + i));
+}
+
+__global__ void __launch_bounds__(KM_THREADS, 1)
+km_kernel(const KmArgs a)
+{
+    extern __shared__ __align__(16) unsigned char km_smem[];
+    __shared__ int s_ok;
+    __shared__ uint32_t s_warp[32];
+    uint32_t *sm = reinterpret_cast<uint32_t *>(km_smem);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int G = gridDim.x, b = blockIdx.x, v = a.v, P = 1 << v, Kc = a.Kc;
+    const uint32_t mask = (uint32_t)P - 1u;
+    const int gid = b * KM_THREADS + tid, gthreads = G * KM_THREADS;
+    unsigned target = 0;
+
+    // ---- clear what the later steps add to
+    for (int i = gid; i < P; i += gthreads) { a.cnt[i] = 0u; a.seed[i] = KM_NONE; }
+    for (int i = gid; i < KM_BINS; i += gthreads) a.bins[i] = 0u;
+    for (int i = gid; i < Kc; i += gthreads) a.C[i] = 0u;
+    for (int i = gid; i < KM_BINS * KM_MAX_CTAS / 8; i += gthreads) reinterpret_cast<uint4 *>(a.cols)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t i = gid; i < (size_t)Kc * a.words; i += gthreads) a.votes[i] = 0ull;
+
+    // ---- histogram
+    const size_t share = ((a.n + G - 1) / G + 3) & ~(size_t)3;
+    const size_t v0 = min(a.n, share * b), v1 = min(a.n, share * (b + 1));
+    if (v <= 16) {
+        const int hw = max(P / 2, 1);
+        for (int i = tid; i < hw; i += KM_THREADS) sm[i] = 0u;
+        constexpr size_t MOST = 65532;                       // (16-bit counters; a multiple of 4)
+        bool cleared = false;
+        for (size_t c0 = v0; c0 < v1 || !cleared; c0 += MOST) {
+            __syncthreads();
+            if (c0 < v1) km_stream(a.vecs, c0, min(v1, c0 + MOST), [&](size_t, uint32_t w) { w &= mask; atomicAdd(sm + (w >> 1), 1u << (16 * (w & 1u))); });
+            if (!cleared) { if (!km_sync(a.st, target, &s_ok)) return; cleared = true; }   // (everybody's counters are clear)
+            __syncthreads();
+            for (int i = tid; i < hw; i += KM_THREADS) {
+                const uint32_t w = sm[i];
+                if (w & 0xffffu) atomicAdd(a.cnt + 2 * i, w & 0xffffu);
+                if (w >> 16) atomicAdd(a.cnt + 2 * i + 1, w >> 16);
+                sm[i] = 0u;
+            }
+        }
+    } else {
+        if (!km_sync(a.st, target, &s_ok)) return;
+        km_stream(a.vecs, v0, v1, [&](size_t, uint32_t w) { atomicAdd(a.cnt + (w & mask), 1u); });
+    }
+    if (!km_sync(a.st, target, &s_ok)) return;
+
+    // ---- patterns per frequency: this CTA's patterns [p0, p1), their frequencies kept in shared memory
+    const int per = (P + G - 1) / G, p0 = min(P, per * b), p1 = min(P, p0 + per);
+    uint32_t *s_bins = sm, *s_cnt = sm + KM_BINS + 1;
+    for (int i = tid; i < KM_BINS; i += KM_THREADS) s_bins[i] = 0u;
+    __syncthreads();
+    for (int p = p0 + tid; p < p1; p += KM_THREADS) {
+        const uint32_t c = __ldcg(a.cnt + p);
+        s_cnt[p - p0] = c;
+        if (c) atomicAdd(s_bins + min(c, (uint32_t)KM_BINS - 1u), 1u);
+        if (c >= KM_BINS - 1) a.over[atomicAdd(&a.st->n_over, 1)] = make_uint2(c, (uint32_t)p);
+    }
+    __syncthreads();
+    for (int i = tid; i < KM_BINS; i += KM_THREADS) {
+        const uint32_t h = s_bins[i];
+        if (h) { a.cols[(size_t)i * KM_MAX_CTAS + b] = (uint16_t)h; atomicAdd(a.bins + i, h); }
+    }
+    if (!km_sync(a.st, target, &s_ok)) return;
+
+    // ---- suffix sums: s_bins[i] = patterns of frequency bin >= i
+    {
+        uint32_t x1 = __ldcg(a.bins + KM_BINS - 1 - 2 * tid), x0 = __ldcg(a.bins + KM_BINS - 2 - 2 * tid);   // (from the top)
+        if (tid == KM_BINS / 2 - 1) x0 = 0u;                 // (frequency 0 does not occur)
+        uint32_t s = x1 + x0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, s, o); if (lane >= o) s += t; }
+        if (lane == 31) s_warp[warp] = s;
+        __syncthreads();
+        if (warp == 0) {
+            uint32_t w = s_warp[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, w, o); if (lane >= o) w += t; }
+            s_warp[lane] = w;
+        }
+        __syncthreads();
+        if (warp) s += s_warp[warp - 1];
+        s_bins[KM_BINS - 2 - 2 * tid] = s;
+        s_bins[KM_BINS - 1 - 2 * tid] = s - x0;
+        if (tid == 0) s_bins[KM_BINS] = 0u;
+        __syncthreads();
+    }
+    const int n_unique = (int)s_bins[1], kc = min(Kc, n_unique);
+
+    // ---- ranks (a warp per pattern that can have one below c): centroids, and the seeds of the first E-step.  The counts of the
+    //      CTAs before this one are one 16-byte load per lane; four patterns' loads are in flight.
+    for (int i0 = warp; i0 < p1 - p0; i0 += 4 * (KM_THREADS / 32)) {
+        uint4 q[4];
+        bool need[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * (KM_THREADS / 32);
+            const uint32_t c = i < p1 - p0 ? s_cnt[i] : 0u;
+            need[u] = c != 0u && c < KM_BINS - 1 && s_bins[c + 1] < (uint32_t)Kc;
+            if (need[u]) q[u] = __ldcg(reinterpret_cast<const uint4 *>(a.cols + (size_t)c * KM_MAX_CTAS) + lane);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * (KM_THREADS / 32);
+            const uint32_t c = i < p1 - p0 ? s_cnt[i] : 0u;
+            const bool over = c >= KM_BINS - 1;
+            if (!need[u] && !over) continue;
+            const uint32_t p = (uint32_t)(p0 + i);
+            uint32_t r = 0;
+            if (over) {
+                const int m = (int)s_bins[KM_BINS - 1];
+                for (int j = lane; j < m; j += 32) {
+                    const uint2 o = __ldcg(a.over + j);
+                    r += (o.x > c || (o.x == c && o.y < p)) ? 1u : 0u;
+                }
+            } else {
+                const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (8 * lane + k < b) r += (w[k >> 1] >> (16 * (k & 1))) & 0xffffu;
+                for (int j = lane; j < i; j += 32) r += s_cnt[j] == c ? 1u : 0u;
+                if (lane == 0) r += s_bins[c + 1];
+            }
+            r = __reduce_add_sync(0xffffffffu, r);
+            if (lane == 0 && r < (uint32_t)Kc) { a.C[r] = p; a.seed[p] = r; }
         }
     }
-    if (live) {
-        const uint32_t z = best & 0xffffu;
-        uint32_t *cur = label + (size_t)(it & 1) * P, *prev = label + (size_t)((it & 1) ^ 1) * P;
-        cur[p] = z;
-        if (it == 0 || prev[p] != z) st->changed = 1;       // (benign race: every writer stores 1)
-    }
-}
+    if (!km_sync(a.st, target, &s_ok)) return;
 
-// After an E-step: count it; if nothing changed the loop is over (its M-step does not run).
-__global__ void km_round_kernel(KmState *st)
-{
-    if (st->done) return;
-    st->iters += 1;
-    if (!st->changed) st->done = 1;
-    st->changed = 0;
-}
-
-__global__ void km_vote_kernel(const uint32_t *__restrict__ cnt, int P, int v, const uint32_t *__restrict__ label,
-                               uint32_t *__restrict__ tot, uint32_t *__restrict__ ones, const KmState *st)
-{
-    if (st->done) return;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const uint32_t c = cnt[p];
-    if (!c) return;
-    const uint32_t k = label[(size_t)((st->iters - 1) & 1) * P + p];     // the E-step just counted wrote half (iters - 1) & 1
-    atomicAdd(tot + k, c);
-    for (int t = 0; t < v; ++t)
-        if ((p >> t) & 1) atomicAdd(ones + (size_t)k * KM_VMAX_SLOTS + t, c);
-}
-
-__global__ void km_update_kernel(int v, uint32_t *__restrict__ C, uint32_t *__restrict__ tot, uint32_t *__restrict__ ones, const KmState *st)
-{
-    if (st->done) return;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= st->kc_eff) return;
-    const uint32_t n = tot[k];
-    if (n) {
-        uint32_t w = 0;
-        for (int t = 0; t < v; ++t) {
-            const uint32_t o = ones[(size_t)k * KM_VMAX_SLOTS + t];
-            if (o >= n - o) w |= 1u << t;                   // at least as many +1 as -1: sign(0) = +1
-            ones[(size_t)k * KM_VMAX_SLOTS + t] = 0;
+    const int low = min(v, KM_LOW), high = v - low;
+    int it = 0, done = 0;
+    while (it < a.max_iter && !done) {
+        // ---- E-step, low bits: 512 neighbouring patterns per half CTA
+        for (int u0 = 2 * b; u0 < (P >> low); u0 += 2 * G) {
+            const int half = tid >> KM_LOW, u = u0 + half, e = tid & ((1 << KM_LOW) - 1);
+            const bool live = u < (P >> low) && e < (1 << low);
+            uint32_t k = KM_NONE;
+            const int p = (u << low) + e;
+            if (live) { k = __ldcg(a.seed + p); a.seed[p] = KM_NONE; }
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1)
+                if (o < (1 << low)) k = min(k, __shfl_xor_sync(0xffffffffu, k, o) + 0x10000u);
+#pragma unroll
+            for (int o = 32; o < (1 << KM_LOW); o <<= 1)
+                if (o < (1 << low)) {                        // (uniform)
+                    __syncthreads();
+                    sm[tid] = k;
+                    __syncthreads();
+                    k = min(k, sm[tid ^ o] + 0x10000u);
+                }
+            if (live) a.key[p] = k;
         }
-        C[k] = w;
-        tot[k] = 0;
+        if (!km_sync(a.st, target, &s_ok)) return;
+        // ---- E-step, high bits, on columns of four patterns; labels and votes
+        const int cols = min(4, 1 << low), E = cols << high, sh = __ffs(cols) - 1;
+        int changed = 0;
+        for (int u = b; u < (1 << low) / cols; u += G) {
+            __syncthreads();
+            for (int e = tid; e < E; e += KM_THREADS) sm[e] = __ldcg(a.key + ((e >> sh) << low) + u * cols + (e & (cols - 1)));
+            for (int h = 0; h < high; ++h) {
+                __syncthreads();
+                const int o = cols << h;
+                for (int q = tid; q < E / 2; q += KM_THREADS) {
+                    const int e = (q & (o - 1)) | ((q & ~(o - 1)) << 1);
+                    const uint32_t x = sm[e], y = sm[e + o];
+                    sm[e] = min(x, y + 0x10000u);
+                    sm[e + o] = min(y, x + 0x10000u);
+                }
+            }
+            __syncthreads();
+            for (int e = tid; e < E; e += KM_THREADS) {
+                const int p = ((e >> sh) << low) + u * cols + (e & (cols - 1));
+                const uint32_t c = __ldcg(a.cnt + p);
+                if (!c) continue;
+                const uint32_t z = sm[e] & 0xffffu;
+                if (it == 0 || a.label[p] != z) changed = 1; // (this thread wrote it in the round before)
+                a.label[p] = (uint16_t)z;
+                unsigned long long *vote = a.votes + (size_t)z * a.words;
+                const int bits = a.fields == 3 ? 21 : 32;
+                uint32_t pat = ((uint32_t)p << 1) | 1u;      // count 0: the total; count 1 + t: element t is +1
+                for (int w = 0; w < a.words; ++w) {
+                    unsigned long long add = 0ull;
+                    for (int f = 0; f < a.fields; ++f) {
+                        if (pat & 1u) add |= (unsigned long long)c << (bits * f);
+                        pat >>= 1;
+                    }
+                    if (add) atomicAdd(vote + w, add);
+                }
+            }
+        }
+        if (__syncthreads_or(changed) && tid == 0) a.st->changed[it & 1] = 1;
+        if (gid == 0) a.st->changed[(it + 1) & 1] = 0;       // (last read before the barrier just passed)
+        if (!km_sync(a.st, target, &s_ok)) return;
+        done = *reinterpret_cast<volatile int *>(&a.st->changed[it & 1]) == 0;
+        ++it;
+        if (done) break;                                     // (its votes are dropped: nothing changed, no M-step)
+        // ---- M-step, and the seeds of the next E-step
+        const int bits = a.fields == 3 ? 21 : 32;
+        const unsigned long long fmask = (1ull << bits) - 1ull;
+        for (int k = tid * G + b; k < kc; k += gthreads) {               // (spread over the SMs)
+            unsigned long long *vote = a.votes + (size_t)k * a.words, x[KM_MAX_WORDS];
+#pragma unroll
+            for (int w = 0; w < KM_MAX_WORDS; ++w)
+                if (w < a.words) x[w] = __ldcg(vote + w);
+            const uint32_t tot = (uint32_t)(x[0] & fmask);
+            uint32_t pat = 0u;                                           // bit 0: the total, bit 1 + t: element t
+            int bit = 0;
+#pragma unroll
+            for (int w = 0; w < KM_MAX_WORDS; ++w)
+                if (w < a.words) {
+                    vote[w] = 0ull;
+                    for (int f = 0; f < a.fields; ++f, ++bit) {
+                        const uint32_t o = (uint32_t)(x[w] & fmask);
+                        x[w] >>= bits;
+                        if (o >= tot - o) pat |= 1u << bit;              // at least as many +1 as -1: sign(0) = +1
+                    }
+                }
+            uint32_t c = (pat >> 1) & mask;
+            if (tot) a.C[k] = c; else c = __ldcg(a.C + k);               // (an empty cluster keeps its centroid)
+            if (it < a.max_iter) atomicMin(a.seed + c, (uint32_t)k);
+        }
+        if (it < a.max_iter && !km_sync(a.st, target, &s_ok)) return;
     }
+
+    // ---- assignments
+    if (v <= 16) {
+        __syncthreads();
+        uint16_t *tab = reinterpret_cast<uint16_t *>(km_smem);
+        if (P >= 8) {
+            for (int i = tid; i < P / 8; i += KM_THREADS) reinterpret_cast<uint4 *>(tab)[i] = __ldcg(reinterpret_cast<const uint4 *>(a.label) + i);
+        } else if (tid < P) {
+            tab[tid] = __ldcg(a.label + tid);
+        }
+        __syncthreads();
+        km_stream(a.vecs, v0, v1, [&](size_t i, uint32_t w) { a.z[i] = tab[w & mask]; });
+    } else {
+        km_stream(a.vecs, v0, v1, [&](size_t i, uint32_t w) { a.z[i] = __ldcg(a.label + (w & mask)); });
+    }
+    if (gid == 0) { a.info[0] = it; a.info[1] = kc; a.info[2] = n_unique; a.info[3] = done; }
 }
 
-__global__ void km_assign_kernel(const uint32_t *__restrict__ vecs, size_t n, uint32_t mask, int P, const uint32_t *__restrict__ label,
-                                 uint16_t *__restrict__ z, int *__restrict__ info, const KmState *st)
+int km_status_reset()
 {
-    const uint32_t *fin = label + (size_t)((st->iters - 1) & 1) * P;
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) { info[0] = st->iters; info[1] = st->kc_eff; info[2] = st->n_unique; info[3] = st->done; }
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (; i < n; i += stride) z[i] = (uint16_t)fin[vecs[i] & mask];
+    const int zero = 0;
+    cudaError_t e = cudaMemcpyToSymbol(g_km_status, &zero, sizeof(int));
+    return e == cudaSuccess ? BTC_OK : cuda_fail(e);
+}
+
+int km_status_read(int *out)
+{
+    int v = 0;
+    cudaError_t e = cudaMemcpyFromSymbol(&v, g_km_status, sizeof(int));
+    if (e != cudaSuccess) return cuda_fail(e);
+    *out = v;
+    return BTC_OK;
 }
 
 }  // namespace btc
@@ -320,26 +423,27 @@ extern "C" BTC_API int btc_codebook_kmeans(const uint32_t *vecs, size_t n, int v
     if (workspace_bytes < km_workspace_bytes(v, Kc)) return BTC_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(workspace) % 256) return BTC_ERR_ALIGN;
     cudaStream_t s = (cudaStream_t)stream;
-    const int P = 1 << v;
-    const uint32_t mask = (v == 32) ? 0xffffffffu : ((1u << v) - 1u);
-    KmWorkspace w = km_carve(workspace, v, Kc);
-    cudaError_t e = cudaMemsetAsync(workspace, 0, km_workspace_bytes(v, Kc), s);
+    KmArgs a;
+    km_carve(a, workspace, v, Kc, n);
+    a.vecs = vecs; a.n = n; a.v = v; a.Kc = Kc; a.max_iter = max_iter; a.C = C_words; a.z = z; a.info = info;
+    static std::atomic<int> sms_of[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
-    e = cudaMemsetAsync(C_words, 0, (size_t)Kc * 4, s);
-    if (e != cudaSuccess) return cuda_fail(e);
-    const unsigned nb = (unsigned)((n + 255) / 256 < 148 * 32 ? (n + 255) / 256 : 148 * 32);
-    const unsigned pb = (unsigned)((P + 255) / 256), kb = (unsigned)((Kc + 255) / 256);
-    km_hist_kernel<<<nb, 256, 0, s>>>(vecs, n, mask, w.cnt);
-    km_threshold_kernel<<<1, 1024, 0, s>>>(w.cnt, P, Kc, w.st);
-    km_candidates_kernel<<<pb, 256, 0, s>>>(w.cnt, P, w.cand_p, w.cand_c, w.st);
-    km_init_rank_kernel<<<(unsigned)((P + KM_RANK_THREADS - 1) / KM_RANK_THREADS), KM_RANK_THREADS, 0, s>>>(w.cand_p, w.cand_c, Kc, C_words, w.st);
-    km_ties_kernel<<<1, 1024, 0, s>>>(w.cnt, P, Kc, C_words, w.st);
-    for (int it = 0; it < max_iter; ++it) {
-        km_estep_kernel<<<pb, 256, 0, s>>>(w.cnt, P, C_words, w.label, w.st);
-        km_round_kernel<<<1, 1, 0, s>>>(w.st);
-        km_vote_kernel<<<pb, 256, 0, s>>>(w.cnt, P, v, w.label, w.tot, w.ones, w.st);
-        km_update_kernel<<<kb, 256, 0, s>>>(v, C_words, w.tot, w.ones, w.st);
+    int sms = dev < 64 ? sms_of[dev].load(std::memory_order_relaxed) : 0;
+    if (!sms) {
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(km_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KM_SMEM);
+        if (e != cudaSuccess) return cuda_fail(e);
+        if (sms > KM_MAX_CTAS) sms = KM_MAX_CTAS;
+        if (dev < 64) sms_of[dev].store(sms, std::memory_order_relaxed);
     }
-    km_assign_kernel<<<nb, 256, 0, s>>>(vecs, n, mask, P, w.label, z, info, w.st);
-    return cuda_check_launch();
+    // a CTA per SM, fewer where there is little to do (a barrier costs more the more of them there are)
+    const size_t want = (n + 1023) / 1024 > (size_t)((1 << v) + 511) / 512 ? (n + 1023) / 1024 : (size_t)((1 << v) + 511) / 512;
+    const int grid = want < (size_t)sms ? (int)want : sms;
+    e = cudaMemsetAsync(a.st, 0, sizeof(KmState), s);
+    if (e != cudaSuccess) return cuda_fail(e);
+    void *params[] = {&a};
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(km_kernel), dim3((unsigned)grid), dim3(KM_THREADS), params, KM_SMEM, s);
+    return e == cudaSuccess ? BTC_OK : cuda_fail(e);
 }

@@ -69,6 +69,25 @@ def test_kmeans_matches_oracle_bit_for_bit(n, v, Kc, max_iter, kind):
     assert info[3] == int(converged)
 
 
+@pytest.mark.parametrize("n,v,Kc,offset", [(300000, 8, 100, 0), (120000, 3, 5, 1), (66000, 16, 2500, 3), (40000, 17, 500, 2),
+                                           (5000, 10, 400, 0), (2049, 9, 512, 1)])
+def test_kmeans_edges(n, v, Kc, offset):
+    """Where the single launch can go wrong: frequencies past the last bin of the frequency histogram, vectors that start
+    off a 16-byte boundary with a ragged end, one more and one less bit than a half of the E-step covers, the
+    histogram in shared memory (v = 16) and in global memory (v = 17)."""
+    B = _vectors(n, v, "noisy", seed=n + v)
+    C_ref, z_ref, iters_ref, n_unique, converged = km.optimize_codebook(B, Kc, 4, with_flag=True)
+    buf = torch.zeros(n + offset, dtype=torch.int32, device="cuda")
+    buf[offset:] = torch.from_numpy(km.pack_words(B).view(np.int32).copy()).cuda()
+    C, z, info = btc.codebook_kmeans(buf[offset:], v, Kc, 4)
+    torch.cuda.synchronize()
+    k_eff = min(Kc, n_unique)
+    assert info.tolist() == [iters_ref, k_eff, n_unique, int(converged)]
+    assert np.array_equal(C.cpu().numpy().view(np.uint32)[:k_eff], km.pack_words(C_ref))
+    assert np.array_equal(z.cpu().numpy().view(np.uint16).astype(np.int64), z_ref)
+    assert btc.device_status() == 0
+
+
 def test_kmeans_feeds_the_layer():
     """The construction's outputs are the layer's inputs: centroids -> btc_codebook_pack, z -> idx; decoding them
     gives the nearest-centroid approximation of the sign matrix, whose Hamming error equals the oracle's objective."""
