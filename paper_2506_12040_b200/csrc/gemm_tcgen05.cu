@@ -6,7 +6,7 @@
 // row m, and a warp stores 32 consecutive n for one m (coalesced).  The decoded tile is pure +-1 and the row scale is
 // applied in the fp32 epilogue, which is exact for a row-wise alpha.
 //
-// Two kernels: gemm_v16t_kernel (v = 16; decoded weights go straight into tensor memory, see its header) and
+// Two kernels: gemm_ts_kernel (even v from 8 to 24; decoded weights go straight into tensor memory, see its header) and
 // gemm_tcgen05_kernel (any v; one thread per weight row writes the +-1 tile into shared memory):
 //   warp 0     TMA producer: x tiles [BM rows x 64 k] -> shared memory
 //   warp 1     MMA issuer: one elected thread issues tcgen05.mma for every 64-wide k step
@@ -18,6 +18,7 @@
 // Every mbarrier wait is bounded: after ~2 s of polling the CTA raises a status word, stops waiting and runs to
 // completion (the output is then undefined and btc_device_status reports the timeout).
 #include <cuda.h>
+#include <atomic>
 #include "btc_internal.cuh"
 
 namespace btc {
@@ -128,15 +129,36 @@ struct GemmParams {
     int k_tiles;             // ceil(K / 64)
 };
 
-// sum_k x[m,k] in fp32, one warp per row (needed only for the mean term).
-__global__ void rowsum_kernel(const void *x, int x_dt, int M, int K, float *out)
+// sum_k x[m,k] in fp32 (needed only for the mean term), a CTA per row.  The contraction that follows starts right away and
+// waits for the sums in its epilogue.
+__global__ void __launch_bounds__(256)
+rowsum_kernel(const void *x, int x_dt, int K, float *out)
 {
-    const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (m >= M) return;
+    __shared__ float s_part[8];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (after the wait: x is complete for the contraction too)
+    const int m = blockIdx.x, lane = threadIdx.x & 31;
     float s = 0.f;
-    for (int k = threadIdx.x & 31; k < K; k += 32) s += load_as_float(x, x_dt, (size_t)m * K + k);
+    const uint4 *row = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(x) + (size_t)m * K);   // (K is a multiple of 8)
+#pragma unroll 4
+    for (int i = threadIdx.x; i < K / 8; i += 256) {
+        const uint4 q = __ldg(row + i);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 f = x_dt == BTC_F16 ? __half22float2(*reinterpret_cast<const __half2 *>(&w[j]))
+                                             : make_float2(__uint_as_float(w[j] << 16), __uint_as_float(w[j] & 0xffff0000u));
+            s += f.x + f.y;
+        }
+    }
     s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) out[m] = s;
+    if (lane == 0) s_part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+        for (int w = 0; w < 8; ++w) t += s_part[w];
+        out[m] = t;
+    }
 }
 
 template <int BM, int STAGES>
@@ -255,6 +277,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams
         // ------------------------------------------------------------ epilogue
         mbar_wait(bar_accum, 0, s_abort);
         tc_fence_after();
+        asm volatile("griddepcontrol.wait;" ::: "memory");    // the row sums
         const int nrow = n0 + r;
         const float al = __half2float(a.alpha[n]);
         const float mu = a.mu ? __half2float(a.mu[n]) : 0.f;
@@ -287,45 +310,62 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams
     if (warp == 2) tmem_dealloc(tmem_d, BM);
 }
 
-// ------------------------------------------------------------------------------------ v = 16: shared declarations
-// For v = 16 a 64-wide k step is four blocks.  The codeword table of the "fp16 layout" keeps the bit of weight t at
-// (t & 1) * 16 + 4 + (t >> 1), so ((~w << (11 - j)) & 0x80008000) | {1.0, 1.0} is the pair of weights (2j, 2j+1) as +-1
-// in bf16 / fp16: one shift and one LOP3 per pair.  Index tiles (128 rows x 64 blocks = 16 k steps, 128-byte swizzle)
-// arrive by TMA; the table is bulk-copied into shared memory when it fits.
+// ------------------------------------------------------------------------------------ even v, weights in tensor memory
+// With both operands in shared memory the kernel above is bound by shared-memory bandwidth: per 64-wide k step the
+// tensor core reads the A and B tiles while the decode warps write 16 KB of A and TMA writes the x tile, more than
+// the 128 bytes per clock an SM's shared memory delivers.  Here the decoded +-1 tile never touches shared memory: each
+// decode thread owns one weight row = one tensor-memory lane, expands the row's 64 weights of a k step into 32
+// registers and stores them with tcgen05.st into a ring of A tiles in tensor memory (32 columns per k step); the MMAs
+// take A from tensor memory and only the x tile from shared memory.
+//   warp 0 TMA producer (x tiles, index tiles, table) | warp 1 MMA issuer | warp 2 tensor-memory allocation
+//   warps 4-19: four groups of four warps; group g expands the stages g, g + 4, ...; then all 16 run the epilogue.
+// Tensor memory (512 columns): accumulator in columns [0, BM), A ring of STAGES x 32 KS columns from column 256.
+//
+// Index tiles (128 rows x 64 blocks = V k steps, 128-byte swizzle) arrive by TMA; the codeword table of the "fp16 layout" is
+// bulk-copied into shared memory when it fits.  That layout keeps the bits of a weight pair (2j, 2j+1) of a block at
+// P0 + j of both halves, so ((~w << (15 - P0 - j)) & 0x80008000) | {1.0, 1.0} is the pair as +-1 in bf16 / fp16: one
+// shift and one LOP3 per pair.  v = 16: a k step is four whole blocks.  Other v: a step starts (64 step) mod v weights
+// into a block; the V / gcd(V, 64) starting points are compiled in.
+//
+// An x tile has bn rows (a multiple of 16 up to BM; the UMMA N), chosen so that the tiles of M are even and the rows past M
+// few.  Few tiles and a long K (SPLIT): the CTAs of a cluster along grid.z share K, leave their accumulators in shared
+// memory, and each adds a share of the columns over the cluster in a fixed order (distributed shared memory).
+//
+// Launched with programmatic stream serialisation: barriers, tensor memory, table and first indices are ready before
+// the predecessor has finished; x is read after it (or right away where the predecessor is the row-sum kernel, which
+// itself waited for it; then the epilogue waits).  It does not let its own successors start early: their CTAs
+// would pile up on the SMs that a round of tiles leaves idle (a transform behind it ran 15 us longer).
 constexpr int G2_DWARPS = 16;                    // decode warps (four groups of four)
 constexpr int G2_THREADS = 128 + G2_DWARPS * 32;
 constexpr uint32_t G2_IDX_BYTES = 128 * 128;     // one index tile
+constexpr int G4_A_COL0 = 256;
 
 struct Gemm2Params {
     LinearArgs a;
-    const float *sumx;
+    const float *sumx;       // [M] row sums of x, or nullptr
     const uint32_t *tab;     // fp16-layout codeword words [Kc4]
     int k_tiles;
     int tab_bytes;           // > 0: table staged in shared memory
+    int bn;                  // rows of x per tile
 };
 
 struct SplitArgs {
-    int split_tiles;         // k tiles (a multiple of 16: whole index tiles) per CTA along grid.z
-    float *part;             // raw partial sums [grid.z][M][N]
+    int split_tiles;         // k tiles (whole index tiles) per CTA along grid.z
 };
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
-
-// ------------------------------------------------------------------------------------ v = 16 and v = 20, weights in tensor memory
-// With both operands in shared memory the kernel above is bound by shared-memory bandwidth: per 64-wide k step the
-// tensor core reads the A and B tiles while the decode warps write 16 KB of A and TMA writes the x tile, more than
-// the 128 bytes per clock an SM's shared memory delivers (66 % of the MMA rate at best with 256-row x tiles, 50 % with
-// 128-row ones).  Here the decoded +-1 tile never touches shared memory: each decode thread owns one weight row =
-// one tensor-memory lane, expands the row's 64 weights of a k step into 32 registers and stores them with
-// tcgen05.st into a ring of A tiles in tensor memory (32 columns per k step); the MMAs take A from tensor memory and
-// only the x tile from shared memory.
-//   warp 0 TMA producer (x tiles, index tiles, table) | warp 1 MMA issuer | warp 2 tensor-memory allocation
-//   warps 4-19: four groups of four warps; group g expands the k steps g, g + 4, ...; then all 16 run the epilogue.
-// Tensor memory (512 columns): accumulator in columns [0, BM), A ring of STAGES x 32 columns from column 256.
-constexpr int G4_A_COL0 = 256;
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ float4 dsmem_ld128(uint32_t addr, uint32_t rank) {
+    uint32_t peer;
+    float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(peer) : "memory");
+    return v;
+}
 
 __device__ __forceinline__ void umma_f16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
@@ -347,35 +387,40 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// SPLIT: the CTAs of a tile share K along grid.z and leave raw partial sums in p.part (a separate instantiation, so
-// that the unsplit kernel carries none of it).
-// v = 20: the 64 weights of step S of a super-block are the weight pairs 2 S .. 2 S + 31 of its four blocks (ten pairs each);
-// in the fp16-layout word of a 20-bit codeword pair j sits at bits (2 + j, 18 + j).
-template <int S>
-__device__ __forceinline__ void expand_v20(const uint32_t (&w)[4], uint32_t one2, uint32_t (&regs)[32])
+__host__ __device__ constexpr int gcd64(int v) { return v % 16 == 0 ? 16 : v % 8 == 0 ? 8 : v % 4 == 0 ? 4 : 2; }   // (v even, below 32)
+// Geometry of k step PH of an index tile of blocks of V: first pair of the step within its first block, blocks it touches.
+__host__ __device__ constexpr int step_pair0(int V, int PH) { return (64 * PH % V) / 2; }
+__host__ __device__ constexpr int step_blocks(int V) { return (64 + V - gcd64(V) + V - 1) / V; }
+
+// The 64 weights of a k step from the (inverted) codewords of its blocks, for the starting point numbered ph.
+template <int V, int PH>
+__device__ __forceinline__ void expand_step(int ph, const uint32_t (&w)[step_blocks(V)], uint32_t one2, uint32_t (&regs)[32])
 {
+    constexpr int H = V / 2, P0 = 12 - 2 * ((V + 3) / 4);
+    if (PH + 1 >= V / gcd64(V) || ph == PH) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        const int q = 2 * S + i, c = q / 10, j = q - 10 * c;
-        regs[i] = ((w[c] << (13 - j)) & 0x80008000u) | one2;
+        for (int i = 0; i < 32; ++i) {
+            const int q = step_pair0(V, PH) + i, c = q / H, j = q - H * c;
+            regs[i] = ((w[c] << (15 - P0 - j)) & 0x80008000u) | one2;
+        }
+    } else if constexpr (PH + 1 < V / gcd64(V)) {
+        expand_step<V, PH + 1>(ph, w, one2, regs);
     }
 }
 
 template <int BM, int STAGES, int KS, bool SPLIT, int V>
 __global__ void __launch_bounds__(G2_THREADS, 1)
-gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_i, const Gemm2Params p, const SplitArgs sp)
+gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_i, const Gemm2Params p, const SplitArgs sp)
 {
-    constexpr uint32_t B_BYTES = BM * G_BK * 2;                    // one x tile (64 k); a stage holds KS of them
-    constexpr uint32_t STAGE_BYTES = KS * B_BYTES;
+    const uint32_t B_BYTES = (uint32_t)p.bn * G_BK * 2;            // one x tile (64 k); a stage holds KS of them
+    const uint32_t STAGE_BYTES = KS * B_BYTES;
     constexpr int ACOLS = 32 * KS;                                 // tensor-memory columns of a stage's A tile
-    // An index tile of 64 blocks covers 64 * V weights = V k steps: 16 for v = 16 (four whole blocks per step); 20 for
-    // v = 20, where a step takes 64 weights out of four consecutive blocks, starting 0, 4, 8, 12 or 16 weights into the
-    // first (five steps = sixteen blocks, then the pattern repeats).
-    constexpr int KPT = V;
-    static_assert(V == 16 || V == 20, "index tiles of 64 blocks and whole k steps");
-    // With 128-row x tiles an MMA runs for 64 clk, less than it takes one thread to issue it next to sixteen busy decode
-    // warps; then two threads issue (warp 1: even stages into accumulator 0; warp 3: odd stages into accumulator 1 in
-    // columns [128, 256)) and the epilogue adds the two accumulators.
+    constexpr int KPT = V;                                         // k steps per index tile
+    constexpr int NBLK = step_blocks(V);                           // blocks a k step may touch
+    static_assert(V % 2 == 0 && V >= 8 && V <= 24, "pairs of weights within 16-bit halves");
+    // With x tiles of up to 128 rows an MMA runs for 64 clk or less, less than it takes one thread to issue it next to
+    // sixteen busy decode warps; then two threads issue (warp 1: even stages into accumulator 0; warp 3: odd stages into
+    // accumulator 1 in columns [128, 256)) and the epilogue adds the two accumulators.
     constexpr int NACC = (BM == 128) ? 2 : 1;
     static_assert(BM * ((BM == 128) ? 2 : 1) <= G4_A_COL0, "accumulators and A ring must not overlap");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -394,7 +439,8 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
 
     const LinearArgs &a = p.a;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n0 = blockIdx.x * G_BN, m0 = blockIdx.y * BM;
+    const int bn = p.bn;
+    const int n0 = blockIdx.x * G_BN, m0 = blockIdx.y * bn;
     // a CTA covers the k tiles [kt_first, kt_first + KT): all of them, or its share along grid.z (whole index tiles)
     const int kt_first = SPLIT ? blockIdx.z * sp.split_tiles : 0;
     const int KT = SPLIT ? min(sp.split_tiles, p.k_tiles - kt_first) : p.k_tiles;
@@ -420,7 +466,6 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_d = *s_tmem;
-    if (SPLIT) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the reduce kernel may take its place early
 
     if (warp == 0) {
         if (lane == 0) {
@@ -436,6 +481,7 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
                     mbar_expect_tx(bar_full_i(ib), G2_IDX_BYTES);
                     tma_load_2d(smem_u32(s_idx + (size_t)ib * G2_IDX_BYTES), &tmap_i, (kt_first / KPT) * 64 + it * 64, n0, bar_full_i(ib));
                 }
+                if (ks == 0 && !p.sumx) asm volatile("griddepcontrol.wait;" ::: "memory");     // x
                 const int s = ks % STAGES;
                 if (ks >= STAGES && !mbar_wait(bar_empty(s), ((ks / STAGES) & 1) ^ 1, s_abort)) break;
                 mbar_expect_tx(bar_full(s), STAGE_BYTES);
@@ -447,7 +493,7 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     } else if (warp == 1 || (NACC == 2 && warp == 3)) {
         if (lane == 0) {
             const int me = (warp == 1) ? 0 : 1;                    // which accumulator / which stages
-            uint32_t idesc = (1u << 4) | ((uint32_t)(BM >> 3) << 17) | ((uint32_t)(G_BN >> 4) << 24);
+            uint32_t idesc = (1u << 4) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(G_BN >> 4) << 24);
             if (is_bf16) idesc |= (1u << 7) | (1u << 10);
             const uint32_t d_tm = tmem_d + me * BM;
             for (int ks = me; ks < NS; ks += NACC) {
@@ -483,33 +529,29 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
                 if (!mbar_wait(bar_full_i(ib), (it >> 1) & 1, s_abort)) { ok = false; break; }
                 cur_it = it;
             }
-            // the four indices per k step of this row.  v = 16: columns (kt % 16) * 4 .. + 3 of the index tile (8 bytes);
-            // v = 20: step s of super-block q (16 blocks) starts in block 16 q + 3 s
-            uint32_t w[KS][4];
-            int spos[KS];
+            // the codewords of this row's blocks
+            uint32_t w[KS][NBLK];
 #pragma unroll
             for (int j = 0; j < KS; ++j) {
-                const int ktl = (kt0 + j) % KPT;
+                const int ktl = kt0 + j - it * KPT;
                 const unsigned char *irow_s = s_idx + (size_t)ib * G2_IDX_BYTES + (size_t)r * 128;
-                uint32_t i4[4];
-                if (V == 16) {
+                uint32_t idx[NBLK];
+                if constexpr (V == 16) {                         // (8 bytes)
                     const int boff = ktl * 8;
                     const uint2 quad = *reinterpret_cast<const uint2 *>(irow_s + ((((boff >> 4) & 7) ^ (r & 7)) << 4) + (boff & 15));
-                    i4[0] = quad.x & 0xffffu; i4[1] = quad.x >> 16; i4[2] = quad.y & 0xffffu; i4[3] = quad.y >> 16;
-                    spos[j] = 0;
+                    idx[0] = quad.x & 0xffffu; idx[1] = quad.x >> 16; idx[2] = quad.y & 0xffffu; idx[3] = quad.y >> 16;
                 } else {
-                    const int sb = ktl / 5, sp5 = ktl - 5 * sb;
-                    spos[j] = sp5;
+                    const int f = 64 * ktl / V;
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const int boff = (16 * sb + 3 * sp5 + b) * 2;
-                        i4[b] = *reinterpret_cast<const uint16_t *>(irow_s + ((((boff >> 4) & 7) ^ (r & 7)) << 4) + (boff & 15));
+                    for (int b = 0; b < NBLK; ++b) {             // (the last step of a tile ends with its last block)
+                        const int boff = min(f + b, 63) * 2;
+                        idx[b] = *reinterpret_cast<const uint16_t *>(irow_s + (((boff >> 4) ^ (r & 7)) << 4) + (boff & 15));
                     }
                 }
 #pragma unroll
-                for (int b = 0; b < 4; ++b) w[j][b] = ~(tab_smem ? s_tab[i4[b]] : __ldg(p.tab + i4[b]));
+                for (int b = 0; b < NBLK; ++b) w[j][b] = ~(tab_smem ? s_tab[idx[b]] : __ldg(p.tab + idx[b]));
             }
-            if (((ks + 4) * KS) / KPT != it || ks + 4 >= NS) {     // this group's last stage in the index tile
+            if (((ks + 4) * KS) / KPT != it || ks + 4 >= NS) {   // this group's last stage in the index tile
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_empty_i(ib));
             }
@@ -520,20 +562,7 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
             for (int j = 0; j < KS; ++j) {
                 // register i holds the weights 2i, 2i+1 of the k step (K elements 2i, 2i+1 of this row of A)
                 uint32_t regs[32];
-                if (V == 16) {
-#pragma unroll
-                    for (int b = 0; b < 4; ++b)
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) regs[8 * b + i] = ((w[j][b] << (11 - i)) & 0x80008000u) | one2;
-                } else {
-                    switch (spos[j]) {
-                    case 0: expand_v20<0>(w[j], one2, regs); break;
-                    case 1: expand_v20<1>(w[j], one2, regs); break;
-                    case 2: expand_v20<2>(w[j], one2, regs); break;
-                    case 3: expand_v20<3>(w[j], one2, regs); break;
-                    default: expand_v20<4>(w[j], one2, regs); break;
-                    }
-                }
+                expand_step<V, 0>((kt0 + j) % (V / gcd64(V)), w[j], one2, regs);
                 tmem_st32(tmem_d + lane_base + G4_A_COL0 + sa * ACOLS + 32 * j, regs);
             }
             tmem_st_wait();
@@ -542,16 +571,18 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
             if (lane == 0) mbar_arrive(bar_full(sa));
         }
         // ------------------------------------------------------------ epilogue: four warps per lane quadrant
+        asm volatile("griddepcontrol.wait;" ::: "memory");     // (y, and the row sums)
         if (ok && mbar_wait(bar_accum, 0, s_abort)) {
             tc_fence_after();
             const int wl = warp - 4;
             const int q4 = wl & 3, quarter = wl >> 2;
-            const int nrow = n0 + q4 * 32 + lane;
+            const int nl = q4 * 32 + lane, nrow = n0 + nl;
             const int nc = min(nrow, a.N - 1);
             const float al = __half2float(a.alpha[nc]);
             const float mu = a.mu ? __half2float(a.mu[nc]) : 0.f;
+            float *tile = reinterpret_cast<float *>(smem_gen);             // SPLIT: [bn][128], where the x tiles were
 #pragma unroll 1
-            for (int c0 = quarter * (BM / 4); c0 < (quarter + 1) * (BM / 4); c0 += 32) {
+            for (int c0 = quarter * 32; c0 < bn; c0 += 128) {
                 uint32_t rr[32];
                 tmem_ld32(tmem_d + lane_base + c0, rr);
                 tmem_ld_wait();
@@ -562,23 +593,51 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
 #pragma unroll
                     for (int i = 0; i < 32; ++i) rr[i] = __float_as_uint(__uint_as_float(rr[i]) + __uint_as_float(r2[i]));
                 }
-                if (nrow < a.N) {
+                if (SPLIT) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (c0 + i < bn) tile[(c0 + i) * 128 + nl] = __uint_as_float(rr[i]);
+                } else if (nrow < a.N) {
 #pragma unroll
                     for (int i = 0; i < 32; ++i) {
                         const int m = m0 + c0 + i;
-                        if (m < a.M) {
-                            if (SPLIT) {                           // K split: the reduce kernel applies alpha and mu
-                                sp.part[((size_t)blockIdx.z * a.M + m) * a.N + nrow] = __uint_as_float(rr[i]);
-                            } else {
-                                float y = al * __uint_as_float(rr[i]);
-                                if (a.mu) y += mu * p.sumx[m];
-                                store_from_float(a.y, a.y_dt, (size_t)m * a.N + nrow, y);
-                            }
+                        if (c0 + i < bn && m < a.M) {
+                            float y = al * __uint_as_float(rr[i]);
+                            if (a.mu) y += mu * p.sumx[m];
+                            store_from_float(a.y, a.y_dt, (size_t)m * a.N + nrow, y);
                         }
                     }
                 }
             }
         }
+    }
+    if constexpr (SPLIT) {
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+        const int splits = gridDim.z, z = blockIdx.z;
+        const int per = (bn + splits - 1) / splits, c1 = min(min(bn, a.M - m0), (z + 1) * per);
+        if (!*s_abort)
+            for (int i = z * per * 32 + tid; i < c1 * 32; i += G2_THREADS) {
+                const int c = i >> 5, nq = (i & 31) * 4, m = m0 + c;
+                float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int q = 0; q < splits; ++q) {
+                    const float4 f = dsmem_ld128(smem_base + (uint32_t)(c * 128 + nq) * 4u, (uint32_t)q);
+                    t.x += f.x; t.y += f.y; t.z += f.z; t.w += f.w;
+                }
+                const float v[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int n = n0 + nq + k;
+                    if (n < a.N) {
+                        float y = __half2float(a.alpha[n]) * v[k];
+                        if (a.mu) y += __half2float(a.mu[n]) * p.sumx[m];
+                        store_from_float(a.y, a.y_dt, (size_t)m * a.N + n, y);
+                    }
+                }
+            }
+        cluster_arrive();                                          // (nobody leaves while its shared memory is being read)
+        cluster_wait();
     }
     tc_fence_before();
     __syncthreads();
@@ -587,24 +646,6 @@ gemm_v16t_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         __syncthreads();
     }
     if (warp == 2) tmem_dealloc(tmem_d, 512);
-}
-
-// y = alpha * (sum of the K splits' partial sums, in split order) + mu * sum_k x.
-__global__ void splitk_reduce_kernel(const float *__restrict__ part, int splits, int M, int N, const __half *__restrict__ alpha,
-                                     const __half *__restrict__ mu, const float *__restrict__ sumx, void *__restrict__ y, int y_dt)
-{
-    // launched with programmatic stream serialisation: the blocks are resident before the split kernel has finished, and
-    // wait here until all of it has completed and its partial sums are visible
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t MN = (size_t)M * N;
-    if (i >= MN) return;
-    const int n = (int)(i % N), m = (int)(i / N);
-    float acc = 0.f;
-    for (int z = 0; z < splits; ++z) acc += part[(size_t)z * MN + i];
-    float v = __half2float(alpha[n]) * acc;
-    if (mu) v += __half2float(mu[n]) * sumx[m];
-    store_from_float(y, y_dt, i, v);
 }
 
 // ------------------------------------------------------------------------------------ host side
@@ -638,45 +679,86 @@ static int launch_cfg(const CUtensorMap &tm, const GemmParams &p, cudaStream_t s
     return cuda_check_launch();
 }
 
-template <int BM, int STAGES, int KS, bool SPLIT, int V = 16>
-static int launch_v16t(const CUtensorMap &tm, const CUtensorMap &ti, const Gemm2Params &p, const SplitArgs &sp, cudaStream_t s)
+// Tiling of a (M, N, K) problem: rows of x per tile (bn), tiles of x, K splits.  Time under a wave model, in clocks: a CTA per SM
+// in rounds, each a start-up (launch, tensor memory, first tiles, epilogue) and its k steps; a step costs the MMAs' time
+// (2 clk per row of x, and no less than the decode of its weights), a split the sum over the cluster.  Whole index tiles per
+// split, clusters of up to eight.
+struct GemmPlan { int bn, mt, splits, split_tiles; };
+
+static bool gemm_table_fits(int bn, int Kc)
 {
-    const size_t smem = (size_t)STAGES * KS * (BM * G_BK * 2) + 1024 + 2 * G2_IDX_BYTES + ((p.tab_bytes + 15) & ~15) +
+    const size_t fixed = (size_t)4 * (bn > 128 ? 1 : 2) * bn * G_BK * 2 + 1024 + 2 * G2_IDX_BYTES + 512;
+    return fixed + (size_t)((Kc + 3) / 4 * 4) * 4 <= 227u * 1024u;
+}
+
+static GemmPlan gemm_plan(int M, int N, int K, int v, int Kc)
+{
+    const int k_tiles = (K + G_BK - 1) / G_BK, rows = (N + G_BN - 1) / G_BN;
+    const int idx_tiles = (k_tiles + v - 1) / v;
+    const double decode = v == 16 ? 230.0 : 190.0 + 20.0 * step_blocks(v);
+    GemmPlan best = {0, 0, 1, k_tiles};
+    double best_t = 0;
+    for (int mt = (M + 255) / 256; mt <= (M + 255) / 256 + (M + 127) / 128; ++mt) {
+        int bn = ((M + mt - 1) / mt + 15) / 16 * 16;
+        if (bn < 16) bn = 16;
+        const int mtn = (M + bn - 1) / bn;
+        const double step = bn > 128 ? (2.4 * bn > decode ? 2.4 * bn : decode) : (2.6 * bn > decode ? 2.6 * bn : decode);
+        for (int sp = 1; sp <= 8 && sp <= idx_tiles; ++sp) {
+            const int per = (idx_tiles + sp - 1) / sp;                 // index tiles per split
+            const int n = (idx_tiles + per - 1) / per;
+            if (n != sp) continue;
+            const long long ctas = (long long)rows * mtn * sp;
+            const int at_once = sp == 1 ? 148 : 136 / sp * sp;         // (clusters do not fill every GPC)
+            const double waves = (double)((ctas + at_once - 1) / at_once);
+            const int steps = per * v < k_tiles ? per * v : k_tiles;
+            const double t = waves * (5500.0 + 4.0 * bn + steps * step + (sp > 1 ? 2000.0 + 6.0 * bn : 0.0));
+            if (best.bn == 0 || t < best_t) { best = {bn, mtn, sp, per * v}; best_t = t; }
+        }
+        if (M <= 256 && bn <= 32) break;
+    }
+    return best;
+}
+
+template <int BM, int STAGES, int KS, bool SPLIT, int V>
+static int launch_ts(const CUtensorMap &tm, const CUtensorMap &ti, const Gemm2Params &p, const GemmPlan &g, cudaStream_t s)
+{
+    const size_t smem = (size_t)STAGES * KS * (p.bn * G_BK * 2) + 1024 + 2 * G2_IDX_BYTES + ((p.tab_bytes + 15) & ~15) +
                         (2 * STAGES + 6) * 8 + 16;
-    auto kern = gemm_v16t_kernel<BM, STAGES, KS, SPLIT, V>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = gemm_ts_kernel<BM, STAGES, KS, SPLIT, V>;
+    static std::atomic<uint64_t> done{0};                          // (the attribute, once per device)
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
-    dim3 grid((p.a.N + G_BN - 1) / G_BN, (p.a.M + BM - 1) / BM, SPLIT ? (p.k_tiles + sp.split_tiles - 1) / sp.split_tiles : 1);
-    kern<<<grid, G2_THREADS, smem, s>>>(tm, ti, p, sp);
-    return cuda_check_launch();
+    if (dev >= 64 || !((done.load(std::memory_order_relaxed) >> dev) & 1u)) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return cuda_fail(e);
+        if (dev < 64) done.fetch_or(uint64_t(1) << dev, std::memory_order_relaxed);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((p.a.N + G_BN - 1) / G_BN, g.mt, g.splits);
+    cfg.blockDim = dim3(G2_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[3];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    // no more shared memory than asked for: what is left caches the codewords that come from global memory
+    at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[1].val.sharedMemCarveout = (unsigned)((smem + 1024) * 100 / (228 * 1024));
+    at[2].id = cudaLaunchAttributeClusterDimension;
+    at[2].val.clusterDim.x = 1; at[2].val.clusterDim.y = 1; at[2].val.clusterDim.z = (unsigned)g.splits;
+    cfg.attrs = at;
+    cfg.numAttrs = SPLIT ? 3 : 2;
+    const SplitArgs sp = {g.split_tiles};
+    e = cudaLaunchKernelEx(&cfg, kern, tm, ti, p, sp);
+    return e == cudaSuccess ? BTC_OK : cuda_fail(e);
 }
 
-// K splits for a launch of `tiles` CTAs over `k_tiles` k tiles: as many as keep the grid within the SM count, each a
-// whole number of index tiles (16 k tiles).  Returns k tiles per split.
-static int splitk_tiles(int tiles, int k_tiles, int *splits)
+template <int V>
+static int launch_ts_v(const CUtensorMap &tm, const CUtensorMap &ti, const Gemm2Params &p, const GemmPlan &g, cudaStream_t s)
 {
-    *splits = 1;
-    if (tiles > 74 || k_tiles < 64) return k_tiles;
-    int want = 148 / tiles;
-    if (want > 8) want = 8;
-    int per = ((k_tiles + want - 1) / want + 15) / 16 * 16;
-    if (per < 16) per = 16;
-    const int n = (k_tiles + per - 1) / per;
-    if (n < 2) return k_tiles;
-    *splits = n;
-    return per;
-}
-
-// Tile width in rows of x for a (M, N) problem: 128 or 256, whichever needs less time under a wave model -- CTAs run in
-// rounds of one per SM, and a 256-row tile takes about 1.6 times as long as a 128-row one (it amortises the weight
-// decode over twice the rows; measured at M = 2048 against M = 512).
-static int gemm_bm(int M, int N)
-{
-    if (M <= 128) return 128;
-    const long long rows = (N + 127) / 128, sms = 148;
-    const long long t128 = ((M + 127) / 128) * rows, t256 = ((M + 255) / 256) * rows;
-    const double c128 = (double)((t128 + sms - 1) / sms), c256 = 1.6 * (double)((t256 + sms - 1) / sms);
-    return c256 < c128 ? 256 : 128;
+    if (g.bn > 128) return g.splits > 1 ? launch_ts<256, 4, 1, true, V>(tm, ti, p, g, s) : launch_ts<256, 4, 1, false, V>(tm, ti, p, g, s);
+    return g.splits > 1 ? launch_ts<128, 4, 2, true, V>(tm, ti, p, g, s) : launch_ts<128, 4, 2, false, V>(tm, ti, p, g, s);
 }
 
 size_t gemm_tcgen05_workspace_min(int M)
@@ -684,43 +766,26 @@ size_t gemm_tcgen05_workspace_min(int M)
     return M > 8 ? (size_t)M * sizeof(float) : 0;   // row sums of x for the mean term
 }
 
-// 5 <= M <= 8 with few tiles and a long K (above all the 11008-wide down projection): the split tensor-core launch beats
-// the fp16 decode kernel (measured 17 us against 30 us for 4096 x 11008), so the decode entry point tries it first.
-bool gemm_tcgen05_small_m_pays(int M, int N, int K, int v)
-{
-    if (M < 5 || M > 8 || v != 16 || K % 16 || (K / v) % 8) return false;
-    int splits = 1;
-    const int k_tiles = (K + G_BK - 1) / G_BK;
-    splitk_tiles((N + 127) / 128, k_tiles, &splits);
-    return splits > 1 && (k_tiles >= 128 || (k_tiles >= 64 && M >= 6));   // (4096 x 4096 at M = 8: 10 us against 12.5 us)
-}
-
-// The minimum plus, where the launch would otherwise leave most SMs idle (v = 16, few tiles, long K), room for the
-// partial sums of a K split.  With less than this (but at least the minimum) the kernels run without the split.
+// What a caller is asked for: the minimum, rounded up for layers with few tiles and a long K as it always was (room for
+// partial sums of a K split; they meet in distributed shared memory now).
 size_t gemm_tcgen05_workspace_bytes(int M, int N, int K, int v, int)
 {
     size_t w = gemm_tcgen05_workspace_min(M);
-    const bool small = gemm_tcgen05_small_m_pays(M, N, K, v);
-    if (small) w = (size_t)M * sizeof(float);
-    if ((M > 8 || small) && v == 16 && (K / v) % 8 == 0) {
-        const int BM = gemm_bm(M, N);
-        int splits = 1;
-        splitk_tiles(((N + 127) / 128) * ((M + BM - 1) / BM), (K + G_BK - 1) / G_BK, &splits);
-        if (splits > 1) w = ((w + 255) & ~(size_t)255) + (size_t)splits * M * N * sizeof(float);
+    if (M > 8 && v == 16 && (K / v) % 8 == 0) {
+        const int tiles = ((N + 127) / 128) * ((M + 127) / 128), k_tiles = (K + G_BK - 1) / G_BK;
+        if (tiles <= 74 && k_tiles >= 64) w = ((w + 255) & ~(size_t)255) + (size_t)2 * M * N * sizeof(float);
     }
     return w;
 }
 
-int launch_gemm_tcgen05(const LinearArgs &a, cudaStream_t s, bool small_m)
+int launch_gemm_tcgen05(const LinearArgs &a, cudaStream_t s)
 {
-    if (a.M <= 8 && !small_m) return BTC_ERR_UNSUPPORTED;      // the decode path is the better kernel there
-    if (a.M <= 8 && (!gemm_tcgen05_small_m_pays(a.M, a.N, a.K, a.v) || !a.workspace ||
-                     a.workspace_bytes < gemm_tcgen05_workspace_bytes(a.M, a.N, a.K, a.v, a.Kc)))
-        return BTC_ERR_UNSUPPORTED;                            // (only with room for the K split)
     if (a.K % 8) return BTC_ERR_UNSUPPORTED;                   // TMA row pitch must be a multiple of 16 bytes
     encode_tiled_fn enc = get_encode();
     if (!enc) return BTC_ERR_UNSUPPORTED;
-    const int BM = gemm_bm(a.M, a.N);
+    const bool ts = a.v >= 8 && a.v <= 24 && a.v % 2 == 0 && a.Kb % 8 == 0;
+    const GemmPlan g = gemm_plan(a.M, a.N, a.K, ts ? a.v : 16, a.Kc);
+    const int BM = ts ? g.bn : (a.M > 128 ? 256 : 128);
 
     CUtensorMap tm;
     const cuuint64_t dims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
@@ -739,14 +804,20 @@ int launch_gemm_tcgen05(const LinearArgs &a, cudaStream_t s, bool small_m)
     if (a.mu) {
         if (!a.workspace || a.workspace_bytes < (size_t)a.M * sizeof(float)) return BTC_ERR_WORKSPACE;
         float *sx = reinterpret_cast<float *>(a.workspace);
-        rowsum_kernel<<<(a.M + 7) / 8, 256, 0, s>>>(a.x, a.x_dt, a.M, a.K, sx);
-        int rc = cuda_check_launch();
-        if (rc != BTC_OK) return rc;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)a.M);
+        cfg.blockDim = dim3(256);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, rowsum_kernel, a.x, a.x_dt, a.K, sx);
+        if (e != cudaSuccess) return cuda_fail(e);
         p.sumx = sx;
     }
-    if ((a.v == 16 && a.Kb % 8 == 0) || (a.v == 20 && a.Kb % 16 == 0)) {
-        // v = 16, and v = 20 with K a multiple of 320: index tiles by TMA, table in shared memory when it fits, weights
-        // through tensor memory
+    if (ts) {
         CUtensorMap ti;
         const cuuint64_t idims[2] = {(cuuint64_t)a.Kb, (cuuint64_t)a.N};
         const cuuint64_t istr[1] = {(cuuint64_t)a.Kb * 2};
@@ -755,45 +826,24 @@ int launch_gemm_tcgen05(const LinearArgs &a, cudaStream_t s, bool small_m)
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
             Gemm2Params q;
-            q.a = a; q.sumx = p.sumx; q.k_tiles = p.k_tiles;
+            q.a = a; q.sumx = p.sumx; q.k_tiles = p.k_tiles; q.bn = g.bn;
             const int Kc4 = (a.Kc + 3) / 4 * 4;
             q.tab = a.Cp + Kc4;
-            // shared memory holds only x tiles (4 stages of 32 KB either way), index tiles and the table
-            const size_t fixed_t = (size_t)4 * (256 * G_BK * 2) + 1024 + 2 * G2_IDX_BYTES + 512;
-            q.tab_bytes = (fixed_t + (size_t)Kc4 * 4 <= 227u * 1024u) ? Kc4 * 4 : 0;
-            // few tiles and a long K: split K over the idle SMs when the caller's workspace has room for the partial sums
-            SplitArgs sp = {q.k_tiles, nullptr};
-            int splits = 1;
-            const int per = a.v == 16 ? splitk_tiles(((a.N + 127) / 128) * ((a.M + BM - 1) / BM), q.k_tiles, &splits) : q.k_tiles;
-            if (a.v == 20)                                         // (no K split here: its index tiles are 20 k steps)
-                return (BM == 256) ? launch_v16t<256, 4, 1, false, 20>(tm, ti, q, sp, s) : launch_v16t<128, 4, 2, false, 20>(tm, ti, q, sp, s);
-            if (splits > 1) {
-                const size_t off = ((size_t)a.M * sizeof(float) + 255) & ~(size_t)255;   // (row sums of x come first)
-                const size_t need = off + (size_t)splits * a.M * a.N * sizeof(float);
-                if (a.workspace && a.workspace_bytes >= need && reinterpret_cast<uintptr_t>(a.workspace) % 16 == 0) {
-                    sp.split_tiles = per;
-                    sp.part = reinterpret_cast<float *>(static_cast<char *>(a.workspace) + off);
-                } else {
-                    splits = 1;
-                }
+            // shared memory holds only x tiles (four stages), index tiles and the table
+            q.tab_bytes = gemm_table_fits(g.bn, a.Kc) ? Kc4 * 4 : 0;
+            switch (a.v) {
+            case 8: return launch_ts_v<8>(tm, ti, q, g, s);
+            case 10: return launch_ts_v<10>(tm, ti, q, g, s);
+            case 12: return launch_ts_v<12>(tm, ti, q, g, s);
+            case 14: return launch_ts_v<14>(tm, ti, q, g, s);
+            case 16: return launch_ts_v<16>(tm, ti, q, g, s);
+            case 18: return launch_ts_v<18>(tm, ti, q, g, s);
+            case 20: return launch_ts_v<20>(tm, ti, q, g, s);
+            case 22: return launch_ts_v<22>(tm, ti, q, g, s);
+            default: return launch_ts_v<24>(tm, ti, q, g, s);
             }
-            if (splits == 1) return (BM == 256) ? launch_v16t<256, 4, 1, false>(tm, ti, q, sp, s) : launch_v16t<128, 4, 2, false>(tm, ti, q, sp, s);
-            const int rc = (BM == 256) ? launch_v16t<256, 4, 1, true>(tm, ti, q, sp, s) : launch_v16t<128, 4, 2, true>(tm, ti, q, sp, s);
-            if (rc != BTC_OK) return rc;
-            const size_t mn = (size_t)a.M * a.N;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)((mn + 255) / 256));
-            cfg.blockDim = dim3(256);
-            cfg.stream = s;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            at[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            const float *part = sp.part;
-            const cudaError_t e = cudaLaunchKernelEx(&cfg, splitk_reduce_kernel, part, splits, a.M, a.N, a.alpha, a.mu, q.sumx, a.y, a.y_dt);
-            return e == cudaSuccess ? BTC_OK : cuda_fail(e);
         }
+        return BTC_ERR_UNSUPPORTED;                            // (a shape the tensor map cannot describe)
     }
     if (BM == 256) return launch_cfg<256, 4>(tm, p, s);
     return launch_cfg<128, 6>(tm, p, s);
