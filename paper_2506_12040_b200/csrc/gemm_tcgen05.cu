@@ -679,10 +679,12 @@ static int launch_cfg(const CUtensorMap &tm, const GemmParams &p, cudaStream_t s
     return cuda_check_launch();
 }
 
-// Tiling of a (M, N, K) problem: rows of x per tile (bn), tiles of x, K splits.  Time under a wave model, in clocks: a CTA per SM
-// in rounds, each a start-up (launch, tensor memory, first tiles, epilogue) and its k steps; a step costs the MMAs' time
-// (2 clk per row of x, and no less than the decode of its weights), a split the sum over the cluster.  Whole index tiles per
-// split, clusters of up to eight.
+// Tiling of a (M, N, K) problem: rows of x per tile (bn), tiles of x, K splits (whole index tiles, clusters of up to eight).
+// Time under a wave model, in clocks, fitted to measurements: a CTA per SM in rounds (the last one shorter when it is not
+// full: less traffic, higher clocks), each a start-up (launch, tensor memory, first tiles, epilogue) and its k steps.  A step
+// costs the MMAs' and the x tile's time, 260 + 1.55 clk per row of x, and no less than the decode of its weights: 350
+// clk for v = 16, about 33 more per block a step touches otherwise.  Codewords gathered from L1 / L2 (table too large for
+// shared memory) share that path with the x tiles: 650 clk + 1 per row.  A split adds the sum over the cluster.
 struct GemmPlan { int bn, mt, splits, split_tiles; };
 
 static bool gemm_table_fits(int bn, int Kc)
@@ -695,23 +697,25 @@ static GemmPlan gemm_plan(int M, int N, int K, int v, int Kc)
 {
     const int k_tiles = (K + G_BK - 1) / G_BK, rows = (N + G_BN - 1) / G_BN;
     const int idx_tiles = (k_tiles + v - 1) / v;
-    const double decode = v == 16 ? 230.0 : 190.0 + 20.0 * step_blocks(v);
+    const double decode = v == 16 ? 350.0 : v == 8 ? 410.0 : 300.0 + 33.0 * step_blocks(v);
     GemmPlan best = {0, 0, 1, k_tiles};
     double best_t = 0;
     for (int mt = (M + 255) / 256; mt <= (M + 255) / 256 + (M + 127) / 128; ++mt) {
         int bn = ((M + mt - 1) / mt + 15) / 16 * 16;
         if (bn < 16) bn = 16;
         const int mtn = (M + bn - 1) / bn;
-        const double step = bn > 128 ? (2.4 * bn > decode ? 2.4 * bn : decode) : (2.6 * bn > decode ? 2.6 * bn : decode);
+        const double mma = 260.0 + 1.55 * bn, fit = mma > decode ? mma : decode;
+        const double step = gemm_table_fits(bn, Kc) ? fit : 650.0 + bn > fit ? 650.0 + bn : fit;
         for (int sp = 1; sp <= 8 && sp <= idx_tiles; ++sp) {
             const int per = (idx_tiles + sp - 1) / sp;                 // index tiles per split
             const int n = (idx_tiles + per - 1) / per;
             if (n != sp) continue;
             const long long ctas = (long long)rows * mtn * sp;
             const int at_once = sp == 1 ? 148 : 136 / sp * sp;         // (clusters do not fill every GPC)
-            const double waves = (double)((ctas + at_once - 1) / at_once);
+            const int rest = (int)(ctas % at_once);
+            const double waves = (double)(ctas / at_once) + (rest ? (ctas < at_once ? 1.0 : 0.45 + 0.55 * rest / at_once) : 0.0);
             const int steps = per * v < k_tiles ? per * v : k_tiles;
-            const double t = waves * (5500.0 + 4.0 * bn + steps * step + (sp > 1 ? 2000.0 + 6.0 * bn : 0.0));
+            const double t = waves * (5500.0 + 4.0 * bn + steps * step + (sp > 1 ? 3500.0 + 20.0 * bn : 0.0));
             if (best.bn == 0 || t < best_t) { best = {bn, mtn, sp, per * v}; best_t = t; }
         }
         if (M <= 256 && bn <= 32) break;

@@ -190,6 +190,27 @@ def test_gemm_parity_small(N, K, v, Kc, M, xdt, mu):
     assert rel <= TOL_GEMM and fwd <= TOL_GEMM, (rel, fwd)
 
 
+@pytest.mark.parametrize("N,K,v,Kc,M,xdt,mu,odt", [
+    # widths of x tiles at their edges, K ending inside an index tile, row tiles ragged; the table in shared memory or not
+    (130, 8 * 9 * 8, 8, 85, 9, "f16", True, torch.float32),
+    (129, 10 * 72, 10, 700, 128, "bf16", False, torch.float16),
+    (300, 12 * 200, 12, 2353, 129, "f16", True, torch.bfloat16),
+    (1, 14 * 64, 14, 9000, 256, "bf16", True, torch.float32),
+    (257, 18 * 136, 18, 21619, 257, "f16", False, torch.float32),
+    (128, 20 * 8, 20, 65536, 31, "bf16", True, torch.float16),
+    (384, 22 * 96, 22, 900, 300, "f16", True, torch.float32),
+    (200, 24 * 328, 24, 5000, 17, "bf16", False, torch.float32),
+    (4000, 16 * 688, 16, 65536, 260, "bf16", True, torch.float32),
+])
+def test_gemm_edges(N, K, v, Kc, M, xdt, mu, odt):
+    L = wl.make_layer(_spec(N, K, v, Kc, x_dtype=xdt, with_mu=mu), M, seed=N + K + M)
+    y, d = run_layer(L, "gemm", out_dtype=odt)
+    tol = TOL_GEMM if odt == torch.float32 else TOL_GEMM + 2.0 ** (-8 if odt == torch.bfloat16 else -11)
+    rel, fwd = errors(y.float(), oracle_y(L), L)
+    assert rel <= tol and fwd <= tol, (rel, fwd)
+    assert btc.device_status() == 0
+
+
 def test_gemm_parity_benchmark_config_M512_every_output():
     """Config 4 at M = 512 in the launch configuration the bench times: the three full-size layers, every one of the
     M x N outputs against the full fp64 product (seconds per shape on the host cores)."""
