@@ -63,14 +63,15 @@ static bool covered(const LinearArgs &a)
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-static Layout layout(bool half, int ncls, int rows, int ib, int nw, int tab_bytes, int stages)
+static Layout layout(bool half, int ncls, int rows, int ib, int nw, int entries, int tab_bytes, int stages)
 {
     Layout L;
+    L.chunk = entries / nw;
     L.stages = stages;
     L.stage_bytes = nw * 16 * (4 * lane_blocks(half, ncls)) * (ib ? ib : 16) / 8;    // (slices x rows per stage is 16 nw, however many slices)
     int o = round_up(stages * L.stage_bytes + (ib ? 16 : 0), 128);   // (a lane's last word of dense fields may lie just past its row)
     L.tab = o; o += round_up(tab_bytes, 16);
-    L.park = o; o += half ? park_bytes<true>() : park_bytes<false>();
+    L.park = o; o += entries * entry_floats(half) * 4;
     L.stage_x_pitch = stage_x_bytes(half, ncls, rows);
     L.stage_x = o; o += (half ? MAX_SLICES : nw) * L.stage_x_pitch;
     L.misc = round_up(o, 16);
@@ -143,53 +144,73 @@ static bool tensor_map(const MapKey &k, int box_words, CUtensorMap *out)
     return true;
 }
 
-// Gives every layer a whole number of CTAs so that the largest load of any CTA -- ceil(groups / CTAs) row groups times the
-// layer's cost, plus its set-up cost -- is as small as the budget allows (bisection), and returns the grid size.
-static int assign_ctas(Batch &b, int budget)
+// Sets how a layer's passes are shared in clusters of `cluster` CTAs, and its costs in sixteenths of a (stage, pass): a
+// pass's fragments cost about as much as one and a half of those, a sum over the cluster about one.
+static void set_split(Problem &p, bool half, int cluster)
+{
+    p.kw = cluster > 1 && p.parts >= cluster ? cluster : 1;
+    const int passes = (p.parts + p.kw - 1) / p.kw;
+    p.cost = passes * 16;
+    p.fixed = passes * 24 * (half ? 1 : p.M) + (p.kw > 1 ? 16 : 0);
+}
+
+// Gives every layer a whole number of clusters so that the largest load of any CTA -- ceil(groups / workers) stages' worth of
+// rows times the layer's cost, plus its set-up cost -- is as small as the budget of clusters allows (bisection).  Returns
+// that load; *grid: CTAs in all.
+static long long assign_ctas(Batch &b, int budget, int cluster, int *grid)
 {
     auto per_cta = [&](int i, long long T) { return (T - b.p[i].fixed) / b.p[i].cost; };
+    auto workers = [&](int i) { return b.p[i].kw > 1 ? 1 : cluster; };      // per cluster
+    auto clusters = [&](int i, long long per) {
+        const long long n = (b.p[i].groups + per - 1) / per;
+        const int w = workers(i);
+        return w > 1 ? (n + w - 1) / w : n;
+    };
     auto needed = [&](long long T) {
         long long sum = 0;
         for (int i = 0; i < b.count; ++i) {
             const long long per = per_cta(i, T);
             if (per < 1) return (long long)1 << 40;
-            sum += (b.p[i].groups + per - 1) / per;
+            sum += clusters(i, per);
         }
         return sum;
     };
-    long long lo = 1, hi = 0;
+    long long lo = 0, hi = 0;                            // (in eighths: every cost is a multiple of 8)
     for (int i = 0; i < b.count; ++i) {
         const long long all = (long long)b.p[i].groups * b.p[i].cost + b.p[i].fixed;
-        if (all > hi) hi = all;                          // one CTA per layer always fits (budget >= count)
+        lo += (long long)b.p[i].groups * b.p[i].cost / workers(i);
+        if (all > hi) hi = all;                          // one cluster per layer always fits (budget >= count)
     }
+    lo = lo / budget / 8;                                // no distribution beats the average
+    hi = (hi + 7) / 8;
     while (lo < hi) {
         const long long mid = (lo + hi) / 2;
-        if (needed(mid) <= budget) hi = mid; else lo = mid + 1;
+        if (needed(8 * mid) <= budget) hi = mid; else lo = mid + 1;
     }
-    int sum = 0;
-    for (int i = 0; i < b.count; ++i) {
-        const long long per = per_cta(i, lo);
-        b.p[i].cta_count = (int)((b.p[i].groups + per - 1) / per);
-        sum += b.p[i].cta_count;
-    }
-    while (sum < budget) {                               // spare CTAs go where the average load is highest
+    lo *= 8;
+    int count[IM_MAXP], sum = 0;
+    for (int i = 0; i < b.count; ++i) { count[i] = (int)clusters(i, per_cta(i, lo)); sum += count[i]; }
+    while (sum < budget) {                               // spare clusters go where the average load is highest
         int best = -1;
         double most = 0;
         for (int i = 0; i < b.count; ++i) {
-            const double load = (double)b.p[i].groups * b.p[i].cost / b.p[i].cta_count + b.p[i].fixed;
-            if (b.p[i].cta_count < b.p[i].groups && (best < 0 || load > most)) { best = i; most = load; }
+            const double load = (double)b.p[i].groups * b.p[i].cost / (count[i] * workers(i)) + b.p[i].fixed;
+            if (count[i] * workers(i) < b.p[i].groups && (best < 0 || load > most)) { best = i; most = load; }
         }
         if (best < 0) break;
-        ++b.p[best].cta_count; ++sum;
+        ++count[best]; ++sum;
     }
     int begin = 0;
     for (int i = 0; i < b.count; ++i) {
+        const int w = count[i] * workers(i);
         b.p[i].cta_begin = begin;
+        b.p[i].cta_count = count[i] * cluster;
         begin += b.p[i].cta_count;
-        b.p[i].per = b.p[i].groups / b.p[i].cta_count;
-        b.p[i].rem = b.p[i].groups % b.p[i].cta_count;
+        b.p[i].per = b.p[i].groups / w;
+        b.p[i].rem = b.p[i].groups % w;
     }
-    return begin;
+    *grid = begin;
+    return lo;
 }
 
 // One launch over layers of one form, class count and index format.
@@ -212,23 +233,27 @@ static int launch_group(const LinearArgs *const *args, int count, cudaStream_t s
     // Table: 16-bit halves in the integer form up to v = 16 (half the shared memory and half the bytes that every CTA loads; 65536
     // codewords take 128 KB), else 32-bit words; two CTAs per SM where that leaves room for them (integer form), else one; else as
     // much of the words as fits (frequency-ordered codebooks: the head serves most lookups).
+    int entries = max_park_entries(s0.half);
     constexpr int half_sm = 113 * 1024, whole_sm = 227 * 1024;
-    auto fits = [&](int nw, int tab, int stages) { return layout(s0.half, s0.ncls, m_even, ib, nw, tab, stages).total <= (nw == 8 ? half_sm : whole_sm); };
+    auto fits = [&](int nw, int tab, int stages) { return layout(s0.half, s0.ncls, m_even, ib, nw, entries, tab, stages).total <= (nw == 8 ? half_sm : whole_sm); };
     int nw = s0.half ? 16 : 8, tab = !s0.half && s0.ncls <= 4 ? TAB_HALVES : TAB_WORDS, tab_bytes = tab == TAB_HALVES ? halves : words;
+    // fp16 form: as few meetings of the warps as four index stages leave room for
+    while (s0.half && entries > 64 && !fits(nw, tab_bytes, 4)) entries -= 16;
     if (!fits(nw, tab_bytes, 3)) {
         if (ib) return BTC_ERR_UNSUPPORTED;
         nw = 16;
         if (!fits(16, tab_bytes, 2)) {
             tab = TAB_HEAD;
-            tab_bytes = (whole_sm - layout(s0.half, s0.ncls, m_even, ib, nw, 0, 3).total - 128) / 128 * 128;
+            tab_bytes = (whole_sm - layout(s0.half, s0.ncls, m_even, ib, nw, entries, 0, 3).total - 128) / 128 * 128;
         }
     }
     b.tab_head = tab_bytes / 4;
     int stages = 2;
     while (stages < MAX_STAGES && fits(nw, tab_bytes, stages + 1)) ++stages;
-    b.L = layout(s0.half, s0.ncls, m_even, ib, nw, tab_bytes, stages);
+    b.L = layout(s0.half, s0.ncls, m_even, ib, nw, entries, tab_bytes, stages);
 
     long long work = 0, groups = 0;
+    int max_parts = 1;
     for (int i = 0; i < count; ++i) {
         const LinearArgs &a = *args[i];
         const Shape sh = shape_of(a);
@@ -247,16 +272,37 @@ static int launch_group(const LinearArgs *const *args, int count, cudaStream_t s
         p.x_dt = a.x_dt; p.y_dt = a.y_dt;
         p.slices_log2 = sh.slices_log2; p.parts = sh.parts;
         p.groups = (a.N + rows - 1) / rows;
-        // in sixteenths of a (stage, pass); a pass's fragments cost about as much as one and a half of them
-        p.cost = p.parts * 16;
-        p.fixed = p.parts * 24 * (sh.half ? 1 : a.M);
+        set_split(p, s0.half, 1);
         groups += p.groups;
         work += (long long)p.groups * p.parts;
+        if (p.parts > max_parts) max_parts = p.parts;
     }
+    // CTAs at once: one per SM, or (integer form) two where there is enough to do; with little, the free half lets the next
+    // launch's CTAs in early
     const int sms = sm_count();
-    const int slots = nw == 8 && work > 3 * sms ? 2 * sms : sms;
-    const int grid = assign_ctas(b, groups < slots ? (int)groups : slots);
-    return (s0.half ? launch_half : launch_int)(b, s0.ncls, tab, ib, nw, args[0]->x_dt == BTC_F32, grid, s);
+    const bool two = nw == 8 && work > 3 * sms;
+    const int slots = two ? 2 * sms : sms;
+    const Pick pick = {s0.ncls, tab, ib, nw, args[0]->x_dt == BTC_F32};
+    int grid = 0, cluster = 1;
+    long long load = assign_ctas(b, groups < slots ? (int)groups : slots, 1, &grid);
+    // fp16 form, long K and too few rows to give every CTA its own: the passes shared in a cluster where that takes a fifth off
+    // the largest load.  1200 x 16320, v = 20, M = 4: 26.6 -> 11.6 us, 4096 x 11008, v = 8, M = 4: 15.4 -> 12.3 us; at 8192 x
+    // 12000, v = 20, M = 3, whose load shrinks by a seventh, 27.5 us became 31.9.  The integer form stays whole: with two CTAs per
+    // SM, clusters that find no room in one GPC beside the launch before start a round late (a 128-launch chain took 927 us, not
+    // 780), and the order of its sums does not depend on what shares the launch.
+    for (int c = 2; s0.half && c <= 8 && c <= max_parts && groups <= 2 * slots; ++c) {
+        if ((max_parts + c - 1) / c == (max_parts + c - 2) / (c - 1)) continue;
+        int fit = 0, g = 0;
+        const int rc = launch_half_split(b, pick, 0, c, &fit, s);
+        if (rc != BTC_OK) return rc;
+        if (fit < count) continue;
+        Batch t = b;
+        for (int i = 0; i < count; ++i) set_split(t.p[i], true, c);
+        const long long l = assign_ctas(t, fit, c, &g);
+        if (10 * l < 8 * load) { load = l; grid = g; cluster = c; b = t; }
+    }
+    if (cluster > 1) return launch_half_split(b, pick, grid, cluster, nullptr, s);
+    return (s0.half ? launch_half : launch_int)(b, pick, grid, 1, nullptr, s);
 }
 
 static bool same_kernel(const LinearArgs &a, const LinearArgs &b)

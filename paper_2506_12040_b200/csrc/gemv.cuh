@@ -19,13 +19,16 @@
 // so that nothing overflows and small activations keep their bits.  Exact products, fp32 sums.  The cost does not depend
 // on M.
 //
-// Work split.  A tile is 16 output rows; a K-pass is P.slices (8, or 4 where those cover K: a function of K/v alone, so that a
-// layer's result does not depend on what shares its launch) slices of 4 BLK blocks, one warp each; the CTA's other warps take
+// Work split.  A tile is 16 output rows; a K-pass is P.slices (8, or 4 where those cover K: a function of K/v alone, so that
+// in the integer form a layer's result does not depend on what shares its launch) slices of 4 BLK blocks, one warp each; the CTA's other warps take
 // further tiles.  Lane (g = lane / 4, t = lane % 4) of a slice's warp owns rows g and g + 8 and the blocks BLK t .. BLK t +
 // BLK - 1 of the slice; its activations stay in registers as B fragments for the pass.  NW = 8 warps (integer form): two CTAs
 // per SM (<= 113 KB, 128 registers), which also lets the next launch's CTAs load their table and first indices while this
 // launch computes.  NW = 16: one CTA per SM, for codeword tables too large for that, and for the fp16 form, whose
 // fragments cost several times as much to build: there the warps of a slice share the work.
+// Long K in the fp16 form (SPLIT): the kw CTAs of a cluster take the same rows and every kw-th pass, and add their sums through
+// distributed shared memory in a fixed order; a CTA then builds fragments once or twice instead of once per pass.  A template
+// parameter: the cluster's code in every launch cost the small ones 0.2 .. 0.5 us.
 // Every tile leaves one partial result per (slice, row, m) in shared memory; after the last pass of a chunk of tiles the
 // warps meet once, add the slices in a fixed order, apply alpha and mu and store.  Indices arrive through a ring of (tiles,
 // pass) stages by TMA (boxes of 64 blocks with the 128-byte swizzle; rows past N and blocks past K/v arrive as zeros).
@@ -59,13 +62,14 @@ struct Problem {
     int acc;                    // 1: add to what y (fp32) holds
     int x_dt, y_dt;
     int slices_log2, parts;     // slices per K-pass (2 or 3), K-passes
+    int kw;                     // CTAs that share the passes: 1, or the cluster's size
     int tab_bytes;              // bytes of the table to stage in shared memory
     int cost, fixed;            // of one stage, and of a CTA's set-up (planning only)
-    int groups, per, rem;       // stages' worth of rows (NW / slices tiles each); groups / cta_count and groups % cta_count
+    int groups, per, rem;       // stages' worth of rows (NW / slices tiles each); groups / workers and groups % workers (CTAs / kw)
     int cta_begin, cta_count;
 };
 
-struct Layout { int misc, stage_x, stage_x_pitch, park, tab, stage_bytes, stages, total; };   // (the ring comes first: 1024-byte alignment)
+struct Layout { int misc, stage_x, stage_x_pitch, park, chunk, tab, stage_bytes, stages, total; };   // (the ring comes first: 1024-byte alignment)
 
 struct Batch {
     CUtensorMap map[IM_MAXP];   // indices: uint16 {K/v, N}, box {64, rows}, 128-byte swizzle; dense fields as 32-bit words, unswizzled
@@ -78,13 +82,13 @@ struct Batch {
 
 enum { TAB_WORDS = 1, TAB_HEAD = 2, TAB_HALVES = 3 };
 
-// Partial results parked between two meetings of the warps: (tile, slice) entries of 128 or 64 floats.
-template <bool HALF> constexpr int park_entries() { return HALF ? 64 : 96; }
-template <bool HALF> constexpr int entry_floats() { return HALF ? 128 : 64; }
-template <bool HALF> constexpr int park_bytes() { return park_entries<HALF>() * entry_floats<HALF>() * 4; }
+// Partial results parked between two meetings of the warps: (tile, slice) entries of 128 or 64 floats, NW per stage.
+constexpr int max_park_entries(bool half) { return half ? 128 : 96; }
+constexpr int entry_floats(bool half) { return half ? 128 : 64; }
 // misc: mbarriers (2 MAX_STAGES + 1), abort flag, sum x per (slice, column)
 constexpr int MISC_ABORT = (2 * MAX_STAGES + 1) * 8, MISC_SX = MISC_ABORT + 8;
-constexpr int MISC_BYTES = MISC_SX + MAX_SLICES * 8 * 4;
+constexpr int MISC_SXT = MISC_SX + MAX_SLICES * 8 * 4;       // (their sum, for the other CTAs of a cluster)
+constexpr int MISC_BYTES = MISC_SXT + 8 * 4;
 // Where x becomes B fragments.  Integer form, per warp: digit planes, 3 digits x (32 blocks, one spare per 8) x NCLS words.
 // fp16 form, per slice: the rows of x (an even number) as 4 BLK blocks of NCLS quads of 16-bit numbers, in four quarters (what
 // one t owns) 16 bytes apart, so that the 16-byte reads of two rows and four quarters fall on different banks; then E per row.
@@ -171,6 +175,24 @@ __device__ __forceinline__ void mma(float (&c)[4], uint32_t a0, uint32_t a1, uin
                      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "l"(b));
 }
 __device__ __forceinline__ uint64_t pack2(uint32_t lo, uint32_t hi) { return (uint64_t)lo | ((uint64_t)hi << 32); }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_addr(uint32_t a, int rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float peer_ld(uint32_t a) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 peer_ld4(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
 // Index stages are rewritten: these loads stay where they are (volatile); the codeword table is not: the compiler may move
 // its loads (their addresses depend on an index that was read after the waits).
 __device__ __forceinline__ uint4 lds128(uint32_t a) {
@@ -356,14 +378,14 @@ __device__ __forceinline__ void mma_part(const Frags<NCLS, true, BLK> &F, const 
 }
 
 // X32 (fp16 form): fp32 activations; the integer form tells by P.x_dt.
-template <int NCLS, bool HALF, int TAB, int IB, int NW, bool X32>
+template <int NCLS, bool HALF, int TAB, int IB, int NW, bool X32, bool SPLIT>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 gemv_kernel(const __grid_constant__ Batch batch)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     constexpr int CT = NW * 32;
     constexpr int BLK = lane_blocks(HALF, NCLS), SLB = 4 * BLK;      // blocks per lane, per slice
-    constexpr int EF = entry_floats<HALF>(), RC = park_entries<HALF>() / NW;     // stages per chunk
+    constexpr int EF = entry_floats(HALF);
     using F = Frags<NCLS, HALF, BLK>;
     using A = typename std::conditional<HALF, float, int>::type;
     constexpr bool HALVES = TAB == TAB_HALVES;
@@ -374,7 +396,7 @@ gemv_kernel(const __grid_constant__ Batch batch)
     float *s_park = reinterpret_cast<float *>(smem + L.park);
     const uint32_t s_tab = sbase + L.tab;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int NST = L.stages;
+    const int NST = L.stages, RC = HALF ? L.chunk : max_park_entries(false) / NW;      // stages of the ring, stages per chunk
     auto bar_full = [&](int s) { return sbase + L.misc + 8 * s; };
     auto bar_empty = [&](int s) { return sbase + L.misc + 8 * (MAX_STAGES + s); };
     const uint32_t bar_tab = sbase + L.misc + 8 * (2 * MAX_STAGES);
@@ -383,7 +405,9 @@ gemv_kernel(const __grid_constant__ Batch batch)
     int pi = 0;
     while (pi + 1 < batch.count && (int)blockIdx.x >= batch.p[pi + 1].cta_begin) ++pi;
     const Problem &P = batch.p[pi];
-    const int rank = (int)blockIdx.x - P.cta_begin;
+    const int kw = SPLIT ? P.kw : 1, cta = (int)blockIdx.x - P.cta_begin;
+    const int rank = SPLIT ? cta / kw : cta, kq = cta - rank * kw;  // worker, and which passes: kq, kq + kw, ...
+    const int nown = SPLIT ? (P.parts - kq + kw - 1) / kw : P.parts;
     const int glo = rank * P.per + min(rank, P.rem), ghi = glo + P.per + (rank < P.rem ? 1 : 0);
     const int sl2 = P.slices_log2, SL = 1 << sl2, RG = NW >> sl2;    // slices, tiles per stage
     const int PW = SLB << sl2, SROWS = 16 * RG;                      // blocks per pass, rows per stage
@@ -391,11 +415,12 @@ gemv_kernel(const __grid_constant__ Batch batch)
 
     // ---- index ring: number n of this CTA's walk (chunks of RC stages, passes, stages) sits in stage n % NST; warp n % NW
     //      sends for it
-    const int total = (ghi - glo) * P.parts;
+    const int total = (ghi - glo) * nown;
     auto issue = [&](int n, int st) {                    // (one lane)
         int c = glo, len = min(RC, ghi - c), j = 0;
-        while (n >= len * P.parts) { n -= len * P.parts; c += len; len = min(RC, ghi - c); }
+        while (n >= len * nown) { n -= len * nown; c += len; len = min(RC, ghi - c); }
         while (n >= len) { n -= len; ++j; }
+        j = kq + j * kw;
         const uint32_t dst = sbase + st * L.stage_bytes, bar = bar_full(st);
         mbar_expect_tx(bar, (uint32_t)L.stage_bytes);
         if constexpr (IB > 0) {
@@ -408,8 +433,10 @@ gemv_kernel(const __grid_constant__ Batch batch)
         mbar_init(bar_tab, 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        mbar_expect_tx(bar_tab, (uint32_t)P.tab_bytes);
-        bulk_g2s(s_tab, P.tab, (uint32_t)P.tab_bytes, bar_tab);
+        if (total > 0) {
+            mbar_expect_tx(bar_tab, (uint32_t)P.tab_bytes);
+            bulk_g2s(s_tab, P.tab, (uint32_t)P.tab_bytes, bar_tab);
+        }
     }
     if (warp < NST && lane == 0) {                       // (NST <= 8 <= NW)
         mbar_init(bar_full(warp), 1);
@@ -449,7 +476,7 @@ gemv_kernel(const __grid_constant__ Batch batch)
         const int c1 = min(c0 + RC, ghi), nrows = (c1 - c0) * SROWS;
         // alpha / mu of the outputs this thread will finish (static data: loaded ahead of the dependency wait).  fp16 form: thread =
         // (tile, lane slot), rows sg and sg + 8; integer form: thread = (m, row)
-        constexpr int OPT = HALF ? (park_entries<true>() / 4 * 32 + CT - 1) / CT * 2 : (park_entries<false>() / 4 * 32 + CT - 1) / CT;
+        constexpr int OPT = (max_park_entries(HALF) / 4 * 32 + CT - 1) / CT * (HALF ? 2 : 1);
         uint32_t am_reg[OPT];                            // alpha below, mu above
         auto out_row = [&](int q) {
             if (HALF) return ((tid + (q >> 1) * CT) >> 5) * 16 + sg + 8 * (q & 1);
@@ -465,9 +492,10 @@ gemv_kernel(const __grid_constant__ Batch batch)
                 if (P.mu) am_reg[q] |= (uint32_t)__ldg(reinterpret_cast<const unsigned short *>(P.mu) + n) << 16;
             }
         }
-        if (P.parts > 1 || c0 == glo) sx0 = sx1 = 0.f;
+        if (nown > 1 || c0 == glo) sx0 = sx1 = 0.f;
 
-        for (int j = 0; j < P.parts && ok; ++j) {
+        for (int jj = 0; jj < nown && ok; ++jj) {
+            const int j = kq + jj * kw;
             const int jb0 = j * PW + slice * SLB;                    // first block of the slice
             const int kleft = (Kb - jb0) * v;                        // activations from there to the end of the row (<= 0: an empty slice)
             // Integer form: a tile's codewords are looked up while the previous tile's MMAs are in flight, those of a pass's first
@@ -512,9 +540,9 @@ gemv_kernel(const __grid_constant__ Batch batch)
             }
             constexpr bool EARLY = HALF || NCLS <= 4;                // (v = 20: registers)
             if (EARLY && ok) fetch();
-            if (j == 0 && c0 == glo) asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (jj == 0 && c0 == glo) asm volatile("griddepcontrol.wait;" ::: "memory");
 
-            if (P.parts > 1 || c0 == glo) {
+            if (nown > 1 || c0 == glo) {
                 if constexpr (HALF) {
                     // ---- the warps of a slice take its rows of x in turn: 8 activations per lane and step, left in shared memory block
                     //      by block; then lane (g = m, t) of each picks up its own blocks.  (Every lane reading its blocks from global
@@ -539,7 +567,7 @@ gemv_kernel(const __grid_constant__ Batch batch)
                             }
                         }
                     }
-                    if (j > 0 || c0 > glo) slice_sync();                 // (the fragments of the pass before have been picked up)
+                    if (jj > 0 || c0 > glo) slice_sync();                 // (the fragments of the pass before have been picked up)
 #pragma unroll
                     for (int i = 0; i < MR; ++i) {
                         const int m = rg + i * RG;
@@ -763,12 +791,12 @@ gemv_kernel(const __grid_constant__ Batch batch)
                     float4 *q = reinterpret_cast<float4 *>(park);
                     float4 o = make_float4(fmaf(acc[0][0] + acc[1][0], ka, -kc), fmaf(acc[0][1] + acc[1][1], kb, -kd),
                                            fmaf(acc[0][2] + acc[1][2], ka, -kc), fmaf(acc[0][3] + acc[1][3], kb, -kd));
-                    if (j > 0) { const float4 p = *q; o.x += p.x; o.y += p.y; o.z += p.z; o.w += p.w; }
+                    if (jj > 0) { const float4 p = *q; o.x += p.x; o.y += p.y; o.z += p.z; o.w += p.w; }
                     *q = o;
                 } else {
                     float lo = fmaf((float)(acc[0][0] + acc[1][0]), ka, fmaf((float)(acc[0][1] + acc[1][1]), kb, -kc));
                     float hi = fmaf((float)(acc[0][2] + acc[1][2]), ka, fmaf((float)(acc[0][3] + acc[1][3]), kb, -kc));
-                    if (j > 0) { lo += park[0]; hi += park[32]; }
+                    if (jj > 0) { lo += park[0]; hi += park[32]; }
                     park[0] = lo;
                     park[32] = hi;
                 }
@@ -785,55 +813,96 @@ gemv_kernel(const __grid_constant__ Batch batch)
         }
         // ---- the slices meet: add them in a fixed order, apply alpha (and mu), store
         __syncthreads();
-        if (ok && !*s_abort) {
+        const bool fine = ok && !*s_abort;
+        {
             auto finish = [&](int m, int n, float dot, float sx, float al, float mu) {
                 float yv = al * dot + mu * sx;
                 if (P.acc) yv += reinterpret_cast<const float *>(P.y)[(size_t)m * P.N + n];
                 store_from_float(P.y, P.y_dt, (size_t)m * P.N + n, yv);
             };
-            if constexpr (HALF) {
+            // sum over the slices of an output's partial results (integer form: output q of this thread; fp16 form: a lane's four)
+            auto half_src = [&](int q) { return reinterpret_cast<float4 *>(s_park) + (size_t)((((tid + (q >> 1) * CT) >> 5)) << sl2) * 32 + lane; };
+            auto half_sum = [&](int q) {
+                float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 *src = half_src(q);
+                for (int w = 0; w < SL; w += 4)
 #pragma unroll
-                for (int q = 0; q < OPT; q += 2) {
-                    const int tl = (tid + (q >> 1) * CT) >> 5;
-                    if (tl * 16 < nrows && 2 * t < M) {
-                        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-                        float2 sx = make_float2(0.f, 0.f);
-                        const float4 *src = reinterpret_cast<const float4 *>(s_park) + (size_t)(tl << sl2) * 32 + lane;
-                        for (int w = 0; w < SL; w += 4)
+                    for (int i = 0; i < 4; ++i) { const float4 p = src[(w + i) * 32]; d.x += p.x; d.y += p.y; d.z += p.z; d.w += p.w; }
+                return d;
+            };
+            auto int_sum = [&](int q, int m) {           // tile row -> lane group g
+                const int rl = out_row(q);
+                const float2 *src = reinterpret_cast<const float2 *>(s_park + ((rl >> 4) << sl2) * EF + ((rl >> 3) & 1) * 32 + ((rl & 3) * 2 + ((rl >> 2) & 1)) * 4 + 2 * m);
+                float d4[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int w = 0; w < SL; w += 4)
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) { const float4 p = src[(w + i) * 32]; d.x += p.x; d.y += p.y; d.z += p.z; d.w += p.w; }
-                        if (P.mu)
-                            for (int w = 0; w < SL; ++w) { sx.x += s_sx[w * 8 + 2 * t]; sx.y += s_sx[w * 8 + 2 * t + 1]; }
+                    for (int i = 0; i < 4; ++i) { const float2 p = src[(w + i) * (EF / 2)]; d4[i] += p.x + p.y; }
+                return (d4[0] + d4[1]) + (d4[2] + d4[3]);
+            };
+            auto half_finish = [&](int q, const float4 &d, float sxa, float sxb) {
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) {
-                            const int n = c0 * SROWS + out_row(q + i);
-                            if (n < P.N) {
-                                const float al = lo_half(am_reg[q + i]), mu = lo_half(am_reg[q + i] >> 16);
-                                finish(2 * t, n, i ? d.z : d.x, sx.x, al, mu);
-                                if (2 * t + 1 < M) finish(2 * t + 1, n, i ? d.w : d.y, sx.y, al, mu);
-                            }
+                for (int i = 0; i < 2; ++i) {
+                    const int n = c0 * SROWS + out_row(q + i);
+                    if (n < P.N) {
+                        const float al = lo_half(am_reg[q + i]), mu = lo_half(am_reg[q + i] >> 16);
+                        finish(2 * t, n, i ? d.z : d.x, sxa, al, mu);
+                        if (2 * t + 1 < M) finish(2 * t + 1, n, i ? d.w : d.y, sxb, al, mu);
+                    }
+                }
+            };
+            // sum of x of a row: over the slices (fp16 form: column c; integer form: c = 2 m, two columns)
+            auto sx_sum = [&](int c) {
+                float sx = 0.f;
+                for (int w = 0; w < SL; ++w) sx += HALF ? s_sx[w * 8 + c] : s_sx[w * 8 + c] + s_sx[w * 8 + c + 1];
+                return sx;
+            };
+            if (!SPLIT || kw == 1) {                     // (with kw == 1 every CTA of the cluster comes this way)
+                if (fine) {
+#pragma unroll
+                    for (int q = 0; q < OPT; q += HALF ? 2 : 1) {
+                        if constexpr (HALF) {
+                            if (((tid + (q >> 1) * CT) >> 5) * 16 < nrows && 2 * t < M)
+                                half_finish(q, half_sum(q), P.mu ? sx_sum(2 * t) : 0.f, P.mu ? sx_sum(2 * t + 1) : 0.f);
+                        } else {
+                            const int m = tid + q * CT >= nrows ? 1 : 0, rl = out_row(q), n = c0 * SROWS + rl;
+                            if (m < M && rl < nrows && n < P.N)
+                                finish(m, n, int_sum(q, m), P.mu ? sx_sum(2 * m) : 0.f, lo_half(am_reg[q]), lo_half(am_reg[q] >> 16));
                         }
                     }
                 }
-            } else {
+            } else if constexpr (SPLIT) {
+                // this CTA's sums go to the entry of slice 0 (read by the same thread alone); a warp's outputs are finished by one CTA
+                float *s_sxt = reinterpret_cast<float *>(smem + L.misc + MISC_SXT);
 #pragma unroll
-                for (int q = 0; q < OPT; ++q) {
-                    const int m = tid + q * CT >= nrows ? 1 : 0, rl = out_row(q), n = c0 * SROWS + rl;
-                    if (m < M && rl < nrows && n < P.N) {
-                        // tile row -> lane group g
-                        const float2 *src = reinterpret_cast<const float2 *>(s_park + ((rl >> 4) << sl2) * EF + ((rl >> 3) & 1) * 32 + ((rl & 3) * 2 + ((rl >> 2) & 1)) * 4 + 2 * m);
-                        float d4[4] = {0.f, 0.f, 0.f, 0.f}, sx = 0.f;
-                        for (int w = 0; w < SL; w += 4)
+                for (int q = 0; q < OPT; q += 2)
+                    if (((tid + (q >> 1) * CT) >> 5) * 16 < nrows && 2 * t < M) *half_src(q) = half_sum(q);
+                if (P.mu && tid < M) s_sxt[tid] = sx_sum(tid);
+                cluster_sync();
+                auto peers = [&](uint32_t a) {           // (in the order of the CTAs)
+                    float f[8], r = 0.f;
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) { const float2 p = src[(w + i) * (EF / 2)]; d4[i] += p.x + p.y; }
-                        if (P.mu)
-                            for (int w = 0; w < SL; ++w) sx += s_sx[w * 8 + 2 * m] + s_sx[w * 8 + 2 * m + 1];
-                        finish(m, n, (d4[0] + d4[1]) + (d4[2] + d4[3]), sx, lo_half(am_reg[q]), lo_half(am_reg[q] >> 16));
-                    }
+                    for (int k = 0; k < 8; ++k) f[k] = k < kw ? peer_ld(peer_addr(a, k)) : 0.f;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) r += f[k];
+                    return r;
+                };
+                const uint32_t sxt = sbase + L.misc + MISC_SXT;
+#pragma unroll
+                for (int q = 0; q < OPT; q += 2) {
+                    const int tl = (tid + (q >> 1) * CT) >> 5;
+                    if (!fine || tl % kw != kq || tl * 16 >= nrows || 2 * t >= M) continue;
+                    const uint32_t a = smem_addr(half_src(q));
+                    float4 d = make_float4(0.f, 0.f, 0.f, 0.f), p[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) p[k] = k < kw ? peer_ld4(peer_addr(a, k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) { d.x += p[k].x; d.y += p[k].y; d.z += p[k].z; d.w += p[k].w; }
+                    half_finish(q, d, P.mu ? peers(sxt + 8 * t) : 0.f, P.mu && 2 * t + 1 < M ? peers(sxt + 8 * t + 4) : 0.f);
                 }
+                cluster_sync();                          // (nobody goes on while its sums are being read)
             }
         }
-        if (c1 < ghi) __syncthreads();                   // the next chunk overwrites what was just read
+        if ((!SPLIT || kw == 1) && c1 < ghi) __syncthreads();        // the next chunk overwrites what was just read
     }
     // A CTA that gave up on a wait may still have copies in flight into its shared memory: let them land before it goes.
     if (*s_abort) {
@@ -843,10 +912,14 @@ gemv_kernel(const __grid_constant__ Batch batch)
     }
 }
 
-template <int NCLS, bool HALF, int TAB, int IB, int NW, bool X32 = false>
-int launch_kernel(const Batch &b, int grid, cudaStream_t s)
+// Which kernel: classes per block (v / 4 rounded up), table form, index bits (0: 16-bit containers), warps, fp32 activations.
+struct Pick { int ncls, tab, ib, nw; bool x32; };
+
+// grid > 0: launches in clusters of `cluster` CTAs.  grid == 0: writes the number of such clusters that fit the device at once.
+template <int NCLS, bool HALF, int TAB, int IB, int NW, bool X32, bool SPLIT>
+int launch_kernel(const Batch &b, int grid, int cluster, int *fit, cudaStream_t s)
 {
-    auto kern = gemv_kernel<NCLS, HALF, TAB, IB, NW, X32>;
+    auto kern = gemv_kernel<NCLS, HALF, TAB, IB, NW, X32, SPLIT>;
     // the attribute is set once per device to all a CTA may ask for; which launch needs how much is the planner's business
     constexpr int most = NW == 8 ? 113 * 1024 : 227 * 1024;
     static std::atomic<uint64_t> done{0};
@@ -863,29 +936,47 @@ int launch_kernel(const Batch &b, int grid, cudaStream_t s)
     cfg.blockDim = dim3(NW * 32);
     cfg.dynamicSmemBytes = (size_t)b.L.total;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    if (grid == 0) {
+        static std::atomic<int> known[16][9];
+        int n = dev < 16 ? known[dev][cluster].load(std::memory_order_relaxed) : 0;
+        if (!n) {
+            cfg.gridDim = dim3((unsigned)cluster);
+            cfg.dynamicSmemBytes = most;
+            cfg.attrs = at + 1;
+            cfg.numAttrs = 1;
+            e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+            if (e != cudaSuccess) return cuda_fail(e);
+            if (dev < 16) known[dev][cluster].store(n, std::memory_order_relaxed);
+        }
+        *fit = n;
+        return BTC_OK;
+    }
     e = cudaLaunchKernelEx(&cfg, kern, b);
     return e == cudaSuccess ? BTC_OK : cuda_fail(e);
 }
 
-// Which kernel: classes per block (v / 4 rounded up), table form, index bits (0: 16-bit containers), warps.
-int launch_int(const Batch &b, int ncls, int tab, int ib, int nw, bool x32, int grid, cudaStream_t s);
-int launch_half(const Batch &b, int ncls, int tab, int ib, int nw, bool x32, int grid, cudaStream_t s);
+// (one translation unit each)
+int launch_int(const Batch &b, const Pick &k, int grid, int cluster, int *fit, cudaStream_t s);
+int launch_half(const Batch &b, const Pick &k, int grid, int cluster, int *fit, cudaStream_t s);
+int launch_half_split(const Batch &b, const Pick &k, int grid, int cluster, int *fit, cudaStream_t s);
 
-template <bool HALF>
-int dispatch(const Batch &b, int ncls, int tab, int ib, int nw, bool x32, int grid, cudaStream_t s)
+template <bool HALF, bool SPLIT>
+int dispatch(const Batch &b, const Pick &k, int grid, int cluster, int *fit, cudaStream_t s)
 {
-#define GV_CASE(C, T, I, W) if (ncls == C && tab == T && ib == I && nw == W) return launch_kernel<C, HALF, T, I, W>(b, grid, s)
+#define GV_CASE(C, T, I, W) if (k.ncls == C && k.tab == T && k.ib == I && k.nw == W) return launch_kernel<C, HALF, T, I, W, false, SPLIT>(b, grid, cluster, fit, s)
 #define GV_TABLES(C, T) GV_CASE(C, T, 0, 8); GV_CASE(C, T, 0, 16)
 #define GV_PACKED(C, T) GV_CASE(C, T, 12, 8); GV_CASE(C, T, 13, 8)
     if constexpr (HALF) {
 #define GV_HALF(C, X) GV_CASE_X(C, TAB_WORDS, 0, X); GV_CASE_X(C, TAB_HEAD, 0, X)
 #define GV_HALF_PACKED(C, X) GV_CASE_X(C, TAB_WORDS, 12, X); GV_CASE_X(C, TAB_WORDS, 13, X)
-#define GV_CASE_X(C, T, I, X) if (ncls == C && tab == T && ib == I && x32 == X) return launch_kernel<C, true, T, I, 16, X>(b, grid, s)
+#define GV_CASE_X(C, T, I, X) if (k.ncls == C && k.tab == T && k.ib == I && k.x32 == X) return launch_kernel<C, true, T, I, 16, X, SPLIT>(b, grid, cluster, fit, s)
         GV_HALF(1, false); GV_HALF(2, false); GV_HALF(3, false); GV_HALF(4, false); GV_HALF(5, false); GV_HALF(6, false);
         GV_HALF(1, true); GV_HALF(2, true); GV_HALF(3, true); GV_HALF(4, true); GV_HALF(5, true);
         GV_HALF_PACKED(1, false); GV_HALF_PACKED(2, false); GV_HALF_PACKED(3, false); GV_HALF_PACKED(4, false);

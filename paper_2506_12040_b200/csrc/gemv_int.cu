@@ -3,6 +3,6 @@
 
 namespace btc {
 namespace gv {
-int launch_int(const Batch &b, int ncls, int tab, int ib, int nw, bool x32, int grid, cudaStream_t s) { return dispatch<false>(b, ncls, tab, ib, nw, x32, grid, s); }
+int launch_int(const Batch &b, const Pick &k, int grid, int cluster, int *fit, cudaStream_t s) { return dispatch<false, false>(b, k, grid, cluster, fit, s); }
 }  // namespace gv
 }  // namespace btc

@@ -118,6 +118,26 @@ def test_gemv_edges(N, K, v, Kc, M, dt, mu):
     assert torch.equal(y, again) and btc.device_status() == 0
 
 
+@pytest.mark.parametrize("N,K,v,Kc,M,mu,beside", [
+    (16, 520 * 20, 20, 40000, 3, True, 0),         # one tile, five passes and a bit
+    (1200, 2048 * 8, 8, 85, 8, True, 0),           # every pass of the cluster full
+    (1190, 1168 * 14, 14, 2353, 1, True, 0),       # last tile ragged, last pass short
+    (2049, 816 * 20, 20, 65536, 4, False, 0),      # table does not fit: its head, the rest from L2
+    (700, 344 * 24, 24, 900, 2, False, 0),         # passes no multiple of the cluster
+    (500, 1032 * 16, 16, 4096, 5, True, 40),       # beside layers with a single pass, in clusters that share nothing
+])
+def test_gemv_long_k_shared_in_clusters(N, K, v, Kc, M, mu, beside):
+    specs = [_spec(N, K, v, Kc, with_mu=mu, outlier_frac=0.01)] + [_spec(n, 32 * v, v, Kc, with_mu=mu) for n in ((beside, 2 * beside) if beside else ())]
+    Ls = [wl.make_layer(s, M, seed=N + K + M + i) for i, s in enumerate(specs)]
+    layers = [dict(x=d["x"], idx=d["idx"], C_packed=d["Cp"], alpha=d["alpha"], mu=d["mu"], v=v, Kc=Kc) for d in map(to_device, Ls)]
+    outs, again = btc.linear_gemv_batch(layers), btc.linear_gemv_batch(layers)
+    for L, y, y2 in zip(Ls, outs, again):
+        rel, fwd = errors(y, oracle_y(L), L)
+        assert rel <= TOL_GEMV and fwd <= TOL_GEMV, (L.spec, rel, fwd)
+        assert torch.equal(y, y2)
+    assert btc.device_status() == 0
+
+
 @pytest.mark.parametrize("config", [1, 2, 3])
 def test_gemv_parity_benchmark_configs(config):
     """Full-size layers of the benchmark configs, every output compared (the oracle needs seconds)."""
