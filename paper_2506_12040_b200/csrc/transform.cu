@@ -3,10 +3,14 @@
 // at inference as X <- X T).  With a row of x viewed row-major as a k1 x k2 matrix X (k1 * k2 = K):
 //     X' = P1^T (X o sigma) P2,     X'[c][d] = sum_a sum_b P1[a][c] * sigma[a k2 + b] * X[a][b] * P2[b][d]
 // computed as two small products with fp32 accumulation: Y = (X o sigma) P2, then X' = P1^T Y.
-// A CTA owns a tile of TR_DT output columns d and a group of rows of x: it stages the k2 x TR_DT slab of P2 and all
-// of P1 in shared memory once, then for each of its rows loads X (K values) and produces X'[:, d-tile]; a decode step
-// with one row of x therefore spreads over k2 / TR_DT SMs instead of one, and a prefill batch shares the staged factors.  The result is written as fp32 for the decode path (which quantises or rounds the activations
-// itself, so no intermediate 16-bit rounding is added) and in the dtype of x for the tensor-core path.
+// The result is written as fp32 for the decode path (which quantises or rounds the activations itself, so no intermediate
+// 16-bit rounding is added) and in the dtype of x for the tensor-core path.
+// transform_kernel (up to eight rows, fp32 activations, factor sizes the other does not take): a CTA owns a tile of TR_DT output
+// columns d and a group of rows of x: it stages the k2 x TR_DT slab of P2 and all of P1 in shared memory once, then for each of
+// its rows loads X (K values) and produces X'[:, d-tile]; a decode step with one row of x therefore spreads over k2 / TR_DT
+// SMs instead of one.
+#include <atomic>
+#include <type_traits>
 #include "btc_internal.cuh"
 
 namespace btc {
@@ -128,285 +132,343 @@ transform_kernel(const void *__restrict__ x, int x_dt, const uint32_t *__restric
     }
 }
 
-// ---- many rows of x (the tensor-core path's prologue): the two products on the warp-level tensor cores ----------------
-// For M >= 64 the two products are dense contractions: (M k1) x k2 x k2 and, per row, k1 x k1 x k2 -- 1.2 G multiply-adds
-// for 512 rows of K = 11008 = 86 x 128.  Here a CTA keeps both factors in shared memory as tf32 and takes whole rows of
-// x: Y = (X o sigma) P2 and X' = P1^T Y as mma.sync.m16n8k8 (tf32 operands, fp32 accumulation).  16-bit activations are
-// exact in tf32; the factors and Y carry a 2^-11 rounding, below the 2^-9 of the 16-bit result this path writes.
-// Shared-memory pitches are 4 or 8 words past a multiple of 32, so the fragment reads of a warp fall on 32 banks.
-constexpr int TM_THREADS = 256;
-constexpr int TM_WARPS = TM_THREADS / 32;
+// ---- 16-bit activations, k2 a multiple of 16, k1 up to 128: the two products on the warp-level tensor cores ---------------
+// bf16 operands, fp32 accumulation; a factor, and Y between the products, is a sum of TERMS bf16 numbers (two hold 16 bits of
+// a value, three all 24 of an fp32), and of the products of terms only those below the last term's own rounding are left out.
+// An f16 activation is the sum of two bf16 numbers, a bf16 one is its own operand: loaded, sign bits flipped, multiplied.
+// An item of work is one row of x, sixteen output columns d (a slice) and a share of the output rows c, and belongs to one
+// warp: Y^T of the slice (16 x k1) stays in registers, where the accumulators of the first product, rounded to terms, are B
+// fragments of the second.  Only the factors go through shared memory, split into terms and laid out as A fragments, once
+// per CTA and before x is waited for; rows then cost no barrier.
+// A lane's columns of x are four neighbours (both products may take their inner index in any order, as long as A and B agree),
+// so x is read from global memory straight into fragments, 8 bytes a load; the warps of a CTA take the slices of the same
+// rows, so all but the first read from L1.  Likewise a lane's results are four neighbouring columns.
+// Bound: instruction issue and, for a few rows, the set-up (factors from L2, split) and one item's chain of MMAs; DRAM is
+// under a tenth busy.  A form with both products through shared memory and two barriers a row (tf32; fp32 FMAs below 64 rows)
+// took 12.6 us for 512 rows of 64 x 64 and 21.4 for 63, now 8.3 and 4.8; 86 x 128, 2048 rows: 134.6 -> 80.8, 63 rows: 41.1 ->
+// 14.9.
+constexpr int TM_WARPS = 8;
 
-__device__ __forceinline__ uint32_t tm_tf32(float f) {
+__device__ __forceinline__ uint32_t tm_pack(float lo, float hi) {
     uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(f));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-__device__ __forceinline__ void tm_mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+__device__ __forceinline__ float tm_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float tm_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+__device__ __forceinline__ void tm_mma(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+// the next term of a pair: taken off what is left of it
+__device__ __forceinline__ uint32_t tm_term(float &lo, float &hi) {
+    const uint32_t w = tm_pack(lo, hi);
+    lo -= tm_lo(w); hi -= tm_hi(w);
+    return w;
 }
 
-struct TmLayout { int k1m, k1k, xp, yp, p1p, p2p; size_t x_off, y_off, p1_off, p2_off, words; };
-__host__ __device__ inline TmLayout tm_layout(int k1, int k2)
-{
-    TmLayout L;
-    L.k1m = (k1 + 15) / 16 * 16;            // k1 as an M dimension (16-row tiles)
-    L.k1k = (k1 + 7) / 8 * 8;               // k1 as a K dimension (8-wide steps)
-    L.xp = k2 + 4;                          // X [k1m][xp]: A operand of the first product (rows a, columns b)
-    L.yp = k2 + 8;                          // Y [k1k][yp]: B operand of the second (rows a, columns d)
-    L.p1p = L.k1m + 8;                      // P1 [k1k][p1p]: A operand of the second, read transposed (rows a, columns c)
-    L.p2p = k2 + 8;                         // P2 [k2][p2p]: B operand of the first (rows b, columns d)
-    L.x_off = 0;
-    L.y_off = L.x_off + (size_t)L.k1m * L.xp;
-    L.p1_off = L.y_off + (size_t)L.k1k * L.yp;
-    L.p2_off = L.p1_off + (size_t)L.k1k * L.p1p;
-    L.words = L.p2_off + (size_t)k2 * L.p2p;
-    return L;
+// One A fragment (16 rows x 16 of the inner index) of P^T as TERMS x 32 lanes x 16 bytes.  f[2 i], f[2 i + 1]: register i.
+template <int TERMS>
+__device__ __forceinline__ void tm_put(uint4 *dst, float (&f)[8]) {
+#pragma unroll
+    for (int u = 0; u < TERMS; ++u) {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = tm_term(f[2 * i], f[2 * i + 1]);
+        dst[u * 32] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
 }
 
-// MT: 16-row tiles of k1.  TK1 / TK2: the factor sizes as compile-time constants (0: taken from the arguments), so
-// that the pitches and loop bounds of the common shapes fold into immediates.
-template <int MT, int TK1, int TK2>
-__global__ void __launch_bounds__(TM_THREADS, 1)
-transform_mma_kernel(const void *__restrict__ x, int x_dt, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
-                     const float *__restrict__ P2, int k1_arg, int k2_arg, void *__restrict__ xt, int out_dt, int M)
+struct TmPlan { int ds, cg, rw, p2_frags, mask_off; };       // slices, shares of c and rows per CTA (ds * cg * rw warps); A fragments of P2
+
+// NA: 8-wide tiles of a (even; k1 rounded up to 16, and beyond to a size instantiated; at least LO of them are full).  F16:
+// activations f16, else bf16.  K2: k2 where it is one of the usual sizes (addresses become immediates), else 0.  DW: 16-wide
+// parts of a slice; two use every activation and every fragment of P1 twice.
+template <int NA, int TERMS, bool F16, int K2, int DW>
+__global__ void __launch_bounds__(TM_WARPS * 32, 1)
+transform_mma_kernel(const uint16_t *__restrict__ x, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
+                     const float *__restrict__ P2, int k1, int k2_arg, void *__restrict__ xt, int out_dt, int M, TmPlan plan)
 {
-    extern __shared__ __align__(16) uint32_t tm_smem[];
-    const int k1 = TK1 ? TK1 : k1_arg, k2 = TK2 ? TK2 : k2_arg;
+    constexpr int LO = NA == 2 ? 0 : NA <= 8 ? NA - 2 : NA - 4, U = 8;
+    extern __shared__ __align__(16) uint4 tm_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const TmLayout L = tm_layout(k1, k2);
-    uint32_t *Xs = tm_smem + L.x_off, *Ys = tm_smem + L.y_off, *P1s = tm_smem + L.p1_off, *P2s = tm_smem + L.p2_off;
+    const int k2 = K2 ? K2 : k2_arg;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-    const int K = k1 * k2;
-    // the factors, once per CTA, zero-padded to whole tiles; so are the pad rows of X and Y.  Loads go out in batches
-    // of eight or sixteen before any of them is used (a loop of load-convert-store would wait for each trip to L2 in turn)
+    const int K = k1 * k2, ks2 = k2 / 16, nc = (k1 + 15) / 16;
+    uint4 *f2 = tm_smem, *f1 = tm_smem + (size_t)plan.p2_frags * TERMS * 32;
+    uint2 *mask = reinterpret_cast<uint2 *>(reinterpret_cast<char *>(tm_smem) + plan.mask_off);
+    // column of a 16-wide part of a slice that rows g and g + 8 of a fragment of P2, and columns 2t, 2t + 1 of the two result
+    // tiles, stand for
+    const int dg = 4 * (g >> 1) + (g & 1);
+    // ---- the factors as fragments, eight loads of eight in flight per thread; the signs as masks of a lane's four activations
     {
-        const int n1 = L.k1k * L.p1p, n2 = k2 * L.p2p;
-        for (int i0 = tid; i0 < n1; i0 += 16 * TM_THREADS) {
-            float f[16];
+        const int part0 = blockIdx.y * plan.ds * DW, nf = plan.p2_frags + nc * (NA / 2), nw = blockDim.x >> 5;
+        for (int i0 = warp; i0 < NA * ks2; i0 += 2 * U * nw) {           // [k][tile of a][lane]
+            uint32_t w[2 * U];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const int i = i0 + u * TM_THREADS, a = i / L.p1p, c = i - a * L.p1p;
-                f[u] = (i < n1 && a < k1 && c < k1) ? __ldg(P1 + (size_t)a * k1 + c) : 0.f;
+            for (int u = 0; u < 2 * U; ++u) {
+                const int i = i0 + u * nw, k = i / NA, a = 8 * (i - k * NA) + g, e = a * k2 + 16 * k;
+                w[u] = i < NA * ks2 && a < k1 ? __ldg(sigma_bits + (e >> 5)) >> ((e & 31) + 4 * t) : 0u;
             }
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const int i = i0 + u * TM_THREADS;
-                if (i < n1) P1s[i] = tm_tf32(f[u]);
+            for (int u = 0; u < 2 * U; ++u) {
+                const uint32_t sb = w[u] & 15u;
+                if (i0 + u * nw < NA * ks2) mask[(i0 + u * nw) * 32 + lane] = make_uint2((sb * 0x40008000u) & 0x80008000u, (sb * 0x10002000u) & 0x80008000u);
             }
         }
-        if ((reinterpret_cast<uintptr_t>(P2) & 15u) == 0) {
-            // rows of P2 are k2 floats, k2 a multiple of 16: four per load, eight loads in flight
-            const int q2 = k2 / 4, nq = k2 * q2;
-            for (int i0 = tid; i0 < nq; i0 += 8 * TM_THREADS) {
-                float4 f[8];
+        for (int i0 = warp; i0 < nf; i0 += U * nw) {
+            float f[U][8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + u * TM_THREADS;
-                    f[u] = i < nq ? __ldg(reinterpret_cast<const float4 *>(P2) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+            for (int u = 0; u < U; ++u) {
+                const int i = i0 + u * nw;
+                const bool second = i >= plan.p2_frags;
+                const int j = second ? i - plan.p2_frags : i, per = second ? NA / 2 : ks2, q = j / per, k = j - q * per;
+                // element (inner, outer) of the factor: rows b of P2 and its columns d, rows a of P1 and its columns c
+                const int n = second ? k1 : k2, in0 = 16 * k + (second ? 2 * t : 4 * t), in1 = in0 + (second ? 8 : 2);
+                const int out0 = 16 * (second ? q : part0 + q) + (second ? g : dg), out1 = out0 + (second ? 8 : 2);
+                const float *src = (second ? P1 : P2) + (size_t)in0 * n + out0;
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + u * TM_THREADS;
-                    if (i < nq) {
-                        const int b = i / q2, d = 4 * (i - b * q2);
-                        *reinterpret_cast<uint4 *>(P2s + (size_t)b * L.p2p + d) = make_uint4(tm_tf32(f[u].x), tm_tf32(f[u].y), tm_tf32(f[u].z), tm_tf32(f[u].w));
-                    }
+                for (int r = 0; r < 8; ++r) {            // (register r / 2, half r % 2)
+                    const int in = (r & 4 ? in1 : in0) + (r & 1), out = r & 2 ? out1 : out0;
+                    f[u][r] = i < nf && in < n && out < n ? __ldg(src + (size_t)(in - in0) * n + (out - out0)) : 0.f;
                 }
             }
-            for (int i = tid; i < k2 * 8; i += TM_THREADS) P2s[(size_t)(i >> 3) * L.p2p + k2 + (i & 7)] = 0u;   // pad columns
-        } else {
-            for (int i0 = tid; i0 < n2; i0 += 8 * TM_THREADS) {
-                float f[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + u * TM_THREADS, b = i / L.p2p, d = i - b * L.p2p;
-                    f[u] = (i < n2 && d < k2) ? __ldg(P2 + (size_t)b * k2 + d) : 0.f;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + u * TM_THREADS;
-                    if (i < n2) P2s[i] = tm_tf32(f[u]);
-                }
-            }
+            for (int u = 0; u < U; ++u)
+                if (i0 + u * nw < nf) tm_put<TERMS>(tm_smem + (size_t)(i0 + u * nw) * TERMS * 32 + lane, f[u]);
         }
     }
-    for (int i = tid; i < L.k1m * L.xp; i += TM_THREADS) Xs[i] = 0u;
-    for (int i = tid; i < L.k1k * L.yp; i += TM_THREADS) Ys[i] = 0u;
+    __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int npairs = k2 / 16;             // pairs of 8-column tiles of d
-    constexpr int MG = (MT + 1) / 2;        // a warp's work item: half of the a (or c) tiles x one pair of d tiles
-    // a row of x: eight 16-bit activations per load (k2 is a multiple of 16: they share a row a of X); the loads of the
-    // next row are in flight while this row's products run
-    constexpr int NQ = 8;                   // loads per thread: K <= 8 * NQ * TM_THREADS
-    const int nvec = K / 8;
-    uint4 q[NQ];
-    auto load_row = [&](int m) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(x) + (size_t)m * K);
+
+    const int cs = warp % plan.cg, sl = (warp / plan.cg) % plan.ds, rw = warp / (plan.cg * plan.ds);
+    const int d0 = 16 * DW * (blockIdx.y * plan.ds + sl);
+    if (d0 >= k2) return;
+    const int c_per = (nc + plan.cg - 1) / plan.cg, ct0 = cs * c_per, ct1 = min(nc, ct0 + c_per);
+    if (ct0 >= ct1) return;
+    const uint4 *A2 = f2 + (size_t)sl * DW * ks2 * TERMS * 32 + lane, *A1 = f1 + lane;
+    mask += lane;
+    // (an MMA cuts its sum off where an fp32 addition rounds: with three terms each step of the inner index is summed from zero, its
+    // smallest products first, and added to the accumulator as an fp32)
+    auto part = [](float (&step)[4], float (&sum)[4]) -> float (&)[4] { return TERMS > 2 ? step : sum; };
+    constexpr int PF = NA <= 4 ? 4 : 2;                  // loads ahead, in steps of the first product
+    for (int m = blockIdx.x * plan.rw + rw; m < M; m += gridDim.x * plan.rw) {
+        const uint16_t *xr = x + (size_t)m * K + (size_t)g * k2 + 4 * t;
+        uint2 q[PF][NA];
+        auto load = [&](int k, uint2 (&dst)[NA]) {
 #pragma unroll
-        for (int u = 0; u < NQ; ++u) {
-            const int i = tid + u * TM_THREADS;
-            q[u] = i < nvec ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
-        }
-    };
-    if ((int)blockIdx.x < M) load_row(blockIdx.x);
-    for (int m = blockIdx.x; m < M; m += gridDim.x) {
-        const size_t row = (size_t)m * K;
-        __syncthreads();                    // (the previous row's X and Y are no longer read; pads and factors are in place)
+            for (int at = 0; at < NA; ++at)
+                dst[at] = at < LO || 8 * at + g < k1 ? __ldg(reinterpret_cast<const uint2 *>(xr + (size_t)(8 * at) * k2 + 16 * k)) : make_uint2(0u, 0u);
+        };
 #pragma unroll
-        for (int u = 0; u < NQ; ++u) {
-            const int i = tid + u * TM_THREADS;
-            if (i < nvec) {
-                const int k = 8 * i, a = k / k2, bcol = k - a * k2;
-                const uint32_t sg = __ldg(sigma_bits + (k >> 5)) >> (k & 31);
-                const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
-                uint32_t o[8];
+        for (int u = 0; u < PF; ++u)
+            if (u < ks2) load(u, q[u]);
+        // ---- Y^T[d][a] = sum_b P2[b][d] X[a][b]
+        float y[DW][NA][4];
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    float lo, hi;
-                    if (x_dt == BTC_F16) { const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&w[h])); lo = f.x; hi = f.y; }
-                    else { lo = __uint_as_float(w[h] << 16); hi = __uint_as_float(w[h] & 0xffff0000u); }
-                    if ((sg >> (2 * h)) & 1u) lo = -lo;
-                    if ((sg >> (2 * h + 1)) & 1u) hi = -hi;
-                    o[2 * h] = tm_tf32(lo); o[2 * h + 1] = tm_tf32(hi);
+        for (int p = 0; p < DW; ++p)
+#pragma unroll
+            for (int at = 0; at < NA; ++at)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) y[p][at][i] = 0.f;
+        for (int k0 = 0; k0 < ks2; k0 += PF) {
+#pragma unroll
+            for (int u = 0; u < PF; ++u) {
+                const int k = k0 + u;
+                if (k < ks2) {
+                    uint4 w[DW][TERMS];
+#pragma unroll
+                    for (int p = 0; p < DW; ++p)
+#pragma unroll
+                        for (int i = 0; i < TERMS; ++i) w[p][i] = A2[(size_t)((p * ks2 + k) * TERMS + i) * 32];
+                    // a few tiles of a at a time, term by term: MMAs on one accumulator are never neighbours
+                    constexpr int G = 4 / DW;
+#pragma unroll
+                    for (int a0 = 0; a0 < NA; a0 += G) {
+                        uint32_t xb[G][2], xl[G][2];
+                        float step[DW][G][4] = {};
+#pragma unroll
+                        for (int n = 0; n < G; ++n) {
+                            const uint2 sg = mask[(k * NA + a0 + n) * 32];
+                            xb[n][0] = q[u][a0 + n].x ^ sg.x;
+                            xb[n][1] = q[u][a0 + n].y ^ sg.y;
+                            if constexpr (F16) {
+#pragma unroll
+                                for (int i = 0; i < 2; ++i) {
+                                    float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&xb[n][i]));
+                                    xb[n][i] = tm_term(f.x, f.y);
+                                    xl[n][i] = tm_pack(f.x, f.y);
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int i = TERMS - 1; i >= 0; --i) {
+                            if (F16 && i < TERMS - 1)
+#pragma unroll
+                                for (int n = 0; n < G; ++n)
+#pragma unroll
+                                    for (int p = 0; p < DW; ++p) tm_mma(part(step[p][n], y[p][a0 + n]), w[p][i], xl[n][0], xl[n][1]);
+#pragma unroll
+                            for (int n = 0; n < G; ++n)
+#pragma unroll
+                                for (int p = 0; p < DW; ++p) tm_mma(part(step[p][n], y[p][a0 + n]), w[p][i], xb[n][0], xb[n][1]);
+                        }
+                        if (TERMS > 2)
+#pragma unroll
+                            for (int n = 0; n < G; ++n)
+#pragma unroll
+                                for (int p = 0; p < DW; ++p)
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) y[p][a0 + n][i] += step[p][n][i];
+                    }
+                    if (k + PF < ks2) load(k + PF, q[u]);
                 }
-                uint4 *dst = reinterpret_cast<uint4 *>(Xs + (size_t)a * L.xp + bcol);
-                dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
             }
         }
-        if (m + (int)gridDim.x < M) load_row(m + gridDim.x);
-        __syncthreads();
-        // ---- Y[a][d] = sum_b X[a][b] P2[b][d]
-        for (int item = warp; item < 2 * npairs; item += TM_WARPS) {
-            const int pr = item >> 1, mt0 = (item & 1) * MG;
-            float acc[MG][2][4];
+        uint32_t yb[DW][NA][2][TERMS];                   // (rows d of the tiles' lower and upper half; terms)
 #pragma unroll
-            for (int mt = 0; mt < MG; ++mt)
+        for (int p = 0; p < DW; ++p)
+#pragma unroll
+            for (int at = 0; at < NA; ++at)
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[mt][h][i] = 0.f;
-            const int d0 = pr * 16;
-            for (int kk = 0; kk < k2; kk += 8) {
-                uint32_t b0[2], b1[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    b0[h] = P2s[(size_t)(kk + t) * L.p2p + d0 + 8 * h + g];
-                    b1[h] = P2s[(size_t)(kk + t + 4) * L.p2p + d0 + 8 * h + g];
-                }
-#pragma unroll
-                for (int mt = 0; mt < MG; ++mt) {
-                    if (mt0 + mt < MT) {
-                        const uint32_t *xa = Xs + (size_t)((mt0 + mt) * 16 + g) * L.xp + kk + t;
-                        const uint32_t a0 = xa[0], a1 = xa[8 * L.xp], a2 = xa[4], a3 = xa[8 * L.xp + 4];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) tm_mma(acc[mt][h], a0, a1, a2, a3, b0[h], b1[h]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int mt = 0; mt < MG; ++mt)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int a = (mt0 + mt) * 16 + g, d = d0 + 8 * h + 2 * t;
-                    if (a < L.k1k) *reinterpret_cast<uint2 *>(Ys + (size_t)a * L.yp + d) = make_uint2(tm_tf32(acc[mt][h][0]), tm_tf32(acc[mt][h][1]));
-                    if (a + 8 < L.k1k) *reinterpret_cast<uint2 *>(Ys + (size_t)(a + 8) * L.yp + d) = make_uint2(tm_tf32(acc[mt][h][2]), tm_tf32(acc[mt][h][3]));
-                }
-        }
-        __syncthreads();
+                    for (int i = 0; i < TERMS; ++i) yb[p][at][h][i] = tm_term(y[p][at][2 * h], y[p][at][2 * h + 1]);
         // ---- X'[c][d] = sum_a P1[a][c] Y[a][d]
-        for (int item = warp; item < 2 * npairs; item += TM_WARPS) {
-            const int pr = item >> 1, mt0 = (item & 1) * MG;
-            float acc[MG][2][4];
+        for (int ct = ct0; ct < ct1; ++ct) {
+            float acc[DW][2][4];
 #pragma unroll
-            for (int mt = 0; mt < MG; ++mt)
+            for (int p = 0; p < DW; ++p)
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
+                for (int i = 0; i < 8; ++i) acc[p][i >> 2][i & 3] = 0.f;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[mt][h][i] = 0.f;
-            const int d0 = pr * 16;
-            for (int kk = 0; kk < L.k1k; kk += 8) {
-                uint32_t b0[2], b1[2];
+            for (int k = 0; k < NA / 2; ++k) {
+                uint4 w[TERMS];
+                float step[DW][2][4] = {};
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    b0[h] = Ys[(size_t)(kk + t) * L.yp + d0 + 8 * h + g];
-                    b1[h] = Ys[(size_t)(kk + t + 4) * L.yp + d0 + 8 * h + g];
-                }
+                for (int i = 0; i < TERMS; ++i) w[i] = A1[(size_t)((ct * (NA / 2) + k) * TERMS + i) * 32];
 #pragma unroll
-                for (int mt = 0; mt < MG; ++mt) {
-                    if (mt0 + mt < MT) {
-                        // A[c][a] = P1[a][c]: element (row c = 16 mt + g (+8), column a = kk + t (+4))
-                        const uint32_t *pa = P1s + (size_t)(kk + t) * L.p1p + (mt0 + mt) * 16 + g;
-                        const uint32_t a0 = pa[0], a1 = pa[8], a2 = pa[4 * L.p1p], a3 = pa[4 * L.p1p + 8];
+                for (int i = TERMS - 1; i >= 0; --i)     // term i of P1 with the terms of Y that leave 8 TERMS bits
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) tm_mma(acc[mt][h], a0, a1, a2, a3, b0[h], b1[h]);
-                    }
-                }
+                    for (int j = TERMS - 1 - i; j >= 0; --j)
+#pragma unroll
+                        for (int p = 0; p < DW; ++p)
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) tm_mma(part(step[p][h], acc[p][h]), w[i], yb[p][2 * k][h][j], yb[p][2 * k + 1][h][j]);
+                if (TERMS > 2)
+#pragma unroll
+                    for (int p = 0; p < DW; ++p)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) acc[p][i >> 2][i & 3] += step[p][i >> 2][i & 3];
             }
 #pragma unroll
-            for (int mt = 0; mt < MG; ++mt)
+            for (int p = 0; p < DW; ++p)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int c = (mt0 + mt) * 16 + g, d = d0 + 8 * h + 2 * t;
-                    if (c < k1) {
-                        store_from_float(xt, out_dt, row + (size_t)c * k2 + d, acc[mt][h][0]);
-                        store_from_float(xt, out_dt, row + (size_t)c * k2 + d + 1, acc[mt][h][1]);
-                    }
-                    if (c + 8 < k1) {
-                        store_from_float(xt, out_dt, row + (size_t)(c + 8) * k2 + d, acc[mt][h][2]);
-                        store_from_float(xt, out_dt, row + (size_t)(c + 8) * k2 + d + 1, acc[mt][h][3]);
+                    const int c = 16 * ct + g + 8 * h;
+                    if (c < k1 && (DW == 1 || d0 + 16 * p < k2)) {
+                        const size_t o = (size_t)m * K + (size_t)c * k2 + d0 + 16 * p + 4 * t;
+                        const float4 r = make_float4(acc[p][0][2 * h], acc[p][0][2 * h + 1], acc[p][1][2 * h], acc[p][1][2 * h + 1]);
+                        if (out_dt == BTC_F32) *reinterpret_cast<float4 *>(reinterpret_cast<float *>(xt) + o) = r;
+                        else if (out_dt == BTC_BF16) *reinterpret_cast<uint2 *>(reinterpret_cast<uint16_t *>(xt) + o) = make_uint2(tm_pack(r.x, r.y), tm_pack(r.z, r.w));
+                        else {
+                            const __half2 lo = __floats2half2_rn(r.x, r.y), hi = __floats2half2_rn(r.z, r.w);
+                            *reinterpret_cast<uint2 *>(reinterpret_cast<uint16_t *>(xt) + o) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+                        }
                     }
                 }
         }
     }
 }
 
-template <int MT, int TK1 = 0, int TK2 = 0>
-static int launch_transform_mma(const void *x, int x_dt, const btc_transform &T, void *xt, int out_dt, int M, size_t smem, cudaStream_t s)
+template <int NA, int TERMS, bool F16, int K2, int DW>
+static int launch_transform_mma(const void *x, const btc_transform &T, void *xt, int out_dt, int M, cudaStream_t s)
 {
-    auto kern = transform_mma_kernel<MT, TK1, TK2>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = transform_mma_kernel<NA, TERMS, F16, K2, DW>;
+    const int ks2 = T.k2 / 16, slices = (ks2 + DW - 1) / DW, nc = (T.k1 + 15) / 16;
+    // Shares of c: as long as every quadrant of every SM gets at most one warp (each share computes Y again).  Slices per CTA:
+    // as many as there are warps left, so that they read the same rows of x.
+    const long long items = (long long)M * slices;
+    int cg = 1;
+    while (cg < 4 && 2 * cg <= nc && items * 2 * cg <= 4 * 148) cg *= 2;
+    const int warps = items * cg <= 4 * 148 ? 4 : TM_WARPS;
+    TmPlan p;
+    p.cg = cg;
+    p.ds = 1;
+    while (2 * p.ds <= warps / cg && p.ds < slices) p.ds *= 2;
+    size_t smem;
+    for (;; p.ds /= 2) {
+        p.p2_frags = p.ds * DW * ks2;
+        p.mask_off = (p.p2_frags + nc * (NA / 2)) * TERMS * 512;
+        smem = p.mask_off + (size_t)NA * ks2 * 256;
+        if (smem <= 227u * 1024u) break;
+        if (p.ds == 1) return BTC_ERR_UNSUPPORTED;
+    }
+    p.rw = warps / (cg * p.ds);
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (dev >= 64 || !((done.load(std::memory_order_relaxed) >> dev) & 1u)) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return cuda_fail(e);
+        if (dev < 64) done.fetch_or(uint64_t(1) << dev, std::memory_order_relaxed);
+    }
+    // as many CTAs as the SMs hold at once, each taking rows in turn
+    const int gy = (slices + p.ds - 1) / p.ds;
+    int gx = (M + p.rw - 1) / p.rw, most = 148 / gy;
+    if (most < 1) most = 1;
+    if (gx > most) gx = most;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(M < sms ? M : sms));
-    cfg.blockDim = dim3(TM_THREADS);
+    cfg.gridDim = dim3((unsigned)gx, (unsigned)gy);
+    cfg.blockDim = dim3(warps * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, x, x_dt, T.sigma_bits, T.P1, T.P2, T.k1, T.k2, xt, out_dt, M);
+    e = cudaLaunchKernelEx(&cfg, kern, static_cast<const uint16_t *>(x), T.sigma_bits, T.P1, T.P2, T.k1, T.k2, xt, out_dt, M, p);
     return e == cudaSuccess ? BTC_OK : cuda_fail(e);
+}
+
+template <int TERMS, bool F16, int K2, int DW>
+static int launch_transform_k2(const void *x, const btc_transform &T, void *xt, int out_dt, int M, cudaStream_t s)
+{
+    if (T.k1 <= 16) return launch_transform_mma<2, TERMS, F16, K2, DW>(x, T, xt, out_dt, M, s);
+    if (T.k1 <= 32) return launch_transform_mma<4, TERMS, F16, K2, DW>(x, T, xt, out_dt, M, s);
+    if (T.k1 <= 48) return launch_transform_mma<6, TERMS, F16, K2, DW>(x, T, xt, out_dt, M, s);
+    if (T.k1 <= 64) return launch_transform_mma<8, TERMS, F16, K2, DW>(x, T, xt, out_dt, M, s);
+    if (T.k1 <= 96) return launch_transform_mma<12, TERMS, F16, K2, DW>(x, T, xt, out_dt, M, s);
+    return launch_transform_mma<16, TERMS, F16, K2, DW>(x, T, xt, out_dt, M, s);
+}
+
+// Slices of 32 columns (half the instructions per product) where they give every quadrant of every SM more than one warp,
+// else slices of 16: 86 x 128 at 200 rows, with a 2048-wide layer behind it, 38.9 -> 35.3 us, but at 130 rows 33.5 -> 37.5.
+template <int TERMS, bool F16>
+static int launch_transform_terms(const void *x, const btc_transform &T, void *xt, int out_dt, int M, cudaStream_t s)
+{
+    if constexpr (TERMS == 2) {
+        const bool wide = (long long)M * (T.k2 / 32) > 4 * 148;
+        if (wide && T.k2 == 64) return launch_transform_k2<TERMS, F16, 64, 2>(x, T, xt, out_dt, M, s);
+        if (wide && T.k2 == 128) return launch_transform_k2<TERMS, F16, 128, 2>(x, T, xt, out_dt, M, s);
+    }
+    if (T.k2 == 64) return launch_transform_k2<TERMS, F16, 64, 1>(x, T, xt, out_dt, M, s);
+    if (T.k2 == 128) return launch_transform_k2<TERMS, F16, 128, 1>(x, T, xt, out_dt, M, s);
+    return launch_transform_k2<TERMS, F16, 0, 1>(x, T, xt, out_dt, M, s);
 }
 
 int launch_transform(const void *x, int x_dt, const btc_transform &T, void *xt, int out_dt, int M, int K, cudaStream_t s)
 {
     if ((long long)T.k1 * T.k2 != K) return BTC_ERR_SHAPE;
-    // many rows: the tensor-core form, when the factors fit shared memory beside one row (k2 a multiple of 16)
-    if (M >= 64 && x_dt != BTC_F32 && T.k2 % 16 == 0 && T.k1 <= 128 && K <= 8 * 8 * TM_THREADS) {
-        const size_t bytes = tm_layout(T.k1, T.k2).words * sizeof(uint32_t);
-        if (bytes <= 227u * 1024u) {
-            const int mt = (T.k1 + 15) / 16;
-            // the factor shapes of the LLaMA-2-7B widths (4096 = 64 x 64, 11008 = 86 x 128) have instantiations of their own
-            if (T.k1 == 64 && T.k2 == 64) return launch_transform_mma<4, 64, 64>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            if (T.k1 == 86 && T.k2 == 128) return launch_transform_mma<6, 86, 128>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            switch (mt) {
-            case 1: return launch_transform_mma<1>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            case 2: return launch_transform_mma<2>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            case 3: return launch_transform_mma<3>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            case 4: return launch_transform_mma<4>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            case 5: return launch_transform_mma<5>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            case 6: return launch_transform_mma<6>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            case 7: return launch_transform_mma<7>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            default: return launch_transform_mma<8>(x, x_dt, T, xt, out_dt, M, bytes, s);
-            }
-        }
+    // (up to 8 rows the fp32 form above, a slab of eight columns per CTA, has the shorter chain: 4.3 us at 64 x 64, one row, where
+    // this one took 4.9.  Below 64 rows three terms: the precision of the fp32 form; above, two carry more than 16-bit x.)
+    if (x_dt != BTC_F32 && M > 8 && T.k2 % 16 == 0 && T.k1 <= 128) {
+        const bool f16 = x_dt == BTC_F16;
+        const int rc = M >= 64 ? (f16 ? launch_transform_terms<2, true>(x, T, xt, out_dt, M, s) : launch_transform_terms<2, false>(x, T, xt, out_dt, M, s))
+                               : (f16 ? launch_transform_terms<3, true>(x, T, xt, out_dt, M, s) : launch_transform_terms<3, false>(x, T, xt, out_dt, M, s));
+        if (rc != BTC_ERR_UNSUPPORTED) return rc;
     }
     const size_t smem = ((size_t)K + 4 * T.k1 + 4 + (size_t)T.k2 * TR_DT + (size_t)T.k1 * TR_DT + (size_t)T.k1 * (T.k1 + 8)) * sizeof(float);
     if (smem > 200 * 1024) return BTC_ERR_UNSUPPORTED;

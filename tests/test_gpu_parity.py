@@ -527,6 +527,30 @@ def test_activation_transform_many_rows(M, k1, k2, xdt):
     assert btc.device_status() == 0
 
 
+@pytest.mark.parametrize("M,k1,k2,xdt", [(9, 1, 16, "f16"), (10, 128, 128, "bf16"), (63, 17, 48, "f16"), (33, 65, 128, "f16"), (64, 16, 64, "f16"), (65, 33, 80, "bf16"),
+                                         (200, 97, 128, "f16"), (1200, 16, 64, "bf16"), (601, 30, 64, "f16"), (150, 49, 128, "bf16"), (70, 8, 256, "bf16"), (11, 5, 512, "f16")])
+def test_activation_transform_edges(M, k1, k2, xdt):
+    """Row counts on both sides of the change of form and of slice width, factors that fill no tile: fp32 results to 1e-6 of the
+    row's largest |x'| below 64 rows, to 2^-14 above."""
+    K = k1 * k2
+    rng = np.random.default_rng(k1 + k2 + M)
+    dt = torch.float16 if xdt == "f16" else torch.bfloat16
+    x = torch.from_numpy(rng.standard_normal((M, K)).astype(np.float32)).to(dt)
+    sigma = rng.choice(np.array([-1, 1], dtype=np.int8), size=K)
+    P1, P2 = (rng.standard_normal((k, k)).astype(np.float32) / np.float32(k ** 0.5) for k in (k1, k2))
+    bits = np.zeros((K + 31) // 32, dtype=np.uint32)
+    for i in np.nonzero(sigma < 0)[0]:
+        bits[i >> 5] |= np.uint32(1) << np.uint32(i & 31)
+    tr = tuple(torch.from_numpy(a).cuda() for a in (bits.view(np.int32), P1, P2))
+    xt, xt16 = btc.activation_transform(x.cuda(), tr), btc.activation_transform(x.cuda(), tr, out_dtype=dt)
+    X = x.double().numpy().reshape(M, k1, k2) * sigma.reshape(k1, k2)
+    ref = np.einsum("ac,mad->mcd", P1.astype(np.float64), X @ P2.astype(np.float64)).reshape(M, K)
+    tol = (1e-6 if M < 64 else 2.0 ** -14) * np.abs(ref).max(axis=1, keepdims=True)
+    assert (np.abs(xt.double().cpu().numpy() - ref) <= tol).all()
+    ulp = 2.0 ** -11 if xdt == "f16" else 2.0 ** -8
+    assert (np.abs(xt16.double().cpu().numpy() - ref) <= tol + ulp * np.abs(ref) + 1e-7).all()
+
+
 def test_online_transform_full_size_M512():
     """The transform in front of the 4096 x 4096 config-4 layer at M = 512 (K = 64 x 64: the tensor-core form of the
     transform, then the tensor-core layer kernel), as the benchmark times it: six rows of x spread over the row tiles,
