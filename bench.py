@@ -40,7 +40,7 @@ WORKLOAD = "config 2: LLaMA-2-7B decode layer set (7 projections, v=16, Kc=8192)
 # profiles/decode_step_traffic.json, which also holds the SHA-256 of the kernel source it was taken on; when the source
 # has changed since, the figure no longer describes the kernel that is timed and `traffic` is reported as null.
 TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "decode_step_traffic.json")
-KERNEL_SOURCE = os.path.join(ROOT, "paper_2506_12040_b200", "csrc", "gemv_imma_wide.cu")
+KERNEL_SOURCE = os.path.join(ROOT, "paper_2506_12040_b200", "csrc", "gemv.cuh")
 
 
 def kernel_source_sha256() -> str:
@@ -774,7 +774,7 @@ def run_gpu(args):
         peak = peaks["hbm_gbs"]
         traffic, traffic_note = recorded_traffic()
         workload = WORKLOAD
-        kernel_name = "wide::gemv_imma_kernel<4,1,1> (integer form, one CTA per SM; 7 layers per launch)"
+        kernel_name = "gemv_kernel (integer form, 16-bit table, two CTAs per SM; 7 layers per launch)"
         if custom:
             traffic, traffic_note = None, "no counters were taken for this workload"
             workload = (f"config {args.config}: {len(specs)} layers, v={specs[0].v}, Kc={specs[0].Kc}, M={HM}, base seed {cfg['seed']}"

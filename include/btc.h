@@ -137,21 +137,16 @@ BTC_API int btc_codebook_kmeans(const uint32_t *vecs, size_t n, int v, int Kc, i
  *   y        [M, N] row-major, y_dtype = BTC_F32 (also BTC_F16 / BTC_BF16, rounded to nearest)
  *   workspace / workspace_bytes: scratch of at least btc_linear_workspace_bytes(...) bytes,
  *            256-byte aligned; may be NULL when that function returns 0.  Contents are
- *            undefined afterwards; concurrent calls need distinct workspaces.  For a layer with
- *            few 128-row tiles and a long K (v = 16) the size includes room for the partial sums
- *            of a K split over the idle SMs, added in a fixed order by a second small kernel.
+ *            undefined afterwards; concurrent calls need distinct workspaces.
  *
  * btc_linear_gemv: the decode path, 1 <= M <= 8, built on the identity <x, c> = 2 * sum_{bit=1} x - sum x.
- *   M <= 2: x is quantised per K-slice to a block-fixed-point integer (2^-20 of the slice's largest magnitude
- *   for v = 16), the sums over set bits are exact integer sums on the warp-level int8 MMA, recombined and added
- *   over the slices in fp32.  M = 3..8: masked codeword bits act as fp16 numbers on the warp-level fp16 MMA with
- *   fp32 accumulation (one layer per call runs on an older kernel of the same arithmetic, a CTA per row tile; the
- *   fused multi-layer launch of btc_linear_gemv_batch on a newer one).  With v = 16, at most 74 tiles of 128 rows and a workspace of the size
- *   btc_linear_workspace_bytes asks for, M = 5..8 at K >= 8192 and M = 6..8 at K >= 4096 go to the tensor-core launch
- *   of btc_linear_gemm with K split over the SMs instead (it is the faster one there).  All stay well inside a
- *   relative error of 2e-3 against the exact product.  Shapes outside what these kernels cover (v not a multiple
- *   of 4 or above 20, K/v not a multiple of 8) run on slower general kernels with the same result.
- * btc_linear_gemm: any M >= 1, built for M >= 128: index tiles are decoded to +-1 bf16 (fp16 for fp16 x) tiles
+ *   M <= 2 and v a multiple of 4 from 8 to 20: x is quantised per K-slice to a block-fixed-point integer (2^-20 of the
+ *   slice's largest magnitude for v = 16), the sums over set bits are exact integer sums on the warp-level int8 MMA,
+ *   recombined and added over the slices in fp32.  Otherwise (M <= 8, v even up to 24): masked codeword bits act as fp16
+ *   numbers on the warp-level fp16 MMA with fp32 accumulation.  Both stay well inside a relative error of 2e-3 against the
+ *   exact product.  Shapes outside (odd v, v above 24, K/v not a multiple of 8) run on slower general kernels with the same
+ *   result.
+ * btc_linear_gemm: any M >= 1, built for M > 8: index tiles are decoded to +-1 bf16 (fp16 for fp16 x) tiles
  *   and multiplied on the tcgen05 tensor cores with fp32 accumulation in tensor memory; alpha (and mu) are
  *   applied in fp32 in the epilogue.  M <= 8 is forwarded to the decode path.
  * Errors: NULL / SHAPE / ALIGN / UNSUPPORTED / WORKSPACE as above; BTC_ERR_CUDA if a launch
