@@ -333,8 +333,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams
 //
 // Launched with programmatic stream serialisation: barriers, tensor memory, table and first indices are ready before
 // the predecessor has finished; x is read after it (or right away where the predecessor is the row-sum kernel, which
-// itself waited for it; then the epilogue waits).  It does not let its own successors start early: their CTAs
-// would pile up on the SMs that a round of tiles leaves idle (a transform behind it ran 15 us longer).
+// itself waited for it; then the epilogue waits).  Its own successors may start early (a transform
+// behind it: 13.0 -> 10.5 us for 24 rows, K = 1024), but not with a mean term: the next call's row sums, small CTAs, would pile up
+// on the SMs that a round of tiles leaves idle (9.0 -> 9.8 us for 16 rows of 4096 x 4096).
 constexpr int G2_DWARPS = 16;                    // decode warps (four groups of four)
 constexpr int G2_THREADS = 128 + G2_DWARPS * 32;
 constexpr uint32_t G2_IDX_BYTES = 128 * 128;     // one index tile
@@ -466,6 +467,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_d = *s_tmem;
+    if (!p.sumx) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == 0) {
         if (lane == 0) {
@@ -680,11 +682,12 @@ static int launch_cfg(const CUtensorMap &tm, const GemmParams &p, cudaStream_t s
 }
 
 // Tiling of a (M, N, K) problem: rows of x per tile (bn), tiles of x, K splits (whole index tiles, clusters of up to eight).
-// Time under a wave model, in clocks, fitted to measurements: a CTA per SM in rounds (the last one shorter when it is not
-// full: less traffic, higher clocks), each a start-up (launch, tensor memory, first tiles, epilogue) and its k steps.  A step
-// costs the MMAs' and the x tile's time, 260 + 1.55 clk per row of x, and no less than the decode of its weights: 350
-// clk for v = 16, about 33 more per block a step touches otherwise.  Codewords gathered from L1 / L2 (table too large for
-// shared memory) share that path with the x tiles: 650 clk + 1 per row.  A split adds the sum over the cluster.
+// Time in clocks, fitted to measurements of every width at K = 2000 and 4096: a CTA per SM in rounds, the last one as long as the
+// others, each a fixed part (launch, tensor memory, first tiles, epilogue) and its k steps.  A step of tiles up to 128 wide
+// costs what their MMAs and x tiles cost or the decode of its weights; wider ones have one issuing thread, which paces
+// them whatever their width: 11008 x 4096 at 300 rows takes 53 us as two tiles of 160 and 36 as three of 112.  Codewords
+// gathered from L1 / L2 (table too large for shared memory) share that path with the x tiles.  A split adds the sum over the
+// cluster.
 struct GemmPlan { int bn, mt, splits, split_tiles; };
 
 static bool gemm_table_fits(int bn, int Kc)
@@ -697,25 +700,24 @@ static GemmPlan gemm_plan(int M, int N, int K, int v, int Kc)
 {
     const int k_tiles = (K + G_BK - 1) / G_BK, rows = (N + G_BN - 1) / G_BN;
     const int idx_tiles = (k_tiles + v - 1) / v;
-    const double decode = v == 16 ? 350.0 : v == 8 ? 410.0 : 300.0 + 33.0 * step_blocks(v);
+    const double decode = v == 16 ? 330.0 : v == 8 ? 430.0 : 350.0 + 20.0 * step_blocks(v);
     GemmPlan best = {0, 0, 1, k_tiles};
     double best_t = 0;
     for (int mt = (M + 255) / 256; mt <= (M + 255) / 256 + (M + 127) / 128; ++mt) {
         int bn = ((M + mt - 1) / mt + 15) / 16 * 16;
         if (bn < 16) bn = 16;
         const int mtn = (M + bn - 1) / bn;
-        const double mma = 260.0 + 1.55 * bn, fit = mma > decode ? mma : decode;
-        const double step = gemm_table_fits(bn, Kc) ? fit : 650.0 + bn > fit ? 650.0 + bn : fit;
+        const bool wide = bn > 128;
+        const double mma = 200.0 + 1.6 * bn, fit = wide ? decode + 230.0 : mma > decode ? mma : decode;
+        const double far = wide ? 400.0 + 2.3 * bn : 480.0 + 2.2 * bn, step = gemm_table_fits(bn, Kc) || far < fit ? fit : far;
         for (int sp = 1; sp <= 8 && sp <= idx_tiles; ++sp) {
             const int per = (idx_tiles + sp - 1) / sp;                 // index tiles per split
             const int n = (idx_tiles + per - 1) / per;
             if (n != sp) continue;
             const long long ctas = (long long)rows * mtn * sp;
             const int at_once = sp == 1 ? 148 : 136 / sp * sp;         // (clusters do not fill every GPC)
-            const int rest = (int)(ctas % at_once);
-            const double waves = (double)(ctas / at_once) + (rest ? (ctas < at_once ? 1.0 : 0.45 + 0.55 * rest / at_once) : 0.0);
             const int steps = per * v < k_tiles ? per * v : k_tiles;
-            const double t = waves * (5500.0 + 4.0 * bn + steps * step + (sp > 1 ? 3500.0 + 20.0 * bn : 0.0));
+            const double t = (double)((ctas + at_once - 1) / at_once) * ((wide ? 16000.0 : 11000.0) + steps * step + (sp > 1 ? 3500.0 + 20.0 * bn : 0.0));
             if (best.bn == 0 || t < best_t) { best = {bn, mtn, sp, per * v}; best_t = t; }
         }
         if (M <= 256 && bn <= 32) break;
