@@ -20,13 +20,14 @@
 //              key(p) = min(key(p), key(p ^ 2^b) + (1, 0)).  v 2^v steps instead of distinct patterns x centroids (1 M
 //              instead of 487 M for a 4096 x 4096 layer at v = 16 with 8192 centroids).  The low nine bits within 512
 //              neighbouring patterns, the others on columns of four, with a grid barrier between.
-//   M-step     every occurring pattern adds cnt[p] to its cluster's total and to the counts of its set bits, several counts
-//              to a 64-bit atomic; then one thread per centroid
+//   M-step     every occurring pattern whose cluster is another than in the round before moves cnt[p] (total and counts of
+//              its set bits, several counts to a 64-bit atomic) from that one's votes to the new one's, so that later rounds
+//              cast few votes and the one that finds nothing changed none; then one thread per centroid
 //   assign     z through the label table in shared memory (v <= 16)
-// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 66 us a call (706 us with an E-step over (pattern,
-// centroid) pairs, a kernel per step and max_iter rounds of launches, of which those after convergence returned at once).
-// Of these ten grid barriers at 1.1 to 1.5 us, clearing and histogram 8 us, ranking 10 us, an E-step 3 + 6 us (half of it
-// the votes' atomics), an M-step 4 us, assignment 4 us.
+// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 60.2 us a call (67.7 us with all votes cast anew in
+// every round, a barrier between clearing the frequencies and the histogram, and two bytes to a store of assignments).
+// Of these nine grid barriers at 1.1 to 1.5 us, histogram 8 us, ranking 10 us, an E-step 3 + 3 us and in the first round as much
+// again for the votes' atomics, an M-step 4 us, assignment 4 us.
 // Integer arithmetic only; results are bit-exact against the definition.
 #include <cuda.h>
 #include <atomic>
@@ -48,7 +49,7 @@ static_assert((1 << KM_VMAX) / KM_PART <= KM_MAX_CTAS && (KM_BINS + 1 + KM_PART)
 
 __device__ int g_km_status = 0;
 
-struct KmState {                             // zeroed by the host
+struct KmState {                             // zeroed by the host, with the frequencies that follow it
     unsigned arrived;     // grid barrier
     int changed[2];       // set by the E-step of round i in slot i & 1
     int n_over;           // patterns whose frequency is past the last bin
@@ -129,9 +130,9 @@ __device__ __forceinline__ bool km_sync(KmState *st, unsigned &target, int *s_ok
     return *s_ok != 0;
 }
 
-// f(word) for every vector of [begin, end): 16-byte loads, four in flight.
-template <typename F>
-__device__ __forceinline__ void km_stream(const uint32_t *__restrict__ vecs, size_t begin, size_t end, F f)
+// f(i, word) for every vector of [begin, end), or f4(i, four words) for four neighbours: 16-byte loads, four in flight.
+template <typename F, typename F4>
+__device__ __forceinline__ void km_stream(const uint32_t *__restrict__ vecs, size_t begin, size_t end, F f, F4 f4)
 {
     if ((reinterpret_cast<uintptr_t>(vecs) & 15u) == 0) {   // (begin is a multiple of 4)
         const uint4 *src = reinterpret_cast<const uint4 *>(vecs);
@@ -146,12 +147,18 @@ __device__ __forceinline__ void km_stream(const uint32_t *__restrict__ vecs, siz
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const size_t q = q0 + threadIdx.x + u * KM_THREADS;
-                if (q < q1) { f(4 * q, w[u].x); f(4 * q + 1, w[u].y); f(4 * q + 2, w[u].z); f(4 * q + 3, w[u].w); }
+                if (q < q1) f4(4 * q, w[u]);
             }
         }
         begin = end & ~(size_t)3;
     }
     for (size_t i = begin + threadIdx.x; i < end; i += KM_THREADS) f(i, __ldg(vecs + i));
+}
+
+template <typename F>
+__device__ __forceinline__ void km_stream(const uint32_t *__restrict__ vecs, size_t begin, size_t end, F f)
+{
+    km_stream(vecs, begin, end, f, [&](size_t i, const uint4 &w) { f(i, w.x); f(i + 1, w.y); f(i + 2, w.z); f(i + 3, w.w); });
 }
 
 __global__ void __launch_bounds__(KM_THREADS, 1)
@@ -167,8 +174,8 @@ km_kernel(const KmArgs a)
     const int gid = b * KM_THREADS + tid, gthreads = G * KM_THREADS;
     unsigned target = 0;
 
-    // ---- clear what the later steps add to
-    for (int i = gid; i < P; i += gthreads) { a.cnt[i] = 0u; a.seed[i] = KM_NONE; }
+    // ---- clear what the steps after the next barrier add to (the frequencies and the state arrive cleared)
+    for (int i = gid; i < P; i += gthreads) a.seed[i] = KM_NONE;
     for (int i = gid; i < KM_BINS; i += gthreads) a.bins[i] = 0u;
     for (int i = gid; i < Kc; i += gthreads) a.C[i] = 0u;
     for (int i = gid; i < KM_BINS * KM_MAX_CTAS / 8; i += gthreads) reinterpret_cast<uint4 *>(a.cols)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -181,11 +188,9 @@ km_kernel(const KmArgs a)
         const int hw = max(P / 2, 1);
         for (int i = tid; i < hw; i += KM_THREADS) sm[i] = 0u;
         constexpr size_t MOST = 65532;                       // (16-bit counters; a multiple of 4)
-        bool cleared = false;
-        for (size_t c0 = v0; c0 < v1 || !cleared; c0 += MOST) {
+        for (size_t c0 = v0; c0 < v1; c0 += MOST) {
             __syncthreads();
-            if (c0 < v1) km_stream(a.vecs, c0, min(v1, c0 + MOST), [&](size_t, uint32_t w) { w &= mask; atomicAdd(sm + (w >> 1), 1u << (16 * (w & 1u))); });
-            if (!cleared) { if (!km_sync(a.st, target, &s_ok)) return; cleared = true; }   // (everybody's counters are clear)
+            km_stream(a.vecs, c0, min(v1, c0 + MOST), [&](size_t, uint32_t w) { w &= mask; atomicAdd(sm + (w >> 1), 1u << (16 * (w & 1u))); });
             __syncthreads();
             for (int i = tid; i < hw; i += KM_THREADS) {
                 const uint32_t w = sm[i];
@@ -195,7 +200,6 @@ km_kernel(const KmArgs a)
             }
         }
     } else {
-        if (!km_sync(a.st, target, &s_ok)) return;
         km_stream(a.vecs, v0, v1, [&](size_t, uint32_t w) { atomicAdd(a.cnt + (w & mask), 1u); });
     }
     if (!km_sync(a.st, target, &s_ok)) return;
@@ -339,9 +343,11 @@ km_kernel(const KmArgs a)
                 const uint32_t c = __ldcg(a.cnt + p);
                 if (!c) continue;
                 const uint32_t z = sm[e] & 0xffffu;
-                if (it == 0 || a.label[p] != z) changed = 1; // (this thread wrote it in the round before)
+                const uint32_t was = it == 0 ? KM_NONE : a.label[p];         // (this thread wrote it in the round before)
+                if (was == z) continue;                      // its votes stand
+                changed = 1;
                 a.label[p] = (uint16_t)z;
-                unsigned long long *vote = a.votes + (size_t)z * a.words;
+                unsigned long long *vote = a.votes + (size_t)z * a.words, *old = a.votes + (size_t)was * a.words;
                 const int bits = a.fields == 3 ? 21 : 32;
                 uint32_t pat = ((uint32_t)p << 1) | 1u;      // count 0: the total; count 1 + t: element t is +1
                 for (int w = 0; w < a.words; ++w) {
@@ -350,7 +356,9 @@ km_kernel(const KmArgs a)
                         if (pat & 1u) add |= (unsigned long long)c << (bits * f);
                         pat >>= 1;
                     }
-                    if (add) atomicAdd(vote + w, add);
+                    if (!add) continue;
+                    atomicAdd(vote + w, add);
+                    if (it) atomicAdd(old + w, 0ull - add);  // (borrows between the counts of a word cancel in its total)
                 }
             }
         }
@@ -364,7 +372,8 @@ km_kernel(const KmArgs a)
         const int bits = a.fields == 3 ? 21 : 32;
         const unsigned long long fmask = (1ull << bits) - 1ull;
         for (int k = tid * G + b; k < kc; k += gthreads) {               // (spread over the SMs)
-            unsigned long long *vote = a.votes + (size_t)k * a.words, x[KM_MAX_WORDS];
+            const unsigned long long *vote = a.votes + (size_t)k * a.words;
+            unsigned long long x[KM_MAX_WORDS];
 #pragma unroll
             for (int w = 0; w < KM_MAX_WORDS; ++w)
                 if (w < a.words) x[w] = __ldcg(vote + w);
@@ -374,7 +383,6 @@ km_kernel(const KmArgs a)
 #pragma unroll
             for (int w = 0; w < KM_MAX_WORDS; ++w)
                 if (w < a.words) {
-                    vote[w] = 0ull;
                     for (int f = 0; f < a.fields; ++f, ++bit) {
                         const uint32_t o = (uint32_t)(x[w] & fmask);
                         x[w] >>= bits;
@@ -398,7 +406,13 @@ km_kernel(const KmArgs a)
             tab[tid] = __ldcg(a.label + tid);
         }
         __syncthreads();
-        km_stream(a.vecs, v0, v1, [&](size_t i, uint32_t w) { a.z[i] = tab[w & mask]; });
+        auto one = [&](size_t i, uint32_t w) { a.z[i] = tab[w & mask]; };
+        if ((reinterpret_cast<uintptr_t>(a.z) & 7u) == 0)    // four assignments to a store
+            km_stream(a.vecs, v0, v1, one, [&](size_t i, const uint4 &w) {
+                *reinterpret_cast<uint2 *>(a.z + i) = make_uint2(tab[w.x & mask] | (uint32_t)tab[w.y & mask] << 16, tab[w.z & mask] | (uint32_t)tab[w.w & mask] << 16);
+            });
+        else
+            km_stream(a.vecs, v0, v1, one);
     } else {
         km_stream(a.vecs, v0, v1, [&](size_t i, uint32_t w) { a.z[i] = __ldcg(a.label + (w & mask)); });
     }
@@ -493,7 +507,7 @@ extern "C" BTC_API int btc_codebook_kmeans(const uint32_t *vecs, size_t n, int v
     const size_t want = (n + 1023) / 1024 > (size_t)((1 << v) + 511) / 512 ? (n + 1023) / 1024 : (size_t)((1 << v) + 511) / 512;
     int grid = want < (size_t)sms ? (int)want : sms;
     const int parts = ((1 << v) + KM_PART - 1) / KM_PART;
-    e = cudaMemsetAsync(a.st, 0, sizeof(KmState), s);
+    e = cudaMemsetAsync(a.st, 0, km_align(sizeof(KmState)) + ((size_t)4 << v), s);
     if (e != cudaSuccess) return cuda_fail(e);
     void *params[] = {&a};
     for (;;) {
