@@ -134,7 +134,7 @@ __device__ __forceinline__ bool km_sync(KmState *st, unsigned &target, int *s_ok
 template <typename F, typename F4>
 __device__ __forceinline__ void km_stream(const uint32_t *__restrict__ vecs, size_t begin, size_t end, F f, F4 f4)
 {
-    if ((reinterpret_cast<uintptr_t>(vecs) & 15u) == 0) {   // (begin is a multiple of 4)
+    if ((reinterpret_cast<uintptr_t>(vecs) & 15u) == 0) {   // (begin is a multiple of 4, or the end)
         const uint4 *src = reinterpret_cast<const uint4 *>(vecs);
         const size_t q1 = end / 4;
         for (size_t q0 = begin / 4; q0 < q1; q0 += 4 * KM_THREADS) {
@@ -150,7 +150,7 @@ __device__ __forceinline__ void km_stream(const uint32_t *__restrict__ vecs, siz
                 if (q < q1) f4(4 * q, w[u]);
             }
         }
-        begin = end & ~(size_t)3;
+        begin = max(begin, end & ~(size_t)3);                // (an empty share may start inside the last four)
     }
     for (size_t i = begin + threadIdx.x; i < end; i += KM_THREADS) f(i, __ldg(vecs + i));
 }

@@ -88,6 +88,16 @@ def test_kmeans_edges(n, v, Kc, offset):
     assert btc.device_status() == 0
 
 
+@pytest.mark.parametrize("n,v,Kc,kind", [(6001, 18, 40, "iid"), (6003, 17, 200, "noisy"), (149, 20, 20, "iid")])
+def test_kmeans_shares_past_the_end(n, v, Kc, kind):
+    """More CTAs than shares of vectors, and a number of vectors that four does not divide: the last ones are counted once."""
+    B = _vectors(n, v, kind, seed=n + v)
+    C_ref, z_ref, iters_ref, n_unique, converged = km.optimize_codebook(B, Kc, 6, with_flag=True)
+    C, z, info = _run(B, v, Kc, 6)
+    assert info.tolist() == [iters_ref, min(Kc, n_unique), n_unique, int(converged)]
+    assert np.array_equal(C[:info[1]], km.pack_words(C_ref)) and np.array_equal(z.astype(np.int64), z_ref)
+
+
 def test_kmeans_feeds_the_layer():
     """The construction's outputs are the layer's inputs: centroids -> btc_codebook_pack, z -> idx; decoding them
     gives the nearest-centroid approximation of the sign matrix, whose Hamming error equals the oracle's objective."""
