@@ -88,6 +88,30 @@ def test_kmeans_edges(n, v, Kc, offset):
     assert btc.device_status() == 0
 
 
+@pytest.mark.parametrize("n,v,Kc,kind,repeat,z_off", [(2000, 12, 20, "iid", 1, 0), (2000, 12, 20, "iid", 1049, 3), (70003, 16, 40, "noisy", 1, 1),
+                                                      (6001, 18, 40, "iid", 1, 2), (50001, 2, 3, "noisy", 1, 4)])
+def test_kmeans_votes_move_over_rounds(n, v, Kc, kind, repeat, z_off):
+    """Three and four rounds, with votes carried from one to the next in counts of 21 and (from 2^21 vectors on; the same
+    vectors over and over have the same result) 32 bits; assignments at every alignment of z; fewer patterns than a
+    16-byte piece of the histogram."""
+    B = _vectors(n, v, kind, seed=n + v)
+    C_ref, z_ref, iters_ref, n_unique, converged = km.optimize_codebook(B, Kc, 6, with_flag=True)
+    B, z_ref, n = np.tile(B, (repeat, 1)), np.tile(z_ref, repeat), n * repeat
+    words = torch.from_numpy(km.pack_words(B).view(np.int32).copy()).cuda()
+    ws = torch.empty(int(btc.lib.btc_codebook_kmeans_workspace_bytes(v, Kc)), dtype=torch.uint8, device="cuda")
+    C, info = torch.empty(Kc, dtype=torch.int32, device="cuda"), torch.empty(4, dtype=torch.int32, device="cuda")
+    z = torch.full((n + 8,), -7, dtype=torch.int16, device="cuda")
+    assert btc.lib.btc_codebook_kmeans(words.data_ptr(), n, v, Kc, 6, C.data_ptr(), z.data_ptr() + 2 * z_off, info.data_ptr(),
+                                       ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream) == 0
+    torch.cuda.synchronize()
+    k_eff = min(Kc, n_unique)
+    assert info.tolist() == [iters_ref, k_eff, n_unique, int(converged)]
+    assert np.array_equal(C.cpu().numpy().view(np.uint32)[:k_eff], km.pack_words(C_ref))
+    got = z.cpu().numpy()
+    assert np.array_equal(got[z_off:z_off + n].view(np.uint16).astype(np.int64), z_ref)
+    assert (got[:z_off] == -7).all() and (got[z_off + n:] == -7).all()
+
+
 @pytest.mark.parametrize("n,v,Kc,kind", [(6001, 18, 40, "iid"), (6003, 17, 200, "noisy"), (149, 20, 20, "iid")])
 def test_kmeans_shares_past_the_end(n, v, Kc, kind):
     """More CTAs than shares of vectors, and a number of vectors that four does not divide: the last ones are counted once."""
