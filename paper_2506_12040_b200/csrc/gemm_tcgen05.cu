@@ -409,6 +409,27 @@ __device__ __forceinline__ void expand_step(int ph, const uint32_t (&w)[step_blo
     }
 }
 
+__device__ __forceinline__ void put(float *p, float f) { *p = f; }
+__device__ __forceinline__ void put(__half *p, float f) { *p = __float2half_rn(f); }
+__device__ __forceinline__ void put(__nv_bfloat16 *p, float f) { *p = __float2bfloat16_rn(f); }
+
+// One feature's results for up to 32 consecutive rows of y, from registers.  The type of y, the mean term and the end of the rows
+// are looked at once per 32 rows: with a look at each of them for every element the epilogue, a quarter of a CTA's time when x
+// tiles are 256 rows high, was bound by the issue of its instructions (11008 x 4096, 2048 rows, fp32 result 164 -> 151 us; 4096 x 4096
+// behind a transform, 512 rows, bf16 27.7 -> 25.1 us).
+template <typename T>
+__device__ __forceinline__ void store_column(T *y, int N, int rows, const uint32_t (&r)[32])
+{
+    if (rows >= 32) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) put(y + (size_t)(unsigned)i * (unsigned)N, __uint_as_float(r[i]));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < rows) put(y + (size_t)(unsigned)i * (unsigned)N, __uint_as_float(r[i]));
+    }
+}
+
 template <int BM, int STAGES, int KS, bool SPLIT, int V>
 __global__ void __launch_bounds__(G2_THREADS, 1)
 gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_i, const Gemm2Params p, const SplitArgs sp)
@@ -574,54 +595,76 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         }
         // ------------------------------------------------------------ epilogue: four warps per lane quadrant
         asm volatile("griddepcontrol.wait;" ::: "memory");     // (y, and the row sums)
+        const int wl = warp - 4;
+        const int q4 = wl & 3, quarter = wl >> 2;
+        const int nl = q4 * 32 + lane, nrow = n0 + nl;
+        const int nc = min(nrow, a.N - 1);
+        const float al = SPLIT ? 0.f : __half2float(a.alpha[nc]);           // (before the wait: the last MMAs cover the loads)
+        const float mu = !SPLIT && a.mu ? __half2float(a.mu[nc]) : 0.f;
         if (ok && mbar_wait(bar_accum, 0, s_abort)) {
             tc_fence_after();
-            const int wl = warp - 4;
-            const int q4 = wl & 3, quarter = wl >> 2;
-            const int nl = q4 * 32 + lane, nrow = n0 + nl;
-            const int nc = min(nrow, a.N - 1);
-            const float al = __half2float(a.alpha[nc]);
-            const float mu = a.mu ? __half2float(a.mu[nc]) : 0.f;
             float *tile = reinterpret_cast<float *>(smem_gen);             // SPLIT: [bn][128], where the x tiles were
 #pragma unroll 1
             for (int c0 = quarter * 32; c0 < bn; c0 += 128) {
                 uint32_t rr[32];
                 tmem_ld32(tmem_d + lane_base + c0, rr);
-                tmem_ld_wait();
                 if (NACC == 2 && NS > 1) {                         // (with a single stage accumulator 1 was never written)
                     uint32_t r2[32];
                     tmem_ld32(tmem_d + lane_base + BM + c0, r2);
                     tmem_ld_wait();
 #pragma unroll
                     for (int i = 0; i < 32; ++i) rr[i] = __float_as_uint(__uint_as_float(rr[i]) + __uint_as_float(r2[i]));
+                } else {
+                    tmem_ld_wait();
                 }
                 if (SPLIT) {
 #pragma unroll
                     for (int i = 0; i < 32; ++i)
                         if (c0 + i < bn) tile[(c0 + i) * 128 + nl] = __uint_as_float(rr[i]);
                 } else if (nrow < a.N) {
+                    const int rows = min(bn - c0, a.M - m0 - c0);
+                    if (a.mu) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const int m = m0 + c0 + i;
-                        if (c0 + i < bn && m < a.M) {
+                        for (int i = 0; i < 32; ++i) {
+                            const float sx = i < rows ? p.sumx[m0 + c0 + i] : 0.f;
                             float y = al * __uint_as_float(rr[i]);
-                            if (a.mu) y += mu * p.sumx[m];
-                            store_from_float(a.y, a.y_dt, (size_t)m * a.N + nrow, y);
+                            y += mu * sx;
+                            rr[i] = __float_as_uint(y);
                         }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) rr[i] = __float_as_uint(al * __uint_as_float(rr[i]));
+                    }
+                    if (rows > 0) {
+                        const size_t o = (size_t)(m0 + c0) * a.N + nrow;
+                        if (a.y_dt == BTC_F32) store_column(reinterpret_cast<float *>(a.y) + o, a.N, rows, rr);
+                        else if (a.y_dt == BTC_F16) store_column(reinterpret_cast<__half *>(a.y) + o, a.N, rows, rr);
+                        else store_column(reinterpret_cast<__nv_bfloat16 *>(a.y) + o, a.N, rows, rr);
                     }
                 }
             }
         }
     }
     if constexpr (SPLIT) {
+        // (columns advance by whole multiples of 32 threads: a thread's four features stay the same, and what belongs to them is
+        // fetched while the cluster meets)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        const int nq = (tid & 31) * 4, n = n0 + nq;
         __syncwarp();
         cluster_arrive();
+        float al[4], mu[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            al[k] = __half2float(a.alpha[min(n + k, a.N - 1)]);
+            mu[k] = a.mu ? __half2float(a.mu[min(n + k, a.N - 1)]) : 0.f;
+        }
         cluster_wait();
         const int splits = gridDim.z, z = blockIdx.z;
         const int per = (bn + splits - 1) / splits, c1 = min(min(bn, a.M - m0), (z + 1) * per);
         if (!*s_abort)
-            for (int i = z * per * 32 + tid; i < c1 * 32; i += G2_THREADS) {
-                const int c = i >> 5, nq = (i & 31) * 4, m = m0 + c;
+            for (int c = z * per + (tid >> 5); c < c1; c += G2_THREADS / 32) {
+                const int m = m0 + c;
+                const float sx = a.mu ? p.sumx[m] : 0.f;
                 float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
                 for (int q = 0; q < splits; ++q) {
                     const float4 f = dsmem_ld128(smem_base + (uint32_t)(c * 128 + nq) * 4u, (uint32_t)q);
@@ -629,14 +672,12 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 }
                 const float v[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int n = n0 + nq + k;
-                    if (n < a.N) {
-                        float y = __half2float(a.alpha[n]) * v[k];
-                        if (a.mu) y += __half2float(a.mu[n]) * p.sumx[m];
-                        store_from_float(a.y, a.y_dt, (size_t)m * a.N + n, y);
+                for (int k = 0; k < 4; ++k)
+                    if (n + k < a.N) {
+                        float y = al[k] * v[k];
+                        if (a.mu) y += mu[k] * sx;
+                        store_from_float(a.y, a.y_dt, (size_t)m * a.N + n + k, y);
                     }
-                }
             }
         cluster_arrive();                                          // (nobody leaves while its shared memory is being read)
         cluster_wait();
@@ -687,7 +728,8 @@ static int launch_cfg(const CUtensorMap &tm, const GemmParams &p, cudaStream_t s
 // costs what their MMAs and x tiles cost or the decode of its weights; wider ones have one issuing thread and cost
 // about the same whatever their width: 11008 x 4096 at 300 rows takes 53 us as two tiles of 160 and 36 as three of 112.  Clock
 // stamps, v = 16: a step 553 at 256 wide (its MMAs alone: 512), 351 at 128, 325 at 80; set-up to first MMA 2.8 k, 3.7 k and
-// 3.8 k, last MMA to end, the epilogue, 12.4 k, 7.6 k and, sum over the cluster included, 6.5 k.  Codewords
+// 3.8 k, last MMA to end, the epilogue, 12.4 k, 7.6 k (both before its stores were batched by 32 rows, about 4 k less since) and,
+// sum over the cluster included, 6.5 k.  Codewords
 // gathered from L1 / L2 (table too large for shared memory) share that path with the x tiles.  A split adds the sum over the
 // cluster.
 struct GemmPlan { int bn, mt, splits, split_tiles; };
