@@ -347,7 +347,7 @@ km_kernel(const KmArgs a)
                 if (was == z) continue;                      // its votes stand
                 changed = 1;
                 a.label[p] = (uint16_t)z;
-                unsigned long long *vote = a.votes + (size_t)z * a.words, *old = a.votes + (size_t)was * a.words;
+                unsigned long long *vote = a.votes + (size_t)z * a.words, *old = it ? a.votes + (size_t)was * a.words : vote;
                 const int bits = a.fields == 3 ? 21 : 32;
                 uint32_t pat = ((uint32_t)p << 1) | 1u;      // count 0: the total; count 1 + t: element t is +1
                 for (int w = 0; w < a.words; ++w) {
