@@ -21,13 +21,19 @@
 //              instead of 487 M for a 4096 x 4096 layer at v = 16 with 8192 centroids).  The low nine bits within 512
 //              neighbouring patterns, the others on columns of four, with a grid barrier between.
 //   M-step     every occurring pattern whose cluster is another than in the round before moves cnt[p] (total and counts of
-//              its set bits, several counts to a 64-bit atomic) from that one's votes to the new one's, so that later rounds
-//              cast few votes and the one that finds nothing changed none; then one thread per centroid
+//              its set bits, several counts to a 64-bit atomic) from that one's votes to the new one's, so that rounds in which
+//              few move cast few votes and the one that finds nothing changed none; then one thread per centroid.  Where many
+//              patterns share few centroids up to 32 copies of the votes are kept, and a warp per centroid adds them up
 //   assign     z through the label table in shared memory (v <= 16)
 // Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 60.2 us a call (67.7 us with all votes cast anew in
 // every round, a barrier between clearing the frequencies and the histogram, and two bytes to a store of assignments).
 // Of these nine grid barriers at 1.1 to 1.5 us, histogram 8 us, ranking 10 us, an E-step 3 + 3 us and in the first round as much
 // again for the votes' atomics, an M-step 4 us, assignment 4 us.
+// A move is two atomics per word where casting anew is one, so a round in which more than half of the patterns move costs more
+// than that; on few centroids, where the votes are most of the call, the copies more than make up for it.  Two rounds, in the second
+// of which three quarters of 65 536 patterns move: 16 centroids 331 us with all votes cast anew, 391 as differences in one copy,
+// 65 in 32; 64 centroids 125, 142, 91; 256 centroids 80, 81, 74; 1024 centroids (one copy) 83.1, 83.6.  A run that converges
+// in R rounds casts fewer votes than anew unless more than (R - 1) / 2 times the patterns move after the first.
 // Integer arithmetic only; results are bit-exact against the definition.
 #include <cuda.h>
 #include <atomic>
@@ -44,6 +50,10 @@ constexpr uint32_t KM_NONE = (255u << 16) | 0xffffu;
 constexpr int KM_MAX_WORDS = 11;             // 64-bit words that hold 21 counts of 32 bits, two each
 constexpr size_t KM_SMEM = 128 * 1024;
 constexpr int KM_PART = 8192;                // most patterns per part of the ranking
+// Patterns per centroid and copy of the votes.  v = 16, 256 centroids, three rounds (us): 98.9 at 32, 97.4 at 64, 100.3 at 128 and
+// 109.2 in one copy; 1024 centroids: 105.4, 99.1, 99.1 and 98.6 (copies have to be cleared and summed).
+constexpr int KM_CROWD = 64;
+constexpr int KM_COPIES = 32;                // at most: a warp sums them up, one per lane
 static_assert((1 << KM_VMAX) / KM_PART <= KM_MAX_CTAS && (KM_BINS + 1 + KM_PART) * 4 <= KM_SMEM && KM_PART < 65536,
               "parts fit the columns, their frequencies shared memory, their counts 16 bits");
 
@@ -297,6 +307,17 @@ km_kernel(const KmArgs a)
     }
     if (!km_sync(a.st, target, &s_ok)) return;
 
+    // ---- where many patterns share few centroids, their votes go to several copies: the atomics on one address follow one another
+    const int copy = kc * a.words;
+    int copies = 1;
+    unsigned long long *votes = a.votes, *mine = votes;
+    if (n_unique >= 2 * KM_CROWD * kc && P >= 2 * copy) {
+        copies = min(min(KM_COPIES, P / copy), n_unique / (KM_CROWD * kc));
+        votes = reinterpret_cast<unsigned long long *>(a.over);                  // (2^v words, last read before the barrier just passed)
+        mine = votes + b % copies * copy;
+        for (int i = gid; i < copy * copies; i += gthreads) votes[i] = 0ull;     // (a barrier before the first is cast)
+    }
+
     const int low = min(v, KM_LOW), high = v - low;
     int it = 0, done = 0;
     while (it < a.max_iter && !done) {
@@ -347,7 +368,7 @@ km_kernel(const KmArgs a)
                 if (was == z) continue;                      // its votes stand
                 changed = 1;
                 a.label[p] = (uint16_t)z;
-                unsigned long long *vote = a.votes + (size_t)z * a.words, *old = it ? a.votes + (size_t)was * a.words : vote;
+                unsigned long long *vote = mine + (size_t)z * a.words, *old = it ? mine + (size_t)was * a.words : vote;
                 const int bits = a.fields == 3 ? 21 : 32;
                 uint32_t pat = ((uint32_t)p << 1) | 1u;      // count 0: the total; count 1 + t: element t is +1
                 for (int w = 0; w < a.words; ++w) {
@@ -371,12 +392,7 @@ km_kernel(const KmArgs a)
         // ---- M-step, and the seeds of the next E-step
         const int bits = a.fields == 3 ? 21 : 32;
         const unsigned long long fmask = (1ull << bits) - 1ull;
-        for (int k = tid * G + b; k < kc; k += gthreads) {               // (spread over the SMs)
-            const unsigned long long *vote = a.votes + (size_t)k * a.words;
-            unsigned long long x[KM_MAX_WORDS];
-#pragma unroll
-            for (int w = 0; w < KM_MAX_WORDS; ++w)
-                if (w < a.words) x[w] = __ldcg(vote + w);
+        auto elect = [&](int k, unsigned long long (&x)[KM_MAX_WORDS], bool write) {
             const uint32_t tot = (uint32_t)(x[0] & fmask);
             uint32_t pat = 0u;                                           // bit 0: the total, bit 1 + t: element t
             int bit = 0;
@@ -389,9 +405,32 @@ km_kernel(const KmArgs a)
                         if (o >= tot - o) pat |= 1u << bit;              // at least as many +1 as -1: sign(0) = +1
                     }
                 }
+            if (!write) return;
             uint32_t c = (pat >> 1) & mask;
             if (tot) a.C[k] = c; else c = __ldcg(a.C + k);               // (an empty cluster keeps its centroid)
             if (it < a.max_iter) atomicMin(a.seed + c, (uint32_t)k);
+        };
+        unsigned long long x[KM_MAX_WORDS];
+        if (copies == 1) {
+            for (int k = tid * G + b; k < kc; k += gthreads) {           // (spread over the SMs)
+                const unsigned long long *vote = votes + (size_t)k * a.words;
+#pragma unroll
+                for (int w = 0; w < KM_MAX_WORDS; ++w)
+                    if (w < a.words) x[w] = __ldcg(vote + w);
+                elect(k, x, true);
+            }
+        } else {
+            for (int k = warp * G + b; k < kc; k += gthreads / 32) {     // (a warp per centroid, a copy per lane)
+                const unsigned long long *vote = votes + (size_t)k * a.words + lane * copy;
+#pragma unroll
+                for (int w = 0; w < KM_MAX_WORDS; ++w)
+                    if (w < a.words) x[w] = lane < copies ? __ldcg(vote + w) : 0ull;
+#pragma unroll
+                for (int w = 0; w < KM_MAX_WORDS; ++w)
+                    if (w < a.words)
+                        for (int o = 16; o; o >>= 1) x[w] += __shfl_xor_sync(0xffffffffu, x[w], o);
+                elect(k, x, lane == 0);
+            }
         }
         if (it < a.max_iter && !km_sync(a.st, target, &s_ok)) return;
     }

@@ -112,6 +112,38 @@ def test_kmeans_votes_move_over_rounds(n, v, Kc, kind, repeat, z_off):
     assert (got[:z_off] == -7).all() and (got[z_off + n:] == -7).all()
 
 
+def _pulled_apart(v, Kc, top, seed):
+    """Every pattern once; the most frequent ones, the first centroids, side by side, the next most frequent ones spread out: after
+    the first round every centroid leaves its place, and most patterns change their cluster."""
+    rng = np.random.default_rng(seed)
+    cnt = np.ones(1 << v, dtype=np.int64)
+    bits = max(Kc - 1, 1).bit_length()
+    for j, far in enumerate(rng.integers(0, 1 << (v - bits), Kc)):
+        cnt[j] = top + 100
+        for q in range(3):
+            cnt[((far ^ (1 << q if q else 0)) << bits) | j] = top - q
+    return rng.permutation(np.repeat(np.arange(1 << v), cnt))
+
+
+@pytest.mark.parametrize("v,Kc,top,max_iter,repeat,rounds,least", [(12, 8, 900, 2, 1, 2, 0.5), (14, 16, 900, 25, 1, 5, 0.5), (14, 16, 3000, 3, 25, 3, 0.5), (14, 100, 900, 25, 1, 5, 0.5),
+                                                                   (13, 1, 900, 25, 1, 2, 0.0), (16, 5, 900, 4, 1, 4, 0.5)])
+def test_kmeans_most_patterns_move(v, Kc, top, max_iter, repeat, rounds, least):
+    """Votes in several copies (64 patterns or more per centroid and copy): 8, 16, 16 (counts of 32 bits, and frequencies past the
+    last bin, whose list was in the same memory), 2, 32 (more copies than CTAs) and 32 of them; most patterns move in the second
+    round, where a run may end."""
+    words = _pulled_apart(v, Kc, top, v + Kc)
+    B = km.unpack_words(words, v)
+    C_ref, z_ref, iters_ref, n_unique, converged = km.optimize_codebook(B, Kc, max_iter, with_flag=True)
+    assert iters_ref == rounds and n_unique >= 2 * 64 * Kc
+    z1, z2 = (km.optimize_codebook(B, Kc, r)[1] for r in (1, 2))
+    first = np.unique(words, return_index=True)[1]
+    assert (z1[first] != z2[first]).mean() >= least
+    C, z, info = _run(np.tile(B, (repeat, 1)), v, Kc, max_iter)
+    assert info.tolist() == [iters_ref, Kc, n_unique, int(converged)]
+    assert np.array_equal(C, km.pack_words(C_ref)) and np.array_equal(z.astype(np.int64), np.tile(z_ref, repeat))
+    assert btc.device_status() == 0
+
+
 @pytest.mark.parametrize("n,v,Kc,kind", [(6001, 18, 40, "iid"), (6003, 17, 200, "noisy"), (149, 20, 20, "iid")])
 def test_kmeans_shares_past_the_end(n, v, Kc, kind):
     """More CTAs than shares of vectors, and a number of vectors that four does not divide: the last ones are counted once."""
