@@ -88,14 +88,15 @@ def test_kmeans_edges(n, v, Kc, offset):
     assert btc.device_status() == 0
 
 
-@pytest.mark.parametrize("n,v,Kc,kind,repeat,z_off", [(2000, 12, 20, "iid", 1, 0), (2000, 12, 20, "iid", 1049, 3), (70003, 16, 40, "noisy", 1, 1),
-                                                      (6001, 18, 40, "iid", 1, 2), (50001, 2, 3, "noisy", 1, 4)])
-def test_kmeans_votes_move_over_rounds(n, v, Kc, kind, repeat, z_off):
+@pytest.mark.parametrize("n,v,Kc,kind,repeat,z_off,rounds", [(2000, 12, 20, "iid", 1, 0, 4), (2000, 12, 20, "iid", 1049, 3, 4), (70003, 16, 40, "noisy", 1, 1, 3),
+                                                             (6001, 18, 40, "iid", 1, 2, 3), (50001, 2, 3, "noisy", 1, 4, 2)])
+def test_kmeans_votes_move_over_rounds(n, v, Kc, kind, repeat, z_off, rounds):
     """Three and four rounds, with votes carried from one to the next in counts of 21 and (from 2^21 vectors on; the same
     vectors over and over have the same result) 32 bits; assignments at every alignment of z; fewer patterns than a
-    16-byte piece of the histogram."""
+    16-byte piece of the histogram (there no votes move)."""
     B = _vectors(n, v, kind, seed=n + v)
     C_ref, z_ref, iters_ref, n_unique, converged = km.optimize_codebook(B, Kc, 6, with_flag=True)
+    assert iters_ref == rounds
     B, z_ref, n = np.tile(B, (repeat, 1)), np.tile(z_ref, repeat), n * repeat
     words = torch.from_numpy(km.pack_words(B).view(np.int32).copy()).cuda()
     ws = torch.empty(int(btc.lib.btc_codebook_kmeans_workspace_bytes(v, Kc)), dtype=torch.uint8, device="cuda")
