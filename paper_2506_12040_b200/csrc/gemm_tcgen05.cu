@@ -416,17 +416,18 @@ __device__ __forceinline__ void put(__nv_bfloat16 *p, float f) { *p = __float2bf
 // One feature's results for up to 32 consecutive rows of y, from registers.  The type of y, the mean term and the end of the rows
 // are looked at once per 32 rows: with a look at each of them for every element the epilogue, a quarter of a CTA's time when x
 // tiles are 256 rows high, was bound by the issue of its instructions (11008 x 4096, 2048 rows, fp32 result 164 -> 151 us; 4096 x 4096
-// behind a transform, 512 rows, bf16 27.7 -> 25.1 us).
+// behind a transform, 512 rows, bf16 27.7 -> 25.1 us).  One pointer that advances, not 32 addresses side by side: those made the form
+// with x tiles above 128 rows spill.
 template <typename T>
 __device__ __forceinline__ void store_column(T *y, int N, int rows, const uint32_t (&r)[32])
 {
     if (rows >= 32) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) put(y + (size_t)(unsigned)i * (unsigned)N, __uint_as_float(r[i]));
+        for (int i = 0; i < 32; ++i, y += N) put(y, __uint_as_float(r[i]));
     } else {
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (i < rows) put(y + (size_t)(unsigned)i * (unsigned)N, __uint_as_float(r[i]));
+        for (int i = 0; i < 32; ++i, y += N)
+            if (i < rows) put(y, __uint_as_float(r[i]));
     }
 }
 
@@ -621,21 +622,22 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
 #pragma unroll
                     for (int i = 0; i < 32; ++i)
                         if (c0 + i < bn) tile[(c0 + i) * 128 + nl] = __uint_as_float(rr[i]);
-                } else if (nrow < a.N) {
+                } else {
                     const int rows = min(bn - c0, a.M - m0 - c0);
                     if (a.mu) {
+                        // (a row's sum per lane, handed to the warp: 32 of them in every thread left no registers for a CTA of the
+                        // row sums beside this one; 11008 x 4096, 2048 rows, bf16 result 129 -> 123 us)
+                        const float sums = lane < rows ? p.sumx[m0 + c0 + lane] : 0.f;
 #pragma unroll
                         for (int i = 0; i < 32; ++i) {
-                            const float sx = i < rows ? p.sumx[m0 + c0 + i] : 0.f;
-                            float y = al * __uint_as_float(rr[i]);
-                            y += mu * sx;
-                            rr[i] = __float_as_uint(y);
+                            const float sx = __shfl_sync(0xffffffffu, sums, i);
+                            rr[i] = __float_as_uint(__fmaf_rn(mu, sx, __fmul_rn(al, __uint_as_float(rr[i]))));
                         }
                     } else {
 #pragma unroll
                         for (int i = 0; i < 32; ++i) rr[i] = __float_as_uint(al * __uint_as_float(rr[i]));
                     }
-                    if (rows > 0) {
+                    if (nrow < a.N && rows > 0) {
                         const size_t o = (size_t)(m0 + c0) * a.N + nrow;
                         if (a.y_dt == BTC_F32) store_column(reinterpret_cast<float *>(a.y) + o, a.N, rows, rr);
                         else if (a.y_dt == BTC_F16) store_column(reinterpret_cast<__half *>(a.y) + o, a.N, rows, rr);

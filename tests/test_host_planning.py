@@ -2,6 +2,7 @@
 large, also where the driver refuses something.  No device."""
 import ctypes
 import os
+import re
 import subprocess
 
 import pytest
@@ -54,6 +55,19 @@ def test_few_tiles_and_a_long_k_share_it_in_a_cluster(fake, N, K, M, split):
         assert call(p(0x1000), 1, p(0x2000), p(0x3000), p(0x4000), None, None, p(0x5000), 2, *shape, *scratch, None) == 0
         (name, _), = _launches(fake)
         assert "gemm_ts_kernel" in name and (fake.fake_cluster(0) > 1) == split
+
+
+def test_registers_of_the_tensor_core_path(tmp_path):
+    """No form spills, and a CTA of the row sums (256 threads) fits the registers that one of 640 threads with x tiles above 128
+    rows leaves of the SM's 65536: they run side by side where a mean term follows."""
+    out = subprocess.check_output([build._nvcc(), *build.NVCC_FLAGS, "-Xptxas=-v", "-I", build.INCLUDE, "-I", build.CSRC, "-c",
+                                   os.path.join(build.CSRC, "gemm_tcgen05.cu"), "-o", str(tmp_path / "gemm.o")], stderr=subprocess.STDOUT, text=True)
+    found = re.findall(r"Compiling entry function '(\S+)'.*?(\d+) bytes spill stores, (\d+) bytes spill loads.*?Used (\d+) registers", out, re.S)
+    regs = {name: -(-int(used) // 8) * 8 for name, _, _, used in found}
+    wide = [r for name, r in regs.items() if re.search("gemm_ts_kernelILi256ELi4ELi1ELb0E", name)]
+    sums, = [r for name, r in regs.items() if "rowsum_kernel" in name]
+    assert len(wide) == 9 and max(wide) * 640 + sums * 256 <= 65536, (wide, sums)
+    assert not [f for f in found if f[1] != "0" or f[2] != "0"]
 
 
 @pytest.mark.parametrize("sms", [148, 64, 16, 4])
