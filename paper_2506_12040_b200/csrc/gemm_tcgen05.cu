@@ -608,6 +608,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
 #pragma unroll 1
             for (int c0 = quarter * 32; c0 < bn; c0 += 128) {
                 uint32_t rr[32];
+                __syncwarp();                                      // (lanes past N did not store in the turn before)
                 tmem_ld32(tmem_d + lane_base + c0, rr);
                 if (NACC == 2 && NS > 1) {                         // (with a single stage accumulator 1 was never written)
                     uint32_t r2[32];

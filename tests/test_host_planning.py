@@ -9,6 +9,7 @@ import pytest
 
 from paper_2506_12040_b200 import build
 from paper_2506_12040_b200.binding import BtcLinearProblem, BtcTransform
+from util import EPILOGUE_SHAPES
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -55,6 +56,18 @@ def test_few_tiles_and_a_long_k_share_it_in_a_cluster(fake, N, K, M, split):
         assert call(p(0x1000), 1, p(0x2000), p(0x3000), p(0x4000), None, None, p(0x5000), 2, *shape, *scratch, None) == 0
         (name, _), = _launches(fake)
         assert "gemm_ts_kernel" in name and (fake.fake_cluster(0) > 1) == split
+
+
+@pytest.mark.parametrize("M,N,K,tile", EPILOGUE_SHAPES)
+def test_tiles_of_the_epilogue_shapes(fake, M, N, K, tile):
+    """The parity test of the results at the edges of tiles meets both forms of the kernel."""
+    p = ctypes.c_void_p
+    fake.fake_reset(148, 0, 0, None)
+    assert fake.btc_linear_gemm(p(0x1000), 1, p(0x2000), p(0x3000), p(0x4000), None, None, p(0x5000), 2, M, N, K, 16, 500, p(0x6000),
+                                ctypes.c_size_t(-(-4 * M // 256) * 256), None) == 0
+    (name, grid), = _launches(fake)
+    assert f"gemm_ts_kernelILi{256 if tile > 128 else 128}E" in name and fake.fake_cluster(0) == 1
+    assert grid == -(-N // 128) * -(-M // tile) and fake.fake_smem(0) == (4 if tile > 128 else 8) * tile * 128 + 1024 + 32768 + 2000 + 14 * 8 + 16
 
 
 def test_registers_of_the_tensor_core_path(tmp_path):

@@ -10,6 +10,11 @@ import paper_2506_12040_b200 as btc
 TOL_GEMV = 2e-3    # fp32 accumulate, M <= 8
 TOL_GEMM = 1e-2    # bf16 tensor-core path
 
+# (M, N, K, rows of x per tile) that the tensor-core path plans on 148 SMs for v = 16 and 500 codewords, K in one piece: ends of
+# tiles, of the 32 rows that leave at a time, and of the 32 features of a warp; up to 128 rows a tile, and above
+EPILOGUE_SHAPES = [(9, 200, 1024, 16), (31, 129, 1024, 32), (33, 128, 1024, 48), (130, 1, 1024, 80), (257, 300, 1024, 80), (300, 127, 1024, 80),
+                   (490, 5000, 512, 256), (333, 6501, 512, 176), (257, 9000, 1024, 144)]
+
 
 def to_device(L, device="cuda"):
     """LayerData (numpy) -> dict of device tensors in the layouts the C ABI takes."""
