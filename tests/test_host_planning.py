@@ -142,3 +142,11 @@ def test_codebook_construction_takes_the_sms_it_is_given(fake, of_stream, most, 
     got, a = _kmeans(fake, 1 << 20, 20)
     assert got == grid or (grid is None and 7 * most // 8 <= got <= most), got
     assert (fake.fake_refused() > 0) == (most > 0) and a.parts == max(got, 128)
+
+
+@pytest.mark.parametrize("n,v,Kc,copies", [(1 << 20, 16, 8192, False), (1 << 20, 16, 512, True), (1 << 20, 16, 513, False), (65535, 16, 512, False), (127, 12, 1, False), (128, 12, 1, True)])
+def test_codebook_construction_keeps_copies_only_where_patterns_can_crowd(fake, n, v, Kc, copies):
+    """128 patterns or more per centroid at most: there are no more of them than vectors, nor than 2^v."""
+    fake.fake_reset(148, 0, 0, None)
+    _kmeans(fake, n, v, Kc)
+    assert f"km_kernelILb{int(copies)}E" in _launches(fake)[0][0]
