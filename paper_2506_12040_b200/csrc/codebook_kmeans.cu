@@ -27,8 +27,9 @@
 //   assign     z through the label table in shared memory (v <= 16)
 // Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 60.2 us a call (67.7 us with all votes cast anew in
 // every round, a barrier between clearing the frequencies and the histogram, and two bytes to a store of assignments).
-// Of these nine grid barriers at 1.1 to 1.5 us, histogram 8 us, ranking 10 us, an E-step 3 + 3 us and in the first round as much
-// again for the votes' atomics, an M-step 4 us, assignment 4 us.
+// Clock stamps of the first CTA in thousands: clearing 2.4, histogram 12.2, patterns per frequency 2.4, ranking 7.2 (and 14.5 more
+// until the slowest CTA has ranked), E-step 5.0 + 10.1 with all votes cast and 4.5 + 5.1 in the round that moves none, M-step 5.5,
+// assignment 7.0; the other seven of the eight grid barriers, with the wait for the slowest CTA, 3.5 to 5.5 each.
 // A move is two atomics per word where casting anew is one, so a round in which more than half of the patterns move costs more
 // than that; on few centroids, where the votes are most of the call, the copies more than make up for it.  Two rounds, in the second
 // of which three quarters of 65 536 patterns move: 16 centroids 331 us with all votes cast anew, 391 as differences in one copy,
@@ -390,7 +391,7 @@ km_kernel(const KmArgs a)
         if (!km_sync(a.st, target, &s_ok)) return;
         done = *reinterpret_cast<volatile int *>(&a.st->changed[it & 1]) == 0;
         ++it;
-        if (done) break;                                     // (its votes are dropped: nothing changed, no M-step)
+        if (done) break;                                     // (nothing changed, so no votes were cast: no M-step)
         // ---- M-step, and the seeds of the next E-step
         const int bits = a.fields == 3 ? 21 : 32;
         const unsigned long long fmask = (1ull << bits) - 1ull;

@@ -414,8 +414,8 @@ __device__ __forceinline__ void put(__half *p, float f) { *p = __float2half_rn(f
 __device__ __forceinline__ void put(__nv_bfloat16 *p, float f) { *p = __float2bfloat16_rn(f); }
 
 // One feature's results for up to 32 consecutive rows of y, from registers.  The type of y, the mean term and the end of the rows
-// are looked at once per 32 rows: with a look at each of them for every element the epilogue, a quarter of a CTA's time when x
-// tiles are 256 rows high, was bound by the issue of its instructions (11008 x 4096, 2048 rows, fp32 result 164 -> 151 us; 4096 x 4096
+// are looked at once per 32 rows: with a look at each of them for every element the epilogue, then a quarter of a CTA's time when x
+// tiles are 256 rows high (a tenth now), was bound by the issue of its instructions (11008 x 4096, 2048 rows, fp32 result 164 -> 151 us; 4096 x 4096
 // behind a transform, 512 rows, bf16 27.7 -> 25.1 us).  One pointer that advances, not 32 addresses side by side: those made the form
 // with x tiles above 128 rows spill.
 template <typename T>
@@ -726,13 +726,16 @@ static int launch_cfg(const CUtensorMap &tm, const GemmParams &p, cudaStream_t s
 }
 
 // Tiling of a (M, N, K) problem: rows of x per tile (bn), tiles of x, K splits (whole index tiles, clusters of up to eight).
-// Time in clocks, fitted to measurements of every width at K = 2000 and 4096: a CTA per SM in rounds, the last one as long as the
-// others, each a fixed part (launch, tensor memory, first tiles, epilogue) and its k steps.  A step of tiles up to 128 wide
+// Time in clocks, fitted to measurements of every width at K = 2000 and 4096, made when the epilogue took longer: a CTA per SM in
+// rounds, the last one as long as the others, each a fixed part (launch, tensor memory, first tiles, epilogue) and its k steps.  A step of tiles up to 128 wide
 // costs what their MMAs and x tiles cost or the decode of its weights; wider ones have one issuing thread and cost
 // about the same whatever their width: 11008 x 4096 at 300 rows takes 53 us as two tiles of 160 and 36 as three of 112.  Clock
-// stamps, v = 16: a step 553 at 256 wide (its MMAs alone: 512), 351 at 128, 325 at 80; set-up to first MMA 2.8 k, 3.7 k and
-// 3.8 k, last MMA to end, the epilogue, 12.4 k, 7.6 k (both before its stores were batched by 32 rows, about 4 k less since) and,
-// sum over the cluster included, 6.5 k.  Codewords
+// stamps, v = 16: a step 553 at 256 wide (its MMAs alone: 512), 351 at 128, 325 at 80; set-up to first MMA 2.7 k, 3.5 k and
+// 3.5 k, last MMA to end, the epilogue, 4.6 k, 2.2 k (12.1 k and 7.0 k when the fixed parts were fitted) and, sum over the cluster
+// included, 5.7 k.  The fixed parts are kept on measurement: with 12 000 and 7 000 for launches without a split the choice changes for
+// one shape in nine and mostly for the worse (us, as is / 4 k less; v = 16, 8192 codewords): 512 x 11008 x 4096 (M x N x K) 47.2 / 46.6,
+// 645 x 7822 x 1024 18.8 / 18.8, 714 x 7739 x 1024 18.1 / 19.0, 1776 x 3270 x 7424 76.6 / 77.1, 539 x 10900 x 5376 56.4 / 58.7, 12 x 6580 x 4352
+// 12.8 / 15.0, 150 x 2050 x 2432 8.3 / 10.3, 230 x 3970 x 4992 16.0 / 18.3, 700 x 8000 x 1200 (v = 10) 25.5 / 32.9.  Codewords
 // gathered from L1 / L2 (table too large for shared memory) share that path with the x tiles.  A split adds the sum over the
 // cluster.
 struct GemmPlan { int bn, mt, splits, split_tiles; };
