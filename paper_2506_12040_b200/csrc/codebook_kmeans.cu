@@ -25,11 +25,11 @@
 //              few move cast few votes and the one that finds nothing changed none; then one thread per centroid.  Where many
 //              patterns share few centroids up to 32 copies of the votes are kept, and a warp per centroid adds them up
 //   assign     z through the label table in shared memory (v <= 16)
-// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 60.2 us a call (67.7 us with all votes cast anew in
-// every round, a barrier between clearing the frequencies and the histogram, and two bytes to a store of assignments).
+// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 50.3 us a call (58.7 us where the round behind an
+// M-step that changed no centroid was run to find that nothing changes: two barriers and both halves of its E-step).
 // Clock stamps of the first CTA in thousands: clearing 2.4, histogram 12.2, patterns per frequency 2.4, ranking 7.2 (and 14.5 more
-// until the slowest CTA has ranked), E-step 5.0 + 10.1 with all votes cast and 4.5 + 5.1 in the round that moves none, M-step 5.5,
-// assignment 7.0; the other seven of the eight grid barriers, with the wait for the slowest CTA, 3.5 to 5.5 each.
+// until the slowest CTA has ranked), E-step 5.0 + 10.1 with all votes cast, M-step 5.5,
+// assignment 7.0; the other five of the six grid barriers, with the wait for the slowest CTA, 3.5 to 5.5 each.
 // A move is two atomics per word where casting anew is one, so a round in which more than half of the patterns move costs more
 // than that; on few centroids, where the votes are most of the call, the copies more than make up for it.  Two rounds, in the second
 // of which three quarters of 65 536 patterns move: 16 centroids 331 us with all votes cast anew, 391 as differences in one copy,
@@ -63,6 +63,7 @@ __device__ int g_km_status = 0;
 struct KmState {                             // zeroed by the host, with the frequencies that follow it
     unsigned arrived;     // grid barrier
     int changed[2];       // set by the E-step of round i in slot i & 1
+    int moved[2];         // the same for a centroid changed by the M-step of round i
     int n_over;           // patterns whose frequency is past the last bin
 };
 
@@ -395,6 +396,7 @@ km_kernel(const KmArgs a)
         // ---- M-step, and the seeds of the next E-step
         const int bits = a.fields == 3 ? 21 : 32;
         const unsigned long long fmask = (1ull << bits) - 1ull;
+        int moved = 0;
         auto elect = [&](int k, unsigned long long (&x)[KM_MAX_WORDS], bool write) {
             const uint32_t tot = (uint32_t)(x[0] & fmask);
             uint32_t pat = 0u;                                           // bit 0: the total, bit 1 + t: element t
@@ -410,7 +412,9 @@ km_kernel(const KmArgs a)
                 }
             if (!write) return;
             uint32_t c = (pat >> 1) & mask;
-            if (tot) a.C[k] = c; else c = __ldcg(a.C + k);               // (an empty cluster keeps its centroid)
+            const uint32_t before = __ldcg(a.C + k);
+            if (!tot) c = before;                                        // (an empty cluster keeps its centroid)
+            if (c != before) { a.C[k] = c; moved = 1; }
             if (it < a.max_iter) atomicMin(a.seed + c, (uint32_t)k);
         };
         unsigned long long x[KM_MAX_WORDS];
@@ -435,7 +439,15 @@ km_kernel(const KmArgs a)
                 elect(k, x, lane == 0);
             }
         }
-        if (it < a.max_iter && !km_sync(a.st, target, &s_ok)) return;
+        if (it < a.max_iter) {
+            // the same centroids give the same assignments, so a round behind an M-step that changed none is not run but only counted
+            const int slot = (it - 1) & 1;
+            if (__syncthreads_or(moved) && tid == 0) a.st->moved[slot] = 1;
+            if (gid == 0) a.st->moved[slot ^ 1] = 0;         // (last read before the barrier of the E-step)
+            if (!km_sync(a.st, target, &s_ok)) return;
+            done = *reinterpret_cast<volatile int *>(&a.st->moved[slot]) == 0;
+            it += done;
+        }
     }
 
     // ---- assignments

@@ -155,6 +155,20 @@ def test_kmeans_shares_past_the_end(n, v, Kc, kind):
     assert np.array_equal(C[:info[1]], km.pack_words(C_ref)) and np.array_equal(z.astype(np.int64), z_ref)
 
 
+@pytest.mark.parametrize("n,v,Kc,kind,max_iter", [(1, 5, 3, "iid", 1), (1, 5, 3, "iid", 2), (1, 5, 3, "iid", 3), (2000, 9, 50, "few", 1), (2000, 9, 50, "few", 2),
+                                                  (20000, 12, 256, "noisy", 1), (20000, 12, 256, "noisy", 2), (20000, 12, 256, "noisy", 3), (20000, 12, 256, "noisy", 4),
+                                                  (300000, 14, 9000, "noisy", 2), (300000, 14, 9000, "noisy", 3)])
+def test_kmeans_ends_where_no_centroid_moves(n, v, Kc, kind, max_iter):
+    """The last round is only counted where no centroid moved before it: with and without a round left to count, centroids that
+    stay from the first round on (as many as patterns) and that move first."""
+    B = _vectors(n, v, kind, seed=n + v)
+    C_ref, z_ref, iters_ref, n_unique, converged = km.optimize_codebook(B, Kc, max_iter, with_flag=True)
+    C, z, info = _run(B, v, Kc, max_iter)
+    assert info.tolist() == [iters_ref, min(Kc, n_unique), n_unique, int(converged)]
+    assert np.array_equal(C[:info[1]], km.pack_words(C_ref)) and np.array_equal(z.astype(np.int64), z_ref)
+    assert btc.device_status() == 0
+
+
 def test_kmeans_feeds_the_layer():
     """The construction's outputs are the layer's inputs: centroids -> btc_codebook_pack, z -> idx; decoding them
     gives the nearest-centroid approximation of the sign matrix, whose Hamming error equals the oracle's objective."""
