@@ -12,8 +12,9 @@
 //   histogram  each CTA counts its vectors in shared memory as 16-bit counters (v <= 16: 128 KB; a hot pattern is a few
 //              per cent of all vectors, and that many atomics on one address of L2 serialise), then adds the non-zero ones
 //   ranking    rank(p) = #{q : (cnt[q], -q) > (cnt[p], -p)}, centroid rank(p) = p when rank(p) < c: a counting sort by frequency
-//              (a histogram of the frequencies per part and in total; word order among equals from the parts before and the
-//              patterns before; frequencies past the last bin are ranked pairwise).  A CTA takes one part of the patterns, its
+//              (a histogram of the frequencies per part and in total; where a frequency's patterns of a part start is added
+//              up once per frequency, and the part's patterns draw their places from there in word order; frequencies past the
+//              last bin are ranked pairwise).  A CTA takes one part of the patterns, its
 //              frequencies in shared memory, or several in turn where few SMs share 2^20 patterns
 //   E-step     the Hamming distance is a sum over the bits, so min over k of (distance, k) for ALL patterns at once is a
 //              separable min-plus convolution: start from key(c_k) = (0, k), and for every bit b
@@ -25,10 +26,10 @@
 //              few move cast few votes and the one that finds nothing changed none; then one thread per centroid.  Where many
 //              patterns share few centroids up to 32 copies of the votes are kept, and a warp per centroid adds them up
 //   assign     z through the label table in shared memory (v <= 16)
-// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 50.3 us a call (58.7 us where the round behind an
+// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 48.1 us a call (50.4 us where a warp added up
+// the parts before, and counted the equals before, for every pattern that it ranked; 58.7 us where in addition the round behind an
 // M-step that changed no centroid was run to find that nothing changes: two barriers and both halves of its E-step).
-// Clock stamps of the first CTA in thousands: clearing 2.4, histogram 12.2, patterns per frequency 2.4, ranking 7.2 (and 14.5 more
-// until the slowest CTA has ranked), E-step 5.0 + 10.1 with all votes cast, M-step 5.5,
+// Clock stamps of the first CTA in thousands: clearing 2.4, histogram 12.2, patterns per frequency 2.4, E-step 5.0 + 10.1 with all votes cast, M-step 5.5,
 // assignment 7.0; the other five of the six grid barriers, with the wait for the slowest CTA, 3.5 to 5.5 each.
 // A move is two atomics per word where casting anew is one, so a round in which more than half of the patterns move costs more
 // than that; on few centroids, where the votes are most of the call, the copies more than make up for it.  Two rounds, in the second
@@ -55,7 +56,7 @@ constexpr int KM_PART = 8192;                // most patterns per part of the ra
 // 109.2 in one copy; 1024 centroids: 105.4, 99.1, 99.1 and 98.6 (copies have to be cleared and summed).
 constexpr int KM_CROWD = 64;
 constexpr int KM_COPIES = 32;                // at most: a warp sums them up, one per lane
-static_assert((1 << KM_VMAX) / KM_PART <= KM_MAX_CTAS && (KM_BINS + 1 + KM_PART) * 4 <= KM_SMEM && KM_PART < 65536,
+static_assert((1 << KM_VMAX) / KM_PART <= KM_MAX_CTAS && (3 * KM_BINS + 1 + KM_PART) * 4 <= KM_SMEM && KM_PART < 65536,
               "parts fit the columns, their frequencies shared memory, their counts 16 bits");
 
 __device__ int g_km_status = 0;
@@ -181,6 +182,7 @@ km_kernel(const KmArgs a)
     extern __shared__ __align__(16) unsigned char km_smem[];
     __shared__ int s_ok;
     __shared__ uint32_t s_warp[32];
+    __shared__ int s_listed;
     uint32_t *sm = reinterpret_cast<uint32_t *>(km_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x, b = blockIdx.x, v = a.v, P = 1 << v, Kc = a.Kc;
@@ -263,49 +265,69 @@ km_kernel(const KmArgs a)
     }
     const int n_unique = (int)s_bins[1], kc = min(Kc, n_unique);
 
-    // ---- ranks (a warp per pattern that can have one below c): centroids, and the seeds of the first E-step.  The counts of the
-    //      parts before this one are one 16-byte load per lane; four patterns' loads are in flight.
+    // ---- ranks: centroids, and the seeds of the first E-step.  A part lists the frequencies that can rank below c, a warp adds up each
+    //      one's patterns in the parts before (a 16-byte load per lane, four in flight), and the part's own patterns then draw their
+    //      places from that start, 32 at a time in word order, those of a frequency found by a match over the warp.
+    uint32_t *s_next = s_cnt + KM_PART, *s_list = s_next + KM_BINS;     // next free rank of a frequency; the frequencies listed
+    constexpr uint32_t UNSEEN = 0xffffffffu, LISTED = 0xfffffffeu;
     for (int q = b; q < a.parts; q += G) {
         const int p0 = min(P, per * q), np = min(P, p0 + per) - p0;
-        if (a.parts > G) {                                   // (several parts: their frequencies again)
-            __syncthreads();
+        __syncthreads();
+        for (int i = tid; i < KM_BINS; i += KM_THREADS) s_next[i] = UNSEEN;
+        if (tid == 0) s_listed = 0;
+        if (a.parts > G)                                     // (several parts: their frequencies again)
             for (int i = tid; i < np; i += KM_THREADS) s_cnt[i] = __ldcg(a.cnt + p0 + i);
-            __syncthreads();
+        __syncthreads();
+        auto ranked = [&](uint32_t c) { return c != 0u && c < KM_BINS - 1 && s_bins[c + 1] < (uint32_t)Kc; };
+        for (int i = tid; i < np; i += KM_THREADS) {
+            const uint32_t c = s_cnt[i];
+            if (ranked(c) && atomicExch(s_next + c, LISTED) == UNSEEN) s_list[atomicAdd(&s_listed, 1)] = c;
         }
-        for (int i0 = warp; i0 < np; i0 += 4 * (KM_THREADS / 32)) {
+        __syncthreads();
+        for (int i0 = warp; i0 < s_listed; i0 += 4 * (KM_THREADS / 32)) {
             uint4 col[4];
-            bool need[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int i = i0 + u * (KM_THREADS / 32);
-                const uint32_t c = i < np ? s_cnt[i] : 0u;
-                need[u] = c != 0u && c < KM_BINS - 1 && s_bins[c + 1] < (uint32_t)Kc;
-                if (need[u]) col[u] = __ldcg(reinterpret_cast<const uint4 *>(a.cols + (size_t)c * KM_MAX_CTAS) + lane);
+                if (i < s_listed) col[u] = __ldcg(reinterpret_cast<const uint4 *>(a.cols + (size_t)s_list[i] * KM_MAX_CTAS) + lane);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int i = i0 + u * (KM_THREADS / 32);
-                const uint32_t c = i < np ? s_cnt[i] : 0u;
-                const bool over = c >= KM_BINS - 1;
-                if (!need[u] && !over) continue;
-                const uint32_t p = (uint32_t)(p0 + i);
+                if (i >= s_listed) continue;
+                const uint32_t w[4] = {col[u].x, col[u].y, col[u].z, col[u].w};
                 uint32_t r = 0;
-                if (over) {
-                    const int m = (int)s_bins[KM_BINS - 1];
-                    for (int j = lane; j < m; j += 32) {
-                        const uint2 o = __ldcg(a.over + j);
-                        r += (o.x > c || (o.x == c && o.y < p)) ? 1u : 0u;
-                    }
-                } else {
-                    const uint32_t w[4] = {col[u].x, col[u].y, col[u].z, col[u].w};
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (8 * lane + k < q) r += (w[k >> 1] >> (16 * (k & 1))) & 0xffffu;
-                    for (int j = lane; j < i; j += 32) r += s_cnt[j] == c ? 1u : 0u;
-                    if (lane == 0) r += s_bins[c + 1];
-                }
+                for (int k = 0; k < 8; ++k)
+                    if (8 * lane + k < q) r += (w[k >> 1] >> (16 * (k & 1))) & 0xffffu;
                 r = __reduce_add_sync(0xffffffffu, r);
-                if (lane == 0 && r < (uint32_t)Kc) { a.C[r] = p; a.seed[p] = r; }
+                if (lane == 0) s_next[s_list[i]] = r + s_bins[s_list[i] + 1];
+            }
+        }
+        __syncthreads();
+        for (int i0 = 0; i0 < np; i0 += KM_THREADS) {        // (uniform)
+            const int i = i0 + tid;
+            const uint32_t p = (uint32_t)(p0 + i), c = i < np ? s_cnt[i] : 0u;
+            const bool mine = ranked(c);
+            const uint32_t same = __match_any_sync(0xffffffffu, mine ? c : 0u);
+            const int first = __ffs(same) - 1;
+            uint32_t r = 0;
+            for (int w = 0; w < KM_THREADS / 32 && i0 + 32 * w < np; ++w) {
+                if (w == warp && mine && lane == first) { r = s_next[c]; s_next[c] = r + __popc(same); }
+                __syncthreads();
+            }
+            r = __shfl_sync(0xffffffffu, r, first) + __popc(same & ((1u << lane) - 1u));
+            if (mine && r < (uint32_t)Kc) { a.C[r] = p; a.seed[p] = r; }
+            // past the last bin: pairwise, a warp per pattern
+            for (uint32_t over = __ballot_sync(0xffffffffu, c >= KM_BINS - 1); over; over &= over - 1u) {
+                const uint32_t co = __shfl_sync(0xffffffffu, c, __ffs(over) - 1), po = __shfl_sync(0xffffffffu, p, __ffs(over) - 1);
+                uint32_t before = 0;
+                for (int j = lane; j < (int)s_bins[KM_BINS - 1]; j += 32) {
+                    const uint2 o = __ldcg(a.over + j);
+                    before += (o.x > co || (o.x == co && o.y < po)) ? 1u : 0u;
+                }
+                before = __reduce_add_sync(0xffffffffu, before);
+                if (lane == 0 && before < (uint32_t)Kc) { a.C[before] = po; a.seed[po] = before; }
             }
         }
     }
