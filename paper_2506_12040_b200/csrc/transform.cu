@@ -5,7 +5,7 @@
 // computed as two small products with fp32 accumulation: Y = (X o sigma) P2, then X' = P1^T Y.
 // The result is written as fp32 for the decode path (which quantises or rounds the activations itself, so no intermediate
 // 16-bit rounding is added) and in the dtype of x for the tensor-core path.
-// transform_kernel (up to eight rows, fp32 activations, factor sizes the other does not take): a CTA owns a tile of TR_DT output
+// transform_kernel (fp32 activations, factor sizes that the other two do not take): a CTA owns a tile of TR_DT output
 // columns d and a group of rows of x: it stages the k2 x TR_DT slab of P2 and all of P1 in shared memory once, then for each of
 // its rows loads X (K values) and produces X'[:, d-tile]; a decode step with one row of x therefore spreads over k2 / TR_DT
 // SMs instead of one.
@@ -130,6 +130,122 @@ transform_kernel(const void *__restrict__ x, int x_dt, const uint32_t *__restric
             }
         }
     }
+}
+
+// ---- up to eight rows of 16-bit activations, k2 = 64 or 128, k1 up to 128 ------------------------------------------------
+// A CTA owns four output columns d of one row of x and, in turn, groups of sixteen output rows c.  Four lanes share a row a of X and
+// read it from global memory straight into registers, each every fourth piece of eight; Y (k1 x 4) goes through shared memory;
+// sixteen lanes share an output row c, each with every sixteenth a.  Lanes that share a sum hand over halves of their columns, so that
+// four sums over four lanes take three shuffles and leave one in each.
+// Bound: latency, of the chain behind the kernel before it: wait, x from L2, two products of K2 / 4 and k1 / 16 steps with one
+// barrier between them, store.  Shared memory (the k2 x 4 slab of P2 and Y) is under 5 KB and 32 registers a thread are enough,
+// so a CTA fits beside the two of the integer decode kernel: it starts, and fetches the factors, while the layers before it run,
+// and those behind it start while it runs.  One row of 64 x 64 and the three 4096 x 4096 layers behind it: 11.2 us with
+// transform_kernel (40 KB of shared memory, so neither; P1 and X through it), now 8.4.
+constexpr int TS_D = 4, TS_C = 16;  // columns per CTA, output rows per group
+
+// acc[i] summed over the four lanes that differ in bits 0 and 1; lane q gets column q
+__device__ __forceinline__ float ts_quad(const float (&acc)[TS_D], int q) {
+    const float k0 = q & 2 ? acc[2] : acc[0], k1 = q & 2 ? acc[3] : acc[1];
+    const float s0 = k0 + __shfl_xor_sync(0xffffffffu, q & 2 ? acc[0] : acc[2], 2);
+    const float s1 = k1 + __shfl_xor_sync(0xffffffffu, q & 2 ? acc[1] : acc[3], 2);
+    return (q & 1 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, q & 1 ? s0 : s1, 1);
+}
+
+// AP: passes of 64 rows a; K2: k2.
+template <int AP, int K2>
+__global__ void __launch_bounds__(TR_THREADS, AP == 1 && K2 == 64 ? 8 : 4)
+transform_few_kernel(const uint16_t *__restrict__ x, int f16, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
+                     const float *__restrict__ P2, int k1, void *__restrict__ xt, int out_dt)
+{
+    constexpr int PIECES = K2 / 32, AQ = 4 * AP;         // pieces of eight activations, and a's, of a lane
+    __shared__ __align__(16) float s_p2[K2 / 8][8 * TS_D + 4];           // (four lanes read pieces next to each other: on different banks)
+    __shared__ __align__(16) float s_y[64 * AP][TS_D];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int tid = threadIdx.x, q = tid & 3, d0 = blockIdx.x * TS_D, nc = (k1 + TS_C - 1) / TS_C;
+    const size_t row = (size_t)blockIdx.z * k1 * K2;
+    for (int i = tid; i < K2 * TS_D; i += TR_THREADS) {
+        const int b = i / TS_D, d = i % TS_D;
+        s_p2[b / 8][b % 8 * TS_D + d] = __ldg(P2 + (size_t)b * K2 + d0 + d);
+    }
+    const int al = tid & 15, cl = tid >> 4;              // second product: first a, output row of the group
+    float pv[AQ];
+    auto load_p1 = [&](int cg) {
+        const int c = cg * TS_C + cl;
+#pragma unroll
+        for (int i = 0; i < AQ; ++i) pv[i] = c < k1 && al + 16 * i < k1 ? __ldg(P1 + (size_t)(al + 16 * i) * k1 + c) : 0.f;
+    };
+    load_p1(blockIdx.y);
+    uint32_t sg[AP][PIECES];                             // sign bits of a piece
+#pragma unroll
+    for (int ap = 0; ap < AP; ++ap)
+#pragma unroll
+        for (int j = 0; j < PIECES; ++j) {
+            const int e = min(64 * ap + (tid >> 2), k1 - 1) * K2 + 8 * (q + 4 * j);
+            sg[ap][j] = __ldg(sigma_bits + (e >> 5)) >> (e & 31);
+        }
+    __syncthreads();
+    // (the factors are parameters of the layer, complete before the call was enqueued; x is read, and x' written, once the kernel
+    // before this one has completed)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll
+    for (int ap = 0; ap < AP; ++ap) {
+        const int a = 64 * ap + (tid >> 2);
+        uint4 w[PIECES];
+#pragma unroll
+        for (int j = 0; j < PIECES; ++j)
+            w[j] = a < k1 ? __ldg(reinterpret_cast<const uint4 *>(x + row + (size_t)a * K2) + q + 4 * j) : make_uint4(0u, 0u, 0u, 0u);
+        float acc[TS_D] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < PIECES; ++j) {
+            const uint32_t h[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+            const float4 *p = reinterpret_cast<const float4 *>(s_p2[q + 4 * j]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t u = h[i] ^ (((sg[ap][j] >> (2 * i)) & 1u) << 15) ^ (((sg[ap][j] >> (2 * i + 1)) & 1u) << 31);
+                const float2 f = f16 ? __half22float2(*reinterpret_cast<const __half2 *>(&u)) : make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+                const float4 p0 = p[2 * i], p1 = p[2 * i + 1];
+                acc[0] = fmaf(f.x, p0.x, acc[0]); acc[1] = fmaf(f.x, p0.y, acc[1]); acc[2] = fmaf(f.x, p0.z, acc[2]); acc[3] = fmaf(f.x, p0.w, acc[3]);
+                acc[0] = fmaf(f.y, p1.x, acc[0]); acc[1] = fmaf(f.y, p1.y, acc[1]); acc[2] = fmaf(f.y, p1.z, acc[2]); acc[3] = fmaf(f.y, p1.w, acc[3]);
+            }
+        }
+        const float y = ts_quad(acc, q);
+        s_y[a][q] = a < k1 ? y : 0.f;                    // (not 0 times what P2 holds)
+    }
+    __syncthreads();
+    for (int cg = blockIdx.y; cg < nc; cg += gridDim.y) {
+        if (cg != (int)blockIdx.y) load_p1(cg);
+        float acc[TS_D] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < AQ; ++i) {
+            const float4 y = *reinterpret_cast<const float4 *>(s_y[al + 16 * i]);
+            acc[0] = fmaf(pv[i], y.x, acc[0]); acc[1] = fmaf(pv[i], y.y, acc[1]); acc[2] = fmaf(pv[i], y.z, acc[2]); acc[3] = fmaf(pv[i], y.w, acc[3]);
+        }
+        float r = ts_quad(acc, q);
+        r += __shfl_xor_sync(0xffffffffu, r, 4);
+        r += __shfl_xor_sync(0xffffffffu, r, 8);
+        const int c = cg * TS_C + cl;
+        if (al < 4 && c < k1) store_from_float(xt, out_dt, row + (size_t)c * K2 + d0 + q, r);
+    }
+}
+
+template <int AP, int K2>
+static int launch_transform_few(const void *x, int x_dt, const btc_transform &T, void *xt, int out_dt, int M, cudaStream_t s)
+{
+    // every group of output rows its own CTA as long as an SM gets two (each computes Y again)
+    const int tiles = K2 / TS_D, nc = (T.k1 + TS_C - 1) / TS_C, most = 2 * device_sms() / (tiles * M);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)tiles, (unsigned)(most < 1 ? 1 : most < nc ? most : nc), (unsigned)M);
+    cfg.blockDim = dim3(TR_THREADS);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, transform_few_kernel<AP, K2>, static_cast<const uint16_t *>(x), x_dt == BTC_F16 ? 1 : 0, T.sigma_bits, T.P1,
+                                             T.P2, T.k1, xt, out_dt);
+    return e == cudaSuccess ? BTC_OK : cuda_fail(e);
 }
 
 // ---- 16-bit activations, k2 a multiple of 16, k1 up to 128: the two products on the warp-level tensor cores ---------------
@@ -465,13 +581,18 @@ static int launch_transform_terms(const void *x, const btc_transform &T, void *x
 int launch_transform(const void *x, int x_dt, const btc_transform &T, void *xt, int out_dt, int M, int K, cudaStream_t s)
 {
     if ((long long)T.k1 * T.k2 != K) return BTC_ERR_SHAPE;
-    // (up to 8 rows the fp32 form above, a slab of eight columns per CTA, has the shorter chain: 4.3 us at 64 x 64, one row, where
-    // this one took 4.9.  Below 64 rows three terms: the precision of the fp32 form; above, two carry more than 16-bit x.)
+    // (up to 8 rows the forms in fp32 have the shorter chain: 4.3 us at 64 x 64, one row, with the slower of them where this one took
+    // 4.9.  Below 64 rows three terms: the precision of the fp32 form; above, two carry more than 16-bit x.)
     if (x_dt != BTC_F32 && M > 8 && T.k2 % 16 == 0 && T.k1 <= 128) {
         const bool f16 = x_dt == BTC_F16;
         const int rc = M >= 64 ? (f16 ? launch_transform_terms<2, true>(x, T, xt, out_dt, M, s) : launch_transform_terms<2, false>(x, T, xt, out_dt, M, s))
                                : (f16 ? launch_transform_terms<3, true>(x, T, xt, out_dt, M, s) : launch_transform_terms<3, false>(x, T, xt, out_dt, M, s));
         if (rc != BTC_ERR_UNSUPPORTED) return rc;
+    }
+    // (k2 as compiled in; k1 up to two passes of 64 rows)
+    if (x_dt != BTC_F32 && M <= 8 && T.k1 <= 128 && (T.k2 == 64 || T.k2 == 128)) {
+        if (T.k2 == 64) return T.k1 <= 64 ? launch_transform_few<1, 64>(x, x_dt, T, xt, out_dt, M, s) : launch_transform_few<2, 64>(x, x_dt, T, xt, out_dt, M, s);
+        return T.k1 <= 64 ? launch_transform_few<1, 128>(x, x_dt, T, xt, out_dt, M, s) : launch_transform_few<2, 128>(x, x_dt, T, xt, out_dt, M, s);
     }
     const size_t smem = ((size_t)K + 4 * T.k1 + 4 + (size_t)T.k2 * TR_DT + (size_t)T.k1 * TR_DT + (size_t)T.k1 * (T.k1 + 8)) * sizeof(float);
     if (smem > 200 * 1024) return BTC_ERR_UNSUPPORTED;
