@@ -133,112 +133,120 @@ transform_kernel(const void *__restrict__ x, int x_dt, const uint32_t *__restric
 }
 
 // ---- up to eight rows of 16-bit activations, k2 = 64 or 128, k1 up to 128 ------------------------------------------------
-// A CTA owns four output columns d of one row of x and, in turn, groups of sixteen output rows c.  Four lanes share a row a of X and
-// read it from global memory straight into registers, each every fourth piece of eight; Y (k1 x 4) goes through shared memory;
-// sixteen lanes share an output row c, each with every sixteenth a.  Lanes that share a sum hand over halves of their columns, so that
-// four sums over four lanes take three shuffles and leave one in each.
-// Bound: latency, of the chain behind the kernel before it: wait, x from L2, two products of K2 / 4 and k1 / 16 steps with one
-// barrier between them, store.  Shared memory (the k2 x 4 slab of P2 and Y) is under 5 KB and 32 registers a thread are enough,
-// so a CTA fits beside the two of the integer decode kernel: it starts, and fetches the factors, while the layers before it run,
-// and those behind it start while it runs.  One row of 64 x 64 and the three 4096 x 4096 layers behind it: 11.2 us with
-// transform_kernel (40 KB of shared memory, so neither; P1 and X through it), now 8.4.
-constexpr int TS_D = 4, TS_C = 16;  // columns per CTA, output rows per group
+// A CTA owns eight output columns d of one row of x.  Four lanes share a row a of X and read it from global memory straight into
+// registers, each every fourth piece of eight; Y (k1 x 8) goes through shared memory; four lanes share an output row c, each with
+// every fourth a.  Lanes that share a sum hand over halves of their columns, so that four sums over four lanes take three shuffles
+// and leave one in each.
+// Bound: latency, of the chain behind the kernel before it: wait, x from L2, two products of K2 / 4 and k1 / 4 steps with one
+// barrier between them, store.  Shared memory (the k2 x 8 slab of P2 and Y, 4 KB at 64 x 64) and 32 registers a thread leave room for a
+// CTA beside the two of the integer decode kernel: it starts, and fetches the factors, while the layers before it run, and those behind
+// it start while it runs; P1 waits in L1.  One row of 64 x 64 and the three 4096 x 4096 layers behind it: 11.2 us with
+// transform_kernel (40 KB of shared memory, so neither; P1 and X through it), now 9.4.
+constexpr int TS_D = 8;             // columns per CTA
 
 // acc[i] summed over the four lanes that differ in bits 0 and 1; lane q gets column q
-__device__ __forceinline__ float ts_quad(const float (&acc)[TS_D], int q) {
+__device__ __forceinline__ float ts_quad(const float *acc, int q) {
     const float k0 = q & 2 ? acc[2] : acc[0], k1 = q & 2 ? acc[3] : acc[1];
     const float s0 = k0 + __shfl_xor_sync(0xffffffffu, q & 2 ? acc[0] : acc[2], 2);
     const float s1 = k1 + __shfl_xor_sync(0xffffffffu, q & 2 ? acc[1] : acc[3], 2);
     return (q & 1 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, q & 1 ? s0 : s1, 1);
 }
+__device__ __forceinline__ void ts_fma(float (&acc)[TS_D], float f, const float *row) {
+    const float4 p = *reinterpret_cast<const float4 *>(row), r = *reinterpret_cast<const float4 *>(row + 4);
+    acc[0] = fmaf(f, p.x, acc[0]); acc[1] = fmaf(f, p.y, acc[1]); acc[2] = fmaf(f, p.z, acc[2]); acc[3] = fmaf(f, p.w, acc[3]);
+    acc[4] = fmaf(f, r.x, acc[4]); acc[5] = fmaf(f, r.y, acc[5]); acc[6] = fmaf(f, r.z, acc[6]); acc[7] = fmaf(f, r.w, acc[7]);
+}
 
-// AP: passes of 64 rows a; K2: k2.
+// AP: passes of 64 rows a, and c; K2: k2.
 template <int AP, int K2>
 __global__ void __launch_bounds__(TR_THREADS, AP == 1 && K2 == 64 ? 8 : 4)
 transform_few_kernel(const uint16_t *__restrict__ x, int f16, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
                      const float *__restrict__ P2, int k1, void *__restrict__ xt, int out_dt)
 {
-    constexpr int PIECES = K2 / 32, AQ = 4 * AP;         // pieces of eight activations, and a's, of a lane
+    constexpr int PIECES = K2 / 32;                      // of eight activations, of a lane
     __shared__ __align__(16) float s_p2[K2 / 8][8 * TS_D + 4];           // (four lanes read pieces next to each other: on different banks)
     __shared__ __align__(16) float s_y[64 * AP][TS_D];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int tid = threadIdx.x, q = tid & 3, d0 = blockIdx.x * TS_D, nc = (k1 + TS_C - 1) / TS_C;
-    const size_t row = (size_t)blockIdx.z * k1 * K2;
+    const int tid = threadIdx.x, q = tid & 3, d0 = blockIdx.x * TS_D;
+    const size_t row = (size_t)blockIdx.y * k1 * K2;
     for (int i = tid; i < K2 * TS_D; i += TR_THREADS) {
         const int b = i / TS_D, d = i % TS_D;
         s_p2[b / 8][b % 8 * TS_D + d] = __ldg(P2 + (size_t)b * K2 + d0 + d);
     }
-    const int al = tid & 15, cl = tid >> 4;              // second product: first a, output row of the group
-    float pv[AQ];
-    auto load_p1 = [&](int cg) {
-        const int c = cg * TS_C + cl;
-#pragma unroll
-        for (int i = 0; i < AQ; ++i) pv[i] = c < k1 && al + 16 * i < k1 ? __ldg(P1 + (size_t)(al + 16 * i) * k1 + c) : 0.f;
-    };
-    load_p1(blockIdx.y);
-    uint32_t sg[AP][PIECES];                             // sign bits of a piece
-#pragma unroll
-    for (int ap = 0; ap < AP; ++ap)
+    for (int i = 8 * tid; i < k1 * k1; i += 8 * TR_THREADS) {            // (a word of every 32 bytes, into L1)
+        float f;
+        asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(f) : "l"(P1 + i));
+    }
+    uint32_t sg[PIECES];                                 // sign bits of a piece
+    auto load_signs = [&](int a) {
 #pragma unroll
         for (int j = 0; j < PIECES; ++j) {
-            const int e = min(64 * ap + (tid >> 2), k1 - 1) * K2 + 8 * (q + 4 * j);
-            sg[ap][j] = __ldg(sigma_bits + (e >> 5)) >> (e & 31);
+            const int e = min(a, k1 - 1) * K2 + 8 * (q + 4 * j);
+            sg[j] = __ldg(sigma_bits + (e >> 5)) >> (e & 31);
         }
+    };
+    load_signs(tid >> 2);
     __syncthreads();
     // (the factors are parameters of the layer, complete before the call was enqueued; x is read, and x' written, once the kernel
     // before this one has completed)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-#pragma unroll
+#pragma unroll 1
     for (int ap = 0; ap < AP; ++ap) {
         const int a = 64 * ap + (tid >> 2);
         uint4 w[PIECES];
 #pragma unroll
         for (int j = 0; j < PIECES; ++j)
             w[j] = a < k1 ? __ldg(reinterpret_cast<const uint4 *>(x + row + (size_t)a * K2) + q + 4 * j) : make_uint4(0u, 0u, 0u, 0u);
-        float acc[TS_D] = {0.f, 0.f, 0.f, 0.f};
+        float acc[TS_D] = {};
 #pragma unroll
         for (int j = 0; j < PIECES; ++j) {
             const uint32_t h[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
-            const float4 *p = reinterpret_cast<const float4 *>(s_p2[q + 4 * j]);
+            const float *p = s_p2[q + 4 * j];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const uint32_t u = h[i] ^ (((sg[ap][j] >> (2 * i)) & 1u) << 15) ^ (((sg[ap][j] >> (2 * i + 1)) & 1u) << 31);
+                const uint32_t u = h[i] ^ (((sg[j] >> (2 * i)) & 1u) << 15) ^ (((sg[j] >> (2 * i + 1)) & 1u) << 31);
                 const float2 f = f16 ? __half22float2(*reinterpret_cast<const __half2 *>(&u)) : make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
-                const float4 p0 = p[2 * i], p1 = p[2 * i + 1];
-                acc[0] = fmaf(f.x, p0.x, acc[0]); acc[1] = fmaf(f.x, p0.y, acc[1]); acc[2] = fmaf(f.x, p0.z, acc[2]); acc[3] = fmaf(f.x, p0.w, acc[3]);
-                acc[0] = fmaf(f.y, p1.x, acc[0]); acc[1] = fmaf(f.y, p1.y, acc[1]); acc[2] = fmaf(f.y, p1.z, acc[2]); acc[3] = fmaf(f.y, p1.w, acc[3]);
+                ts_fma(acc, f.x, p + 2 * i * TS_D);
+                ts_fma(acc, f.y, p + (2 * i + 1) * TS_D);
             }
         }
-        const float y = ts_quad(acc, q);
-        s_y[a][q] = a < k1 ? y : 0.f;                    // (not 0 times what P2 holds)
+        const float y0 = ts_quad(acc, q), y1 = ts_quad(acc + 4, q);
+        s_y[a][q] = a < k1 ? y0 : 0.f;                   // (not 0 times what P2 holds)
+        s_y[a][4 + q] = a < k1 ? y1 : 0.f;
+        if (AP > 1) load_signs(a + 64);
     }
     __syncthreads();
-    for (int cg = blockIdx.y; cg < nc; cg += gridDim.y) {
-        if (cg != (int)blockIdx.y) load_p1(cg);
-        float acc[TS_D] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int cp = 0; cp < AP; ++cp) {
+        const int c = 64 * cp + (tid >> 2);
+        float acc[TS_D] = {};
+#pragma unroll 1
+        for (int i0 = 0; i0 < 16 * AP; i0 += 8) {
+            float pv[8];
 #pragma unroll
-        for (int i = 0; i < AQ; ++i) {
-            const float4 y = *reinterpret_cast<const float4 *>(s_y[al + 16 * i]);
-            acc[0] = fmaf(pv[i], y.x, acc[0]); acc[1] = fmaf(pv[i], y.y, acc[1]); acc[2] = fmaf(pv[i], y.z, acc[2]); acc[3] = fmaf(pv[i], y.w, acc[3]);
+            for (int i = 0; i < 8; ++i) {
+                const int a = q + 4 * (i0 + i);
+                pv[i] = c < k1 && a < k1 ? __ldg(P1 + (size_t)a * k1 + c) : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ts_fma(acc, pv[i], s_y[q + 4 * (i0 + i)]);
         }
-        float r = ts_quad(acc, q);
-        r += __shfl_xor_sync(0xffffffffu, r, 4);
-        r += __shfl_xor_sync(0xffffffffu, r, 8);
-        const int c = cg * TS_C + cl;
-        if (al < 4 && c < k1) store_from_float(xt, out_dt, row + (size_t)c * K2 + d0 + q, r);
+        const float r0 = ts_quad(acc, q), r1 = ts_quad(acc + 4, q);
+        if (c < k1) {
+            store_from_float(xt, out_dt, row + (size_t)c * K2 + d0 + q, r0);
+            store_from_float(xt, out_dt, row + (size_t)c * K2 + d0 + 4 + q, r1);
+        }
     }
 }
 
 template <int AP, int K2>
 static int launch_transform_few(const void *x, int x_dt, const btc_transform &T, void *xt, int out_dt, int M, cudaStream_t s)
 {
-    // every group of output rows its own CTA as long as an SM gets two (each computes Y again)
-    const int tiles = K2 / TS_D, nc = (T.k1 + TS_C - 1) / TS_C, most = 2 * device_sms() / (tiles * M);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)tiles, (unsigned)(most < 1 ? 1 : most < nc ? most : nc), (unsigned)M);
+    cfg.gridDim = dim3(K2 / TS_D, (unsigned)M);
     cfg.blockDim = dim3(TR_THREADS);
     cfg.stream = s;
     cfg.attrs = at;
