@@ -317,7 +317,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams
 // decode thread owns one weight row = one tensor-memory lane, expands the row's 64 weights of a k step into 32
 // registers and stores them with tcgen05.st into a ring of A tiles in tensor memory (32 columns per k step); the MMAs
 // take A from tensor memory and only the x tile from shared memory.
-//   warp 0 TMA producer (x tiles, index tiles, table) | warp 1 MMA issuer | warp 2 tensor-memory allocation
+//   warp 0 TMA producer (x tiles, table) | warp 1 MMA issuer | warp 2 tensor-memory allocation, index tiles
 //   warps 4-19: four groups of four warps; group g expands the stages g, g + 4, ...; then all 16 run the epilogue.
 // Tensor memory (512 columns): accumulator in columns [0, BM), A ring of STAGES x 32 KS columns from column 256.
 //
@@ -499,12 +499,6 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             }
             for (int ks = 0; ks < NS; ++ks) {
                 const int kt0 = ks * KS;
-                if (kt0 % KPT == 0) {
-                    const int it = kt0 / KPT, ib = it & 1;
-                    if (it >= 2 && !mbar_wait(bar_empty_i(ib), ((it >> 1) & 1) ^ 1, s_abort)) break;
-                    mbar_expect_tx(bar_full_i(ib), G2_IDX_BYTES);
-                    tma_load_2d(smem_u32(s_idx + (size_t)ib * G2_IDX_BYTES), &tmap_i, (kt_first / KPT) * 64 + it * 64, n0, bar_full_i(ib));
-                }
                 if (ks == 0 && !p.sumx) asm volatile("griddepcontrol.wait;" ::: "memory");     // x
                 const int s = ks % STAGES;
                 if (ks >= STAGES && !mbar_wait(bar_empty(s), ((ks / STAGES) & 1) ^ 1, s_abort)) break;
@@ -514,6 +508,21 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                     tma_load_2d(smem_base + s * STAGE_BYTES + j * B_BYTES, &tmap_x, (kt_first + kt0 + j) * G_BK, m0, bar_full(s));
             }
         }
+    } else if (warp == 2) {
+        // Index tiles, as soon as there is room.  In turn with the x tiles, which wait for MMAs, a tile was sent for four stages before
+        // its first use, less than it takes to arrive, and the decode warps stood there at every tile (1.6 k clk a stage of two k
+        // steps, most of a round of the ring).  With this, and a stage's first step expanded before the stage is free: 4096 x
+        // 11008, 77 rows 17.4 -> 15.8 us, 4096 x 4096 behind a transform, 512 rows 25.2 -> 23.1 (16.9 and 25.0 with the latter alone).
+        // A ring of up to eight x tiles with its own barriers beside the four A tiles took it all back (17.3, 24.7).
+        if (lane == 0) {
+            for (int it = 0; it * KPT < KT; ++it) {
+                const int ib = it & 1;
+                if (it >= 2 && !mbar_wait(bar_empty_i(ib), ((it >> 1) & 1) ^ 1, s_abort)) break;
+                mbar_expect_tx(bar_full_i(ib), G2_IDX_BYTES);
+                tma_load_2d(smem_u32(s_idx + (size_t)ib * G2_IDX_BYTES), &tmap_i, (kt_first / KPT) * 64 + it * 64, n0, bar_full_i(ib));
+            }
+        }
+        __syncwarp();
     } else if (warp == 1 || (NACC == 2 && warp == 3)) {
         if (lane == 0) {
             const int me = (warp == 1) ? 0 : 1;                    // which accumulator / which stages
@@ -580,13 +589,20 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 if (lane == 0) mbar_arrive(bar_empty_i(ib));
             }
             const int sa = ks % STAGES;
+            // register i holds the weights 2i, 2i+1 of the k step (K elements 2i, 2i+1 of this row of A); those of a stage's first
+            // step are ready before the stage is where it has two (with one the
+            // MMAs set the pace)
+            uint32_t regs[32];
+            if (KS > 1) {
+                expand_step<V, 0>(kt0 % (V / gcd64(V)), w[0], one2, regs);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) asm volatile("" : "+r"(regs[i]));
+            }
             if (ks >= STAGES && !mbar_wait(bar_empty(sa), ((ks / STAGES) & 1) ^ 1, s_abort)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll
             for (int j = 0; j < KS; ++j) {
-                // register i holds the weights 2i, 2i+1 of the k step (K elements 2i, 2i+1 of this row of A)
-                uint32_t regs[32];
-                expand_step<V, 0>((kt0 + j) % (V / gcd64(V)), w[j], one2, regs);
+                if (KS == 1 || j) expand_step<V, 0>((kt0 + j) % (V / gcd64(V)), w[j], one2, regs);
                 tmem_st32(tmem_d + lane_base + G4_A_COL0 + sa * ACOLS + 32 * j, regs);
             }
             tmem_st_wait();
