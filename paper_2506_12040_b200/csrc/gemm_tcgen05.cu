@@ -334,8 +334,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams
 // Launched with programmatic stream serialisation: barriers, tensor memory, table and first indices are ready before
 // the predecessor has finished; x is read after it (or right away where the predecessor is the row-sum kernel, which
 // itself waited for it; then the epilogue waits).  Its own successors may start early (a transform
-// behind it: 13.0 -> 10.5 us for 24 rows, K = 1024), but not with a mean term: the next call's row sums, small CTAs, would pile up
-// on the SMs that a round of tiles leaves idle (9.0 -> 9.8 us for 16 rows of 4096 x 4096).
+// behind it: 13.0 -> 10.5 us for 24 rows, K = 1024), with a mean term only when its k steps are done: from the start, the next
+// call's row sums, small CTAs, would pile up on the SMs that a round of tiles leaves idle (9.0 -> 9.8 us for 16 rows of 4096 x 4096);
+// from there on they are in place when the epilogue ends (4096 x 11008, 77 rows: 15.8 -> 15.1 us; 16 rows 8.9 where they came at 9.0).
 constexpr int G2_DWARPS = 16;                    // decode warps (four groups of four)
 constexpr int G2_THREADS = 128 + G2_DWARPS * 32;
 constexpr uint32_t G2_IDX_BYTES = 128 * 128;     // one index tile
@@ -611,6 +612,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             if (lane == 0) mbar_arrive(bar_full(sa));
         }
         // ------------------------------------------------------------ epilogue: four warps per lane quadrant
+        if (p.sumx) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");     // (y, and the row sums)
         const int wl = warp - 4;
         const int q4 = wl & 3, quarter = wl >> 2;
