@@ -447,12 +447,17 @@ gemv_kernel(const __grid_constant__ Batch batch)
         mbar_init(bar_full(warp), 1);
         mbar_init(bar_empty(warp), NW);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (warp < total) issue(warp, warp);
+        if ((HALF || warp == 0) && warp < total) issue(warp, warp);
     }
     if (HALF && P.v != 4 * NCLS)                         // the last class of a block has two weights: its other half stays zero
         for (int i = tid; i < MAX_SLICES * L.stage_x_pitch / 4; i += CT) reinterpret_cast<uint32_t *>(smem + L.stage_x)[i] = 0u;
     __syncthreads();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // Integer form: the other stages behind the table and the first one, which are waited for first, as copies are served in order (a
+    // chain of 128 dependent launches 784.8 -> 779.0 us, q, k and v behind a transform 9.5 -> 9.4).  The fp16 form, which waits for
+    // its activations longer, sends all before (6001 x 4096, v = 8, five rows 8.1 us, 8.3 that way).
+    if (!HALF && warp > 0 && warp < NST && warp < total && lane == 0) issue(warp, warp);
+    __syncwarp();
 
     const int g = lane >> 2, t = lane & 3;
     // MMA row g (and g + 8) carries tile row sg (and sg + 8): neighbouring g differ in bit 2 of the row, so the lanes of a
