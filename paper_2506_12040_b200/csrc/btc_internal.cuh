@@ -87,6 +87,20 @@ __device__ __forceinline__ void store_from_float(void *p, int dt, size_t i, floa
     else if (dt == BTC_F16) reinterpret_cast<__half *>(p)[i] = __float2half_rn(f);
     else reinterpret_cast<__nv_bfloat16 *>(p)[i] = __float2bfloat16_rn(f);
 }
+// Activations in a kernel that starts before the one in front of it has ended: that one may be writing them while this one runs, so
+// they are not read-only for its lifetime as ld.global.nc (__ldg, const __restrict__) demands, and a line of them that an
+// SM's L1 still holds from a pass before would not have to be given up.  Plain loads, which griddepcontrol.wait orders; volatile, so that none
+// moves in front of it.
+__device__ __forceinline__ uint4 ld_x128(const void *p) {
+    uint4 q;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w) : "l"(p));
+    return q;
+}
+__device__ __forceinline__ uint2 ld_x64(const void *p) {
+    uint2 q;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(q.x), "=r"(q.y) : "l"(p));
+    return q;
+}
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

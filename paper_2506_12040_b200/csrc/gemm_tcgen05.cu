@@ -142,7 +142,7 @@ rowsum_kernel(const void *x, int x_dt, int K, float *out)
     const uint4 *row = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(x) + (size_t)m * K);   // (K is a multiple of 8)
 #pragma unroll 4
     for (int i = threadIdx.x; i < K / 8; i += 256) {
-        const uint4 q = __ldg(row + i);
+        const uint4 q = ld_x128(row + i);
         const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {

@@ -298,13 +298,15 @@ __device__ __forceinline__ void load8(const unsigned char *xrow, int dt, int k, 
     if (dt == BTC_F32) {
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
         if (in) {
-            const float4 *src = reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(xrow) + k);
-            a = __ldg(src); b = __ldg(src + 1);
+            const float *src = reinterpret_cast<const float *>(xrow) + k;
+            const uint4 qa = ld_x128(src), qb = ld_x128(src + 4);
+            a = make_float4(__uint_as_float(qa.x), __uint_as_float(qa.y), __uint_as_float(qa.z), __uint_as_float(qa.w));
+            b = make_float4(__uint_as_float(qb.x), __uint_as_float(qb.y), __uint_as_float(qb.z), __uint_as_float(qb.w));
         }
         f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
     } else {
         uint4 q = make_uint4(0u, 0u, 0u, 0u);
-        if (in) q = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(xrow) + k));
+        if (in) q = ld_x128(reinterpret_cast<const uint16_t *>(xrow) + k);
         cvt8(q, dt, f);
     }
 }
@@ -573,7 +575,7 @@ gemv_kernel(const __grid_constant__ Batch batch)
 #pragma unroll
                             for (int u = 0; u < NPR; ++u) {
                                 raw[i][u] = make_uint4(0u, 0u, 0u, 0u);
-                                if (m < M && 8 * (lane + 32 * u) < kin) raw[i][u] = __ldg(reinterpret_cast<const uint4 *>(src + u * 512));
+                                if (m < M && 8 * (lane + 32 * u) < kin) raw[i][u] = ld_x128(src + u * 512);
                             }
                         }
                     }
@@ -688,7 +690,7 @@ gemv_kernel(const __grid_constant__ Batch batch)
                             const int k = 8 * (lane + 32 * u);
                             cur[u] = make_uint4(0u, 0u, 0u, 0u);
                             if (!x32 && k < min(kleft, 8 * NGR))
-                                cur[u] = __ldg(reinterpret_cast<const uint4 *>(x + ((size_t)m * P.xs + (size_t)jb0 * (4 * NCLS) + k) * 2));
+                                cur[u] = ld_x128(x + ((size_t)m * P.xs + (size_t)jb0 * (4 * NCLS) + k) * 2);
                         }
                     };
                     load_row(0);

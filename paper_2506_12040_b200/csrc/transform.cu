@@ -19,7 +19,7 @@ constexpr int TR_THREADS = 256;
 constexpr int TR_DT = 8;            // output columns d per CTA
 
 __global__ void __launch_bounds__(TR_THREADS)
-transform_kernel(const void *__restrict__ x, int x_dt, const uint32_t *__restrict__ sigma_bits,
+transform_kernel(const void *x, int x_dt, const uint32_t *__restrict__ sigma_bits,
                  const float *__restrict__ P1, const float *__restrict__ P2, int k1, int k2, void *__restrict__ xt, int out_dt,
                  int M, int rows_per_cta)
 {
@@ -51,7 +51,7 @@ transform_kernel(const void *__restrict__ x, int x_dt, const uint32_t *__restric
             // 16-bit activations, eight per 16-byte load (rows are 16-byte aligned when 8 divides K)
             const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(x) + row);
             for (int i = threadIdx.x; i < K / 8; i += TR_THREADS) {
-                const uint4 q = __ldg(src + i);
+                const uint4 q = ld_x128(src + i);
                 const uint32_t sg = __ldg(sigma_bits + (i >> 2)) >> ((i & 3) * 8);
                 const uint32_t w[4] = {q.x, q.y, q.z, q.w};
                 const int rr = 4 * ((8 * i) / k2);     // the eight elements share a row of X (8 divides k2 here)
@@ -160,7 +160,7 @@ __device__ __forceinline__ void ts_fma(float (&acc)[TS_D], float f, const float 
 // AP: passes of 64 rows a, and c; K2: k2.
 template <int AP, int K2>
 __global__ void __launch_bounds__(TR_THREADS, AP == 1 && K2 == 64 ? 8 : 4)
-transform_few_kernel(const uint16_t *__restrict__ x, int f16, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
+transform_few_kernel(const uint16_t *x, int f16, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
                      const float *__restrict__ P2, int k1, void *__restrict__ xt, int out_dt)
 {
     constexpr int PIECES = K2 / 32;                      // of eight activations, of a lane
@@ -196,7 +196,7 @@ transform_few_kernel(const uint16_t *__restrict__ x, int f16, const uint32_t *__
         uint4 w[PIECES];
 #pragma unroll
         for (int j = 0; j < PIECES; ++j)
-            w[j] = a < k1 ? __ldg(reinterpret_cast<const uint4 *>(x + row + (size_t)a * K2) + q + 4 * j) : make_uint4(0u, 0u, 0u, 0u);
+            w[j] = a < k1 ? ld_x128(x + row + (size_t)a * K2 + 8 * (q + 4 * j)) : make_uint4(0u, 0u, 0u, 0u);
         float acc[TS_D] = {};
 #pragma unroll
         for (int j = 0; j < PIECES; ++j) {
@@ -310,7 +310,7 @@ struct TmPlan { int ds, cg, rw, p2_frags, mask_off; };       // slices, shares o
 // parts of a slice; two use every activation and every fragment of P1 twice.
 template <int NA, int TERMS, bool F16, int K2, int DW>
 __global__ void __launch_bounds__(TM_WARPS * 32, 1)
-transform_mma_kernel(const uint16_t *__restrict__ x, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
+transform_mma_kernel(const uint16_t *x, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
                      const float *__restrict__ P2, int k1, int k2_arg, void *__restrict__ xt, int out_dt, int M, TmPlan plan)
 {
     constexpr int LO = NA == 2 ? 0 : NA <= 8 ? NA - 2 : NA - 4, U = 8;
@@ -382,7 +382,7 @@ transform_mma_kernel(const uint16_t *__restrict__ x, const uint32_t *__restrict_
         auto load = [&](int k, uint2 (&dst)[NA]) {
 #pragma unroll
             for (int at = 0; at < NA; ++at)
-                dst[at] = at < LO || 8 * at + g < k1 ? __ldg(reinterpret_cast<const uint2 *>(xr + (size_t)(8 * at) * k2 + 16 * k)) : make_uint2(0u, 0u);
+                dst[at] = at < LO || 8 * at + g < k1 ? ld_x64(xr + (size_t)(8 * at) * k2 + 16 * k) : make_uint2(0u, 0u);
         };
 #pragma unroll
         for (int u = 0; u < PF; ++u)
