@@ -56,8 +56,8 @@ constexpr int KM_PART = 8192;                // most patterns per part of the ra
 // 109.2 in one copy; 1024 centroids: 105.4, 99.1, 99.1 and 98.6 (copies have to be cleared and summed).
 constexpr int KM_CROWD = 64;
 constexpr int KM_COPIES = 32;                // at most: a warp sums them up, one per lane
-static_assert((1 << KM_VMAX) / KM_PART <= KM_MAX_CTAS && (3 * KM_BINS + 1 + KM_PART) * 4 <= KM_SMEM && KM_PART < 65536,
-              "parts fit the columns, their frequencies shared memory, their counts 16 bits");
+static_assert((1 << KM_VMAX) / KM_PART <= KM_MAX_CTAS && (3 * KM_BINS + 1 + 2 * KM_PART) * 4 <= KM_SMEM && KM_PART < 65536,
+              "parts fit the columns, their frequencies and places shared memory, their counts 16 bits");
 
 __device__ int g_km_status = 0;
 
@@ -182,7 +182,7 @@ km_kernel(const KmArgs a)
     extern __shared__ __align__(16) unsigned char km_smem[];
     __shared__ int s_ok;
     __shared__ uint32_t s_warp[32];
-    __shared__ int s_listed;
+    __shared__ int s_listed, s_overs;
     uint32_t *sm = reinterpret_cast<uint32_t *>(km_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x, b = blockIdx.x, v = a.v, P = 1 << v, Kc = a.Kc;
@@ -269,12 +269,13 @@ km_kernel(const KmArgs a)
     //      one's patterns in the parts before (a 16-byte load per lane, four in flight), and the part's own patterns then draw their
     //      places from that start, 32 at a time in word order, those of a frequency found by a match over the warp.
     uint32_t *s_next = s_cnt + KM_PART, *s_list = s_next + KM_BINS;     // next free rank of a frequency; the frequencies listed
+    uint32_t *s_over = s_list + KM_BINS;                                // patterns of the part past the last bin
     constexpr uint32_t UNSEEN = 0xffffffffu, LISTED = 0xfffffffeu;
     for (int q = b; q < a.parts; q += G) {
         const int p0 = min(P, per * q), np = min(P, p0 + per) - p0;
         __syncthreads();
         for (int i = tid; i < KM_BINS; i += KM_THREADS) s_next[i] = UNSEEN;
-        if (tid == 0) s_listed = 0;
+        if (tid == 0) s_listed = s_overs = 0;
         if (a.parts > G)                                     // (several parts: their frequencies again)
             for (int i = tid; i < np; i += KM_THREADS) s_cnt[i] = __ldcg(a.cnt + p0 + i);
         __syncthreads();
@@ -282,6 +283,7 @@ km_kernel(const KmArgs a)
         for (int i = tid; i < np; i += KM_THREADS) {
             const uint32_t c = s_cnt[i];
             if (ranked(c) && atomicExch(s_next + c, LISTED) == UNSEEN) s_list[atomicAdd(&s_listed, 1)] = c;
+            if (c >= KM_BINS - 1) s_over[atomicAdd(&s_overs, 1)] = (uint32_t)i;
         }
         __syncthreads();
         for (int i0 = warp; i0 < s_listed; i0 += 4 * (KM_THREADS / 32)) {
@@ -318,17 +320,18 @@ km_kernel(const KmArgs a)
             }
             r = __shfl_sync(0xffffffffu, r, first) + __popc(same & ((1u << lane) - 1u));
             if (mine && r < (uint32_t)Kc) { a.C[r] = p; a.seed[p] = r; }
-            // past the last bin: pairwise, a warp per pattern
-            for (uint32_t over = __ballot_sync(0xffffffffu, c >= KM_BINS - 1); over; over &= over - 1u) {
-                const uint32_t co = __shfl_sync(0xffffffffu, c, __ffs(over) - 1), po = __shfl_sync(0xffffffffu, p, __ffs(over) - 1);
-                uint32_t before = 0;
-                for (int j = lane; j < (int)s_bins[KM_BINS - 1]; j += 32) {
-                    const uint2 o = __ldcg(a.over + j);
-                    before += (o.x > co || (o.x == co && o.y < po)) ? 1u : 0u;
-                }
-                before = __reduce_add_sync(0xffffffffu, before);
-                if (lane == 0 && before < (uint32_t)Kc) { a.C[before] = po; a.seed[po] = before; }
+        }
+        // past the last bin: pairwise, a warp per pattern (4 194 304 vectors, where most patterns are past it: v = 10, 256 centroids
+        // 45 us a call, v = 12, 777 47; 61 and 60 where a warp took those among its 32 neighbours one after another)
+        for (int i = warp; i < s_overs; i += KM_THREADS / 32) {
+            const uint32_t c = s_cnt[s_over[i]], p = (uint32_t)p0 + s_over[i];
+            uint32_t before = 0;
+            for (int j = lane; j < (int)s_bins[KM_BINS - 1]; j += 32) {
+                const uint2 o = __ldcg(a.over + j);
+                before += (o.x > c || (o.x == c && o.y < p)) ? 1u : 0u;
             }
+            before = __reduce_add_sync(0xffffffffu, before);
+            if (lane == 0 && before < (uint32_t)Kc) { a.C[before] = p; a.seed[p] = before; }
         }
     }
     if (!km_sync(a.st, target, &s_ok)) return;

@@ -169,6 +169,22 @@ def test_kmeans_ends_where_no_centroid_moves(n, v, Kc, kind, max_iter):
     assert btc.device_status() == 0
 
 
+@pytest.mark.parametrize("v,Kc", [(3, 5), (5, 32), (8, 60), (9, 400)])
+def test_kmeans_frequencies_around_the_last_bin(v, Kc):
+    """All patterns, at frequencies on both sides of the last bin (2047 and more are ranked pairwise), many of them equal: parts of
+    one pattern and of several; where a rank is wrong a centroid is another, or starts in another's place."""
+    cnt = np.random.default_rng(v).integers(2041, 2053, 1 << v)
+    words = np.random.default_rng(Kc).permutation(np.repeat(np.arange(1 << v, dtype=np.uint32), cnt))
+    C_ref, n_unique = km.initial_codebook(km.unpack_words(words, v), Kc)
+    C, z, info = (t.cpu().numpy() for t in btc.codebook_kmeans(torch.from_numpy(words.view(np.int32)).cuda(), v, Kc, 1))
+    z_pat = km.e_step(km.unpack_words(np.arange(1 << v), v), C_ref)
+    assert info.tolist() == [1, Kc, n_unique, 0] and np.array_equal(z.view(np.uint16), z_pat[words])
+    U = km.unpack_words(np.arange(1 << v), v).astype(np.int64) * cnt[:, None]
+    sums = np.stack([U[z_pat == k].sum(axis=0) for k in range(Kc)])
+    assert np.array_equal(C.view(np.uint32), km.pack_words(np.where(sums >= 0, 1, -1)))
+    assert btc.device_status() == 0
+
+
 def test_kmeans_feeds_the_layer():
     """The construction's outputs are the layer's inputs: centroids -> btc_codebook_pack, z -> idx; decoding them
     gives the nearest-centroid approximation of the sign matrix, whose Hamming error equals the oracle's objective."""

@@ -124,14 +124,15 @@ def _kmeans(L, n, v, Kc=256):
 @pytest.mark.parametrize("n", [1, 3000, 1 << 20, (1 << 31) - 1])
 @pytest.mark.parametrize("sms", [1, 2, 18, 35, 148, 300])
 def test_codebook_construction_fits_its_tables_on_any_number_of_sms(fake, sms, n, v):
-    """A part of the 2^v patterns: its frequencies beside 2049 bins in shared memory, its counts in 16 bits, a column of the
-    256 per bin; every pattern in one part, every CTA one part or more."""
+    """A part of the 2^v patterns: its frequencies, and as many places for those past the last bin, beside 2049 bins and twice 2048 words for
+    the ranks in shared memory, its counts in 16 bits, a column of the 256 per bin; every pattern in one part, every CTA one
+    part or more."""
     fake.fake_reset(sms, 0, 0, None)
     grid, a = _kmeans(fake, n, v)
     assert (a.n, a.v, a.fields) == (n, v, 3 if n < 1 << 21 else 2)
     per = -(-(1 << v) // a.parts)
     assert 1 <= grid <= min(sms, 256) and grid <= a.parts <= 256
-    assert (2049 + per) * 4 <= fake.fake_smem(0) and per < 1 << 16
+    assert (2049 + 2 * 2048 + 2 * per) * 4 <= fake.fake_smem(0) and per < 1 << 16
 
 
 @pytest.mark.parametrize("of_stream,most,grid", [(0, 0, 148), (16, 0, 16), (200, 0, 148), (0, 20, None), (64, 1, 1)])
