@@ -138,11 +138,20 @@ transform_kernel(const void *x, int x_dt, const uint32_t *__restrict__ sigma_bit
 // every fourth a.  Lanes that share a sum hand over halves of their columns, so that four sums over four lanes take three shuffles
 // and leave one in each.
 // Bound: latency, of the chain behind the kernel before it: wait, x from L2, two products of K2 / 4 and k1 / 4 steps with one
-// barrier between them, store.  Shared memory (the k2 x 8 slab of P2 and Y, 4 KB at 64 x 64) and 32 registers a thread leave room for a
-// CTA beside the two of the integer decode kernel: it starts, and fetches the factors, while the layers before it run, and those behind
-// it start while it runs; P1 waits in L1.  One row of 64 x 64 and the three 4096 x 4096 layers behind it: 11.2 us with
-// transform_kernel (40 KB of shared memory, so neither; P1 and X through it), now 9.4.
+// barrier between them, store; P1 waits in L1.  A CTA asks for more than half of an SM's shared memory, so that no two share one: small
+// CTAs, up to eight on an SM, all went to the few SMs that a layer in front of them left first, worked there side by side, and kept
+// those SMs from the layer behind, which has CTAs for all of them.  That layer is let in when the wait is over: it has the transform's time
+// to fetch its first indices, needs no more, and takes no SM from transforms that wait.
+// us a call, transform and one or three 4096 x K layers behind it (v = 16), of transform_kernel, of small CTAs that let the layer in at
+// once, and of this one:
+//             one row: one layer    three layers          eight rows: one layer    three layers
+//   32 x 64    7.1 /  6.9 /  5.9     8.8 /  8.7 /  7.4     10.0 / 10.2 /  9.5     14.0 / 20.2 / 11.6
+//   64 x 64    8.3 /  7.9 /  7.6    11.1 /  9.4 /  9.1     20.5 / 17.2 / 13.1     22.8 / 25.4 / 15.2
+//   40 x 128  10.3 /  9.5 /  9.4    15.6 / 14.9 / 12.6     25.0 / 24.0 / 18.6     28.6 / 28.1 / 22.9
+//   86 x 128  16.9 / 15.9 / 15.1    21.6 / 26.0 / 20.3     29.2 / 33.0 / 29.2     39.9 / 50.6 / 35.4
+// (The small ones were the faster only beside the integer decode kernel at 64 x 64 and less, three layers of 11008: 13.0 and now 13.5.)
 constexpr int TS_D = 8;             // columns per CTA
+constexpr int TS_ALONE = 115 * 1024; // bytes of dynamic shared memory, unused: half of an SM's and more
 
 // acc[i] summed over the four lanes that differ in bits 0 and 1; lane q gets column q
 __device__ __forceinline__ float ts_quad(const float *acc, int q) {
@@ -157,7 +166,8 @@ __device__ __forceinline__ void ts_fma(float (&acc)[TS_D], float f, const float 
     acc[4] = fmaf(f, r.x, acc[4]); acc[5] = fmaf(f, r.y, acc[5]); acc[6] = fmaf(f, r.z, acc[6]); acc[7] = fmaf(f, r.w, acc[7]);
 }
 
-// AP: passes of 64 rows a, and c; K2: k2.
+// AP: passes of 64 rows a, and c; K2: k2.  (The second bound is there for the registers that it has the compiler spend, which keep more loads
+// in flight: 64 where it takes 44 to 51 by itself; 128 x 64, one row, alone 6.7 us, and 7.5)
 template <int AP, int K2>
 __global__ void __launch_bounds__(TR_THREADS, AP == 1 && K2 == 64 ? 8 : 4)
 transform_few_kernel(const uint16_t *x, int f16, const uint32_t *__restrict__ sigma_bits, const float *__restrict__ P1,
@@ -166,7 +176,6 @@ transform_few_kernel(const uint16_t *x, int f16, const uint32_t *__restrict__ si
     constexpr int PIECES = K2 / 32;                      // of eight activations, of a lane
     __shared__ __align__(16) float s_p2[K2 / 8][8 * TS_D + 4];           // (four lanes read pieces next to each other: on different banks)
     __shared__ __align__(16) float s_y[64 * AP][TS_D];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, q = tid & 3, d0 = blockIdx.x * TS_D;
     const size_t row = (size_t)blockIdx.y * k1 * K2;
     for (int i = tid; i < K2 * TS_D; i += TR_THREADS) {
@@ -190,6 +199,7 @@ transform_few_kernel(const uint16_t *x, int f16, const uint32_t *__restrict__ si
     // (the factors are parameters of the layer, complete before the call was enqueued; x is read, and x' written, once the kernel
     // before this one has completed)
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #pragma unroll 1
     for (int ap = 0; ap < AP; ++ap) {
         const int a = 64 * ap + (tid >> 2);
@@ -220,8 +230,9 @@ transform_few_kernel(const uint16_t *x, int f16, const uint32_t *__restrict__ si
     for (int cp = 0; cp < AP; ++cp) {
         const int c = 64 * cp + (tid >> 2);
         float acc[TS_D] = {};
+        int i0 = 0;
 #pragma unroll 1
-        for (int i0 = 0; i0 < 16 * AP; i0 += 8) {
+        do {
             float pv[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -230,7 +241,8 @@ transform_few_kernel(const uint16_t *x, int f16, const uint32_t *__restrict__ si
             }
 #pragma unroll
             for (int i = 0; i < 8; ++i) ts_fma(acc, pv[i], s_y[q + 4 * (i0 + i)]);
-        }
+            i0 += 8;
+        } while (4 * i0 < k1);
         const float r0 = ts_quad(acc, q), r1 = ts_quad(acc + 4, q);
         if (c < k1) {
             store_from_float(xt, out_dt, row + (size_t)c * K2 + d0 + q, r0);
@@ -242,17 +254,27 @@ transform_few_kernel(const uint16_t *x, int f16, const uint32_t *__restrict__ si
 template <int AP, int K2>
 static int launch_transform_few(const void *x, int x_dt, const btc_transform &T, void *xt, int out_dt, int M, cudaStream_t s)
 {
+    auto kern = transform_few_kernel<AP, K2>;
+    static std::atomic<uint64_t> done{0};                          // (the attribute, once per device)
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (dev >= 64 || !((done.load(std::memory_order_relaxed) >> dev) & 1u)) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_ALONE);
+        if (e != cudaSuccess) return cuda_fail(e);
+        if (dev < 64) done.fetch_or(uint64_t(1) << dev, std::memory_order_relaxed);
+    }
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(K2 / TS_D, (unsigned)M);
     cfg.blockDim = dim3(TR_THREADS);
+    cfg.dynamicSmemBytes = TS_ALONE;
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, transform_few_kernel<AP, K2>, static_cast<const uint16_t *>(x), x_dt == BTC_F16 ? 1 : 0, T.sigma_bits, T.P1,
-                                             T.P2, T.k1, xt, out_dt);
+    e = cudaLaunchKernelEx(&cfg, kern, static_cast<const uint16_t *>(x), x_dt == BTC_F16 ? 1 : 0, T.sigma_bits, T.P1, T.P2, T.k1, xt, out_dt);
     return e == cudaSuccess ? BTC_OK : cuda_fail(e);
 }
 
@@ -589,16 +611,17 @@ static int launch_transform_terms(const void *x, const btc_transform &T, void *x
 int launch_transform(const void *x, int x_dt, const btc_transform &T, void *xt, int out_dt, int M, int K, cudaStream_t s)
 {
     if ((long long)T.k1 * T.k2 != K) return BTC_ERR_SHAPE;
-    // (up to 8 rows the forms in fp32 have the shorter chain: 4.3 us at 64 x 64, one row, with the slower of them where this one took
-    // 4.9.  Below 64 rows three terms: the precision of the fp32 form; above, two carry more than 16-bit x.)
+    // (up to 8 rows the forms in fp32 have the shorter chain: with three layers of 4096 behind it, 64 x 64, one row 9.1 us where this one
+    // took 11.5, eight rows 15.2 and 18.3, 86 x 128 35.4 and 42.3.  Below 64 rows three terms: the precision of the fp32 form; above, two carry more than 16-bit x.)
     if (x_dt != BTC_F32 && M > 8 && T.k2 % 16 == 0 && T.k1 <= 128) {
         const bool f16 = x_dt == BTC_F16;
         const int rc = M >= 64 ? (f16 ? launch_transform_terms<2, true>(x, T, xt, out_dt, M, s) : launch_transform_terms<2, false>(x, T, xt, out_dt, M, s))
                                : (f16 ? launch_transform_terms<3, true>(x, T, xt, out_dt, M, s) : launch_transform_terms<3, false>(x, T, xt, out_dt, M, s));
         if (rc != BTC_ERR_UNSUPPORTED) return rc;
     }
-    // (k2 as compiled in; k1 up to two passes of 64 rows)
-    if (x_dt != BTC_F32 && M <= 8 && T.k1 <= 128 && (T.k2 == 64 || T.k2 == 128)) {
+    // (k2 as compiled in; k1 up to two passes of 64 rows.  Up to 16 rows of X most of a pass is empty and a CTA of transform_kernel is small
+    // too: 16 x 64, three rows, two layers of 4096 behind it 8.5 us, and 8.9 with this one; 32 x 64 9.4 and 9.0, 86 x 128 29.5 and 25.6.)
+    if (x_dt != BTC_F32 && M <= 8 && T.k1 > 16 && T.k1 <= 128 && (T.k2 == 64 || T.k2 == 128)) {
         if (T.k2 == 64) return T.k1 <= 64 ? launch_transform_few<1, 64>(x, x_dt, T, xt, out_dt, M, s) : launch_transform_few<2, 64>(x, x_dt, T, xt, out_dt, M, s);
         return T.k1 <= 64 ? launch_transform_few<1, 128>(x, x_dt, T, xt, out_dt, M, s) : launch_transform_few<2, 128>(x, x_dt, T, xt, out_dt, M, s);
     }

@@ -104,6 +104,20 @@ def test_launches_follow_the_sms_of_the_device(fake, sms):
     assert "gemm_ts_kernel" in name and grid == 8 * fake.fake_cluster(0) and (fake.fake_cluster(0) > 1) == (sms > 16)
 
 
+@pytest.mark.parametrize("M,k1,k2,kernel", [(1, 64, 64, "few"), (8, 17, 64, "few"), (3, 128, 128, "few"), (8, 65, 128, "few"), (8, 16, 64, ""), (1, 129, 64, ""),
+                                            (8, 64, 80, ""), (9, 64, 64, "mma")])
+def test_transform_of_a_few_rows_shares_no_sm(fake, M, k1, k2, kernel):
+    """No two CTAs fit an SM (228 KB of shared memory, 1 KB of it per CTA taken by the system): as many as there are together would
+    go to the SMs that a layer in front leaves first, and keep the layer behind from them."""
+    T = BtcTransform(0x1000, 0x2000, 0x3000, k1, k2)
+    fake.fake_reset(148, 0, 0, None)
+    assert fake.btc_activation_transform(ctypes.c_void_p(0x4000), 0, ctypes.byref(T), ctypes.c_void_p(0x50000), 0, M, k1 * k2, None) == 0
+    (name, grid), = _launches(fake)
+    assert ("transform_few_kernel" in name) == (kernel == "few") and ("transform_mma_kernel" in name) == (kernel == "mma")
+    if kernel == "few":
+        assert grid == M * k2 // 8 and 2 * (fake.fake_smem(0) + 1024) > 228 * 1024
+
+
 class KmArgs(ctypes.Structure):
     _fields_ = ([("vecs", ctypes.c_void_p), ("n", ctypes.c_size_t)] + [(k, ctypes.c_int) for k in ("v", "Kc", "max_iter")]
                 + [(f"p{i}", ctypes.c_void_p) for i in range(12)] + [(k, ctypes.c_int) for k in ("words", "fields", "parts")])
