@@ -88,6 +88,7 @@ static int run_linear(Path path, const void *x, int x_dt, const uint16_t *idx, c
         rc = launch_transform(x, x_dt, *T, ws, xt_f32 ? BTC_F32 : x_dt, M, K, s);
         if (rc != BTC_OK) return rc;
         a.x = ws;
+        a.transformed = true;
         if (xt_f32) a.x_dt = BTC_F32;
         a.workspace = static_cast<char *>(ws) + xt_bytes;
         a.workspace_bytes = ws_bytes - xt_bytes;

@@ -28,6 +28,7 @@ struct LinearArgs {
     int x_stride = 0;
     int idx_stride = 0;
     int accumulate = 0;
+    bool transformed = false;   // x comes from the activation transform, run in front of this layer
 };
 
 // Records a CUDA error for btc_last_cuda_error() and maps it to BTC_ERR_CUDA.

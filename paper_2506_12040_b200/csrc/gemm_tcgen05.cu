@@ -333,10 +333,13 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams
 //
 // Launched with programmatic stream serialisation: barriers, tensor memory, table and first indices are ready before
 // the predecessor has finished; x is read after it (or right away where the predecessor is the row-sum kernel, which
-// itself waited for it; then the epilogue waits).  Its own successors may start early (a transform
-// behind it: 13.0 -> 10.5 us for 24 rows, K = 1024), with a mean term only when its k steps are done: from the start, the next
-// call's row sums, small CTAs, would pile up on the SMs that a round of tiles leaves idle (9.0 -> 9.8 us for 16 rows of 4096 x 4096);
-// from there on they are in place when the epilogue ends (4096 x 11008, 77 rows: 15.8 -> 15.1 us; 16 rows 8.9 where they came at 9.0).
+// itself waited for it; then the epilogue waits).  Its own successors may start early (a transform behind it: 13.0 -> 10.5 us for 24 rows,
+// K = 1024).  With a mean term only when the accumulator has been read (launch_ts), and only where the next call is likely to begin with no
+// more CTAs than there are SMs, a transform or row sums of few rows.  Small CTAs that come while tiles of x still run go to the
+// SMs that are idle or end first, eight to one, and the next contraction waits for those: 4096 x 4096 (v = 8) at 256 and 512 rows 16.1 and
+// 19.9 us without, 17.5 and 22.8 when they came from the epilogue on, as with any number of rows before; below 33 rows there is nothing to gain
+// (4096 x 11008, 16 rows 13.2 and 13.8).  4096 x 11008 at 33 and 77 rows 14.8 and 15.8 without, 14.3 and 15.3 from the epilogue on, 14.0 and 15.1
+// now; 40 x 64 transform and the layer behind it, 33 and 129 rows 15.4 and 18.3, 13.2 and 15.8, 13.0 and 15.3.
 constexpr int G2_DWARPS = 16;                    // decode warps (four groups of four)
 constexpr int G2_THREADS = 128 + G2_DWARPS * 32;
 constexpr uint32_t G2_IDX_BYTES = 128 * 128;     // one index tile
@@ -353,6 +356,7 @@ struct Gemm2Params {
 
 struct SplitArgs {
     int split_tiles;         // k tiles (whole index tiles) per CTA along grid.z
+    int early;               // with a mean term: the next kernel may start when the accumulator has been read
 };
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
@@ -612,7 +616,6 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             if (lane == 0) mbar_arrive(bar_full(sa));
         }
         // ------------------------------------------------------------ epilogue: four warps per lane quadrant
-        if (p.sumx) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");     // (y, and the row sums)
         const int wl = warp - 4;
         const int q4 = wl & 3, quarter = wl >> 2;
@@ -666,6 +669,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             }
         }
     }
+    if (sp.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if constexpr (SPLIT) {
         // (columns advance by whole multiples of 32 threads: a thread's four features stay the same, and what belongs to them is
         // fetched while the cluster meets)
@@ -824,7 +828,7 @@ static int launch_ts(const CUtensorMap &tm, const CUtensorMap &ti, const Gemm2Pa
     at[2].val.clusterDim.x = 1; at[2].val.clusterDim.y = 1; at[2].val.clusterDim.z = (unsigned)g.splits;
     cfg.attrs = at;
     cfg.numAttrs = SPLIT ? 3 : 2;
-    const SplitArgs sp = {g.split_tiles};
+    const SplitArgs sp = {g.split_tiles, p.a.mu && (p.a.transformed || (p.a.M > 32 && p.a.M <= device_sms()))};
     e = cudaLaunchKernelEx(&cfg, kern, tm, ti, p, sp);
     return e == cudaSuccess ? BTC_OK : cuda_fail(e);
 }
