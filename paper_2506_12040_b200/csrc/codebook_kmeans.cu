@@ -26,11 +26,11 @@
 //              few move cast few votes and the one that finds nothing changed none; then one thread per centroid.  Where many
 //              patterns share few centroids up to 32 copies of the votes are kept, and a warp per centroid adds them up
 //   assign     z through the label table in shared memory (v <= 16)
-// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 48.1 us a call (50.4 us where a warp added up
+// Bound: latency.  1 048 576 vectors, v = 16, 8192 centroids, two rounds: 46.0 us a call (50.4 us where a warp added up
 // the parts before, and counted the equals before, for every pattern that it ranked; 58.7 us where in addition the round behind an
 // M-step that changed no centroid was run to find that nothing changes: two barriers and both halves of its E-step).
-// Clock stamps of the first CTA in thousands: clearing 2.4, histogram 12.2, patterns per frequency 2.4, E-step 5.0 + 10.1 with all votes cast, M-step 5.5,
-// assignment 7.0; the other five of the six grid barriers, with the wait for the slowest CTA, 3.5 to 5.5 each.
+// Clock stamps of the first CTA in thousands: clearing 2.3, histogram 12.9, patterns per frequency 2.8, suffix sums 1.6, ranking 5.6, E-step
+// 2.8 + 9.6 with all votes cast, M-step 4.7, assignment 6.7; the six grid barriers, with the wait for the slowest CTA, 3.6 to 6.6 each.
 // A move is two atomics per word where casting anew is one, so a round in which more than half of the patterns move costs more
 // than that; on few centroids, where the votes are most of the call, the copies more than make up for it.  Two rounds, in the second
 // of which three quarters of 65 536 patterns move: 16 centroids 331 us with all votes cast anew, 391 as differences in one copy,

@@ -751,10 +751,12 @@ static int launch_cfg(const CUtensorMap &tm, const GemmParams &p, cudaStream_t s
 // Time in clocks, fitted to measurements of every width at K = 2000 and 4096, made when the epilogue took longer: a CTA per SM in
 // rounds, the last one as long as the others, each a fixed part (launch, tensor memory, first tiles, epilogue) and its k steps.  A step of tiles up to 128 wide
 // costs what their MMAs and x tiles cost or the decode of its weights; wider ones have one issuing thread and cost
-// about the same whatever their width: 11008 x 4096 at 300 rows takes 53 us as two tiles of 160 and 36 as three of 112.  Clock
-// stamps, v = 16: a step 553 at 256 wide (its MMAs alone: 512), 351 at 128, 325 at 80; set-up to first MMA 2.7 k, 3.5 k and
-// 3.5 k, last MMA to end, the epilogue, 4.6 k, 2.2 k (12.1 k and 7.0 k when the fixed parts were fitted) and, sum over the cluster
-// included, 5.7 k.  The fixed parts are kept on measurement: with 12 000 and 7 000 for launches without a split the choice changes for
+// about the same whatever their width: 11008 x 4096 at 300 rows took 53 us as two tiles of 160 and 36 as three of 112.  Clock
+// stamps of the kernel as it is, v = 16, and as it was when this was fitted: a step 553 at 256 wide (its MMAs alone: 512), 232 at 128 and 219
+// at 80 (351 and 325, index tiles in turn with x); set-up to first MMA 2.7 k, 3.2 k and 3.2 k (2.7 k, 3.5 k, 3.5 k), last MMA to end, the epilogue,
+// 4.6 k, 2.2 k (12.1 k, 7.0 k) and, sum over the cluster included, 5.7 k.  So narrow steps are priced above what they now cost, and a wide
+// tile may be taken where three rounds of narrow ones would be faster: the steps have not been fitted again.  The fixed parts alone
+// have, and are kept on measurement (of the slower steps): with 12 000 and 7 000 for launches without a split the choice changes for
 // one shape in nine and mostly for the worse (us, as is / 4 k less; v = 16, 8192 codewords): 512 x 11008 x 4096 (M x N x K) 47.2 / 46.6,
 // 645 x 7822 x 1024 18.8 / 18.8, 714 x 7739 x 1024 18.1 / 19.0, 1776 x 3270 x 7424 76.6 / 77.1, 539 x 10900 x 5376 56.4 / 58.7, 12 x 6580 x 4352
 // 12.8 / 15.0, 150 x 2050 x 2432 8.3 / 10.3, 230 x 3970 x 4992 16.0 / 18.3, 700 x 8000 x 1200 (v = 10) 25.5 / 32.9.  Codewords
