@@ -88,7 +88,6 @@ static int run_linear(Path path, const void *x, int x_dt, const uint16_t *idx, c
         rc = launch_transform(x, x_dt, *T, ws, xt_f32 ? BTC_F32 : x_dt, M, K, s);
         if (rc != BTC_OK) return rc;
         a.x = ws;
-        a.transformed = true;
         if (xt_f32) a.x_dt = BTC_F32;
         a.workspace = static_cast<char *>(ws) + xt_bytes;
         a.workspace_bytes = ws_bytes - xt_bytes;
@@ -100,7 +99,7 @@ static int run_linear(Path path, const void *x, int x_dt, const uint16_t *idx, c
         rc = launch_gemv(&a, 1, s);
         if (rc == BTC_ERR_UNSUPPORTED) rc = launch_gemv_decode(a, s);
     }
-    else rc = launch_gemm_tcgen05(a, s);
+    else rc = launch_gemm_tcgen05(a, T != nullptr, s);
     if (rc == BTC_ERR_UNSUPPORTED) {
         if (path == PATH_GEMM && M <= 8) rc = launch_gemv_decode(a, s);
         if (rc == BTC_ERR_UNSUPPORTED) rc = launch_linear_generic(a, s);

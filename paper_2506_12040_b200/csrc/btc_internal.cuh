@@ -28,7 +28,6 @@ struct LinearArgs {
     int x_stride = 0;
     int idx_stride = 0;
     int accumulate = 0;
-    bool transformed = false;   // x comes from the activation transform, run in front of this layer
 };
 
 // Records a CUDA error for btc_last_cuda_error() and maps it to BTC_ERR_CUDA.
@@ -47,8 +46,8 @@ int launch_linear_generic(const LinearArgs &a, cudaStream_t s);
 // Returns BTC_ERR_UNSUPPORTED when the shape is outside what it covers, in which case the caller falls back to the generic kernel.
 int launch_gemv_decode(const LinearArgs &a, cudaStream_t s);
 
-// gemm_tcgen05.cu: tensor-core path.  Same UNSUPPORTED convention.
-int launch_gemm_tcgen05(const LinearArgs &a, cudaStream_t s);
+// gemm_tcgen05.cu: tensor-core path; `transformed`: x comes from the activation transform, run in front of it.  Same UNSUPPORTED convention.
+int launch_gemm_tcgen05(const LinearArgs &a, bool transformed, cudaStream_t s);
 size_t gemm_tcgen05_workspace_bytes(int M);   // row sums of x (a split of K sums in distributed shared memory)
 
 // gemv.cu: the decode path; runs up to IM_MAXP independent layers (M <= 8 each), one launch for those that share a kernel.

@@ -334,12 +334,13 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams
 // Launched with programmatic stream serialisation: barriers, tensor memory, table and first indices are ready before
 // the predecessor has finished; x is read after it (or right away where the predecessor is the row-sum kernel, which
 // itself waited for it; then the epilogue waits).  Its own successors may start early (a transform behind it: 13.0 -> 10.5 us for 24 rows,
-// K = 1024).  With a mean term only when the accumulator has been read (launch_ts), and only where the next call is likely to begin with no
-// more CTAs than there are SMs, a transform or row sums of few rows.  Small CTAs that come while tiles of x still run go to the
-// SMs that are idle or end first, eight to one, and the next contraction waits for those: 4096 x 4096 (v = 8) at 256 and 512 rows 16.1 and
-// 19.9 us without, 17.5 and 22.8 when they came from the epilogue on, as with any number of rows before; below 33 rows there is nothing to gain
-// (4096 x 11008, 16 rows 13.2 and 13.8).  4096 x 11008 at 33 and 77 rows 14.8 and 15.8 without, 14.3 and 15.3 from the epilogue on, 14.0 and 15.1
-// now; 40 x 64 transform and the layer behind it, 33 and 129 rows 15.4 and 18.3, 13.2 and 15.8, 13.0 and 15.3.
+// K = 1024).  With a mean term only when its k steps are done, and only where the next call is likely to begin with no
+// more CTAs than there are SMs: a transform, or row sums of few rows.  Small CTAs that come while other tiles run go to the SMs
+// that are idle or end first, eight to one, and the next contraction waits for those: 4096 x 4096 (v = 8) at 256 and 512 rows 16.1 and
+// 19.9 us without, 17.5 and 22.7 when they came with any number of rows; below 33 rows there is nothing to gain (4096 x 11008, 16 rows 13.2 and
+// 13.8).  With it 4096 x 11008 at 33 and 77 rows 14.8 -> 14.3 and 15.8 -> 15.3, a 40 x 64 transform and the layer behind it at 33 and 129
+// rows 15.4 -> 13.2 and 18.3 -> 15.8.  (When the accumulator has been read, another 0.2 us with a mean term, but small calls
+// without one took 0.1 us longer: 1000 x 1024, 77 rows 5.05 and 5.19.)
 constexpr int G2_DWARPS = 16;                    // decode warps (four groups of four)
 constexpr int G2_THREADS = 128 + G2_DWARPS * 32;
 constexpr uint32_t G2_IDX_BYTES = 128 * 128;     // one index tile
@@ -352,11 +353,11 @@ struct Gemm2Params {
     int k_tiles;
     int tab_bytes;           // > 0: table staged in shared memory
     int bn;                  // rows of x per tile
+    int early;               // with a mean term: the next kernel may start during the epilogue
 };
 
 struct SplitArgs {
     int split_tiles;         // k tiles (whole index tiles) per CTA along grid.z
-    int early;               // with a mean term: the next kernel may start when the accumulator has been read
 };
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
@@ -616,6 +617,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             if (lane == 0) mbar_arrive(bar_full(sa));
         }
         // ------------------------------------------------------------ epilogue: four warps per lane quadrant
+        if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");     // (y, and the row sums)
         const int wl = warp - 4;
         const int q4 = wl & 3, quarter = wl >> 2;
@@ -669,7 +671,6 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             }
         }
     }
-    if (sp.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if constexpr (SPLIT) {
         // (columns advance by whole multiples of 32 threads: a thread's four features stay the same, and what belongs to them is
         // fetched while the cluster meets)
@@ -830,7 +831,7 @@ static int launch_ts(const CUtensorMap &tm, const CUtensorMap &ti, const Gemm2Pa
     at[2].val.clusterDim.x = 1; at[2].val.clusterDim.y = 1; at[2].val.clusterDim.z = (unsigned)g.splits;
     cfg.attrs = at;
     cfg.numAttrs = SPLIT ? 3 : 2;
-    const SplitArgs sp = {g.split_tiles, p.a.mu && (p.a.transformed || (p.a.M > 32 && p.a.M <= device_sms()))};
+    const SplitArgs sp = {g.split_tiles};
     e = cudaLaunchKernelEx(&cfg, kern, tm, ti, p, sp);
     return e == cudaSuccess ? BTC_OK : cuda_fail(e);
 }
@@ -847,7 +848,7 @@ size_t gemm_tcgen05_workspace_bytes(int M)
     return M > 8 ? (size_t)M * sizeof(float) : 0;   // row sums of x for the mean term
 }
 
-int launch_gemm_tcgen05(const LinearArgs &a, cudaStream_t s)
+int launch_gemm_tcgen05(const LinearArgs &a, bool transformed, cudaStream_t s)
 {
     if (a.K % 8) return BTC_ERR_UNSUPPORTED;                   // TMA row pitch must be a multiple of 16 bytes
     encode_tiled_fn enc = get_encode();
@@ -896,6 +897,7 @@ int launch_gemm_tcgen05(const LinearArgs &a, cudaStream_t s)
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
             Gemm2Params q;
             q.a = a; q.sumx = p.sumx; q.k_tiles = p.k_tiles; q.bn = g.bn;
+            q.early = a.mu && (transformed || (a.M > 32 && a.M <= device_sms()));
             const int Kc4 = (a.Kc + 3) / 4 * 4;
             q.tab = a.Cp + Kc4;
             // shared memory holds only x tiles (four stages), index tiles and the table
